@@ -42,120 +42,143 @@ __global__ void k_gamma5_reflect(const C* __restrict__ in, C* __restrict__ out, 
     }
 }
 
-// conj(a) . M . b for a 2x2 spin matrix M = (1 + sgn gamma_mu) (2-d basis)
-__device__ __forceinline__ double2 bilinear(double2 a0, double2 a1, double2 b0, double2 b1, int mu, int sgn) {
-    // M b
-    double2 m0, m1;
-    if (mu == 0) {           // gamma_1 = sigma_1
-        m0 = make_double2(b0.x + sgn * b1.x, b0.y + sgn * b1.y);
-        m1 = make_double2(b1.x + sgn * b0.x, b1.y + sgn * b0.y);
-    } else {                 // gamma_2 = sigma_2 = [[0,-i],[i,0]]
-        m0 = make_double2(b0.x + sgn * b1.y, b0.y - sgn * b1.x);   // b0 - i sgn b1
-        m1 = make_double2(b1.x - sgn * b0.y, b1.y + sgn * b0.x);   // b1 + i sgn b0
-    }
-    return make_double2(a0.x * m0.x + a0.y * m0.y + a1.x * m1.x + a1.y * m1.y,
-                        a0.x * m0.y - a0.y * m0.x + a1.x * m1.y - a1.y * m1.x);
+// ---------------------------------------------------------------------------
+// Link derivatives.  Both kernels run at the FP64 rate of the chip (two FMAs per
+// clock and SM), far above their memory time, so they are written for the fewest
+// FP64 instructions: 1 -+ gamma_mu has half the rank of the spin space, and
+//   sum_a lam_a ((1 -+ gamma_mu) x)_a^dag = sum_{a < rank} h(lam)_a h(x)_a^dag
+// with the same half spinors h on both sides, since the lower spins of
+// (1 -+ gamma_mu) x are unitary images of the upper ones.
+//
+// A block is (LINK_THREADS / SP) links x SP groups of slices: group g sums the slices g,
+// g + SP, ..; the groups' sums meet in shared memory in group order.  SP
+// (link_slice_groups) splits a small lattice until its threads fill the SMs,
+// and a large one no further than leaves several blocks per SM to even out
+// the last wave.
+// ---------------------------------------------------------------------------
+constexpr int LINK_THREADS = 128;
+
+// 152 SMs hold 16 warps each at the 128 registers of the SU(3) kernel: the slices are split until
+// two such waves are there.  SU(3) force at 12^3 x 24 x 12 (2.1 waves unsplit) with 1, 2, 4, 8
+// groups: 756, 767, 760, 884 us.
+static int link_slice_groups(long long threads, int Ls) {
+    int sp = 1;
+    while (sp < 8 && 2 * sp <= Ls && threads * sp < 2LL * 152 * 512) sp *= 2;
+    return sp;
 }
 
-__global__ void k_force_u1_2d(const double2* __restrict__ U, const double2* __restrict__ lam,
-                              const double2* __restrict__ x, double* __restrict__ F, int L0, long long V, int Ls,
-                              int anti0, int anti1) {
-    const long long site = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (site >= V) return;
-    const int x0 = (int)(site % L0);
-    for (int mu = 0; mu < 2; ++mu) {
-        long long nb;
-        bool cross;
-        if (mu == 0) { cross = (x0 == L0 - 1); nb = cross ? site - (L0 - 1) : site + 1; }
-        else         { cross = (site + L0 >= V); nb = cross ? site + L0 - V : site + L0; }
-        const double ph = (cross && (mu == 0 ? anti0 : anti1)) ? -1.0 : 1.0;
-        const double2 u = U[mu * V + site];
-        double2 acc1 = make_double2(0.0, 0.0), acc2 = make_double2(0.0, 0.0);
-        for (int s = 0; s < Ls; ++s) {
-            const long long b = (long long)s * V;
-            const double2* l0 = lam + 2 * (b + site);
-            const double2* xn = x + 2 * (b + nb);
-            const double2* ln = lam + 2 * (b + nb);
-            const double2* x0p = x + 2 * (b + site);
-            // lambda(site)^dag (1 - gamma_mu) x(site + mu)
-            double2 t1 = bilinear(l0[0], l0[1], xn[0], xn[1], mu, -1);
-            // lambda(site + mu)^dag (1 + gamma_mu) x(site)
-            double2 t2 = bilinear(ln[0], ln[1], x0p[0], x0p[1], mu, +1);
-            acc1.x += t1.x; acc1.y += t1.y;
-            acc2.x += t2.x; acc2.y += t2.y;
-        }
-        // -1/2 * i U * acc1  +  -1/2 * (-i) conj(U) * acc2, real part
-        const double2 iu = make_double2(-u.y, u.x);                 // i U
-        const double2 miuc = make_double2(-u.y, -u.x);              // -i conj(U)
-        const double r1 = iu.x * acc1.x - iu.y * acc1.y;
-        const double r2 = miuc.x * acc2.x - miuc.y * acc2.y;
-        F[mu * V + site] = -0.5 * ph * (r1 + r2);
-    }
-}
-
-// Complex link gradient of the 2-d U(1) hops: G_mu(y) with
-// Re(lam^dag dD x) = Re(conj(G) dU) for any change dU of U_mu(y) (the backward
-// hop reads conj(U)): G = -1/2 ph [ conj(lam(y)^dag (1 - gamma_mu) x(y + mu))
-//                                 + lam(y + mu)^dag (1 + gamma_mu) x(y) ], summed over s.
-__global__ void k_linkgrad_u1_2d(const double2* __restrict__ lam, const double2* __restrict__ x,
-                                 double2* __restrict__ G, int L0, long long V, int Ls, int anti0, int anti1) {
-    const long long site = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (site >= V) return;
-    const int x0 = (int)(site % L0);
-    for (int mu = 0; mu < 2; ++mu) {
-        long long nb;
-        bool cross;
-        if (mu == 0) { cross = (x0 == L0 - 1); nb = cross ? site - (L0 - 1) : site + 1; }
-        else         { cross = (site + L0 >= V); nb = cross ? site + L0 - V : site + L0; }
-        const double ph = (cross && (mu == 0 ? anti0 : anti1)) ? -1.0 : 1.0;
-        double2 acc = make_double2(0.0, 0.0);
-        for (int s = 0; s < Ls; ++s) {
-            const long long b = (long long)s * V;
-            const double2* l0 = lam + 2 * (b + site);
-            const double2* xn = x + 2 * (b + nb);
-            const double2* ln = lam + 2 * (b + nb);
-            const double2* x0p = x + 2 * (b + site);
-            const double2 t1 = bilinear(l0[0], l0[1], xn[0], xn[1], mu, -1);
-            const double2 t2 = bilinear(ln[0], ln[1], x0p[0], x0p[1], mu, +1);
-            acc.x += t1.x + t2.x;
-            acc.y += -t1.y + t2.y;
-        }
-        G[mu * V + site] = make_double2(-0.5 * ph * acc.x, -0.5 * ph * acc.y);
-    }
-}
-
-// gamma_mu[a][b] of the 4-d chiral basis: [[0, A_mu], [A_mu^dag, 0]] with
-// A_mu = -i sigma_1, -i sigma_2, -i sigma_3, 1 (the basis of the fine operator)
-__device__ __forceinline__ double2 amat64(int mu, int r, int c) {
-    if (mu == 0) return r != c ? make_double2(0.0, -1.0) : make_double2(0.0, 0.0);
-    if (mu == 1) return (r == 0 && c == 1) ? make_double2(-1.0, 0.0)
-                        : (r == 1 && c == 0) ? make_double2(1.0, 0.0) : make_double2(0.0, 0.0);
-    if (mu == 2) return r != c ? make_double2(0.0, 0.0) : make_double2(0.0, r == 0 ? -1.0 : 1.0);
-    return r == c ? make_double2(1.0, 0.0) : make_double2(0.0, 0.0);
-}
-__device__ __forceinline__ double2 gamma64(int mu, int a, int b) {
-    if (a < 2 && b >= 2) return amat64(mu, a, b - 2);
-    if (a >= 2 && b < 2) { const double2 A = amat64(mu, b, a - 2); return make_double2(A.x, -A.y); }
-    return make_double2(0.0, 0.0);
-}
-
-// y = (1 + sgn gamma_mu) v on one site's 4 x 3 spinor
-__device__ __forceinline__ void spin_proj4(const double2* __restrict__ v, int mu, double sgn, double2 (&y)[12]) {
+// v[k] of group 0 += v[k] of groups 1 .. SP - 1, in order; sh holds (SP - 1) * N * TX doubles
+template <int N>
+__device__ __forceinline__ void sum_slice_groups(double (&v)[N], double* sh) {
+    const int TX = blockDim.x, tx = threadIdx.x, ty = threadIdx.y;
+    if (blockDim.y == 1) return;
+    if (ty > 0)
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+        for (int k = 0; k < N; ++k) sh[((ty - 1) * N + k) * TX + tx] = v[k];
+    __syncthreads();
+    if (ty == 0)
+        for (int g = 0; g + 1 < (int)blockDim.y; ++g)
+#pragma unroll
+            for (int k = 0; k < N; ++k) v[k] += sh[(g * N + k) * TX + tx];
+}
+
+// 2-d U(1).  Per link, summed over s, with t1 = lam(y)^dag (1 - gamma_mu) x(y + mu) and
+// t2 = lam(y + mu)^dag (1 + gamma_mu) x(y):  R = Re(t1 + t2), I = Im(t2 - t1).
+//   gradient: Re(lam^dag dD x) = Re(conj(G) dU) for any change dU (the backward hop reads
+//     conj(U)): G = -1/2 ph (R + i I);
+//   FORCE: the derivative along theta (dU = i U dtheta): -1/2 ph (U.x I - U.y R).
+// 16 FP64 instructions per (link, slice) and 4 adds of half spinors per side.
+template <bool FORCE>
+__global__ void __launch_bounds__(LINK_THREADS)
+k_linkgrad_u1_2d(const double2* __restrict__ U, const double2* __restrict__ lam, const double2* __restrict__ x,
+                 double* __restrict__ out, int L0, long long V, int Ls, int anti0, int anti1) {
+    extern __shared__ double link_sh[];
+    const long long site = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const bool in = site < V;
+    const int x0 = (int)(site % L0);
+    const bool cross[2] = {x0 == L0 - 1, site + L0 >= V};
+    const long long nb[2] = {cross[0] ? site - (L0 - 1) : site + 1, cross[1] ? site + L0 - V : site + L0};
+    double v[4] = {0.0, 0.0, 0.0, 0.0};           // R, I for mu = 0, 1
+    if (in)
+        for (int s = threadIdx.y; s < Ls; s += blockDim.y) {
+            const long long b = (long long)s * V;
+            const double2 l0 = __ldg(lam + 2 * (b + site)), l1 = __ldg(lam + 2 * (b + site) + 1);
+            const double2 x0v = __ldg(x + 2 * (b + site)), x1v = __ldg(x + 2 * (b + site) + 1);
+#pragma unroll
+            for (int mu = 0; mu < 2; ++mu) {
+                const double2 m0 = __ldg(lam + 2 * (b + nb[mu])), m1 = __ldg(lam + 2 * (b + nb[mu]) + 1);
+                const double2 y0 = __ldg(x + 2 * (b + nb[mu])), y1 = __ldg(x + 2 * (b + nb[mu]) + 1);
+                // h = c0 -+ (c1 or -i c1): gamma_1 pairs c0 with c1, gamma_2 with -i c1
+                const double2 p = mu == 0 ? l0 - l1 : l0 + times_i(l1), q = mu == 0 ? y0 - y1 : y0 + times_i(y1);
+                const double2 r = mu == 0 ? m0 + m1 : m0 - times_i(m1), t = mu == 0 ? x0v + x1v : x0v - times_i(x1v);
+                v[2 * mu] += p.x * q.x; v[2 * mu] += p.y * q.y; v[2 * mu] += r.x * t.x; v[2 * mu] += r.y * t.y;
+                v[2 * mu + 1] += p.y * q.x; v[2 * mu + 1] -= p.x * q.y;
+                v[2 * mu + 1] += r.x * t.y; v[2 * mu + 1] -= r.y * t.x;
+            }
+        }
+    sum_slice_groups<4>(v, link_sh);
+    if (!in || threadIdx.y != 0) return;
+#pragma unroll
+    for (int mu = 0; mu < 2; ++mu) {
+        const double ph = (cross[mu] && (mu == 0 ? anti0 : anti1)) ? 0.5 : -0.5;
+        const long long t = mu * V + site;
+        if (FORCE) {
+            const double2 u = __ldg(U + t);
+            out[t] = ph * (u.x * v[2 * mu + 1] - u.y * v[2 * mu]);
+        } else {
+            reinterpret_cast<double2*>(out)[t] = make_double2(ph * v[2 * mu], ph * v[2 * mu + 1]);
+        }
+    }
+}
+
+// the half spinor h of (1 + SGN gamma_MU) v in the chiral basis gamma_mu = [[0, A], [A^dag, 0]],
+// A = -i sigma_1, -i sigma_2, -i sigma_3, 1: h = v_up + SGN A v_low
+template <int MU, int SGN>
+__device__ __forceinline__ void half_spinor(const double2* __restrict__ v, double2 (&h)[6]) {
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            double2 acc = v[a * 3 + c];
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const double2 gm = gamma64(mu, a, b);
-                if (gm.x == 0.0 && gm.y == 0.0) continue;
-                const double2 w = v[b * 3 + c];
-                acc.x += sgn * (gm.x * w.x - gm.y * w.y);
-                acc.y += sgn * (gm.x * w.y + gm.y * w.x);
-            }
-            y[a * 3 + c] = acc;
+            const double2 up = __ldg(v + a * 3 + c);
+            const double2 low = __ldg(v + (2 + (MU < 2 ? 1 - a : a)) * 3 + c);
+            double2 w;                                         // A v_low
+            if (MU == 0) w = make_double2(low.y, -low.x);      // -i
+            if (MU == 1) w = a == 0 ? make_double2(-low.x, -low.y) : low;
+            if (MU == 2) w = a == 0 ? make_double2(low.y, -low.x) : make_double2(-low.y, low.x);
+            if (MU == 3) w = low;
+            h[a * 3 + c] = SGN > 0 ? up + w : up - w;
         }
+}
+
+// G += sum_a a_a b_a^dag (colour outer products over the two half spins)
+__device__ __forceinline__ void outer_half(const double2 (&a)[6], const double2 (&b)[6], double (&G)[18]) {
+#pragma unroll
+    for (int sp = 0; sp < 2; ++sp)
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const double2 u = a[sp * 3 + i], w = b[sp * 3 + j];
+                double& re = G[2 * (i * 3 + j)];
+                double& im = G[2 * (i * 3 + j) + 1];
+                re = fma(u.x, w.x, re); re = fma(u.y, w.y, re);
+                im = fma(u.y, w.x, im); im = fma(-u.x, w.y, im);
+            }
+}
+
+template <int MU>
+__device__ __forceinline__ void link_sum_su3(const double2* __restrict__ lam, const double2* __restrict__ x,
+                                             long long V, int Ls, long long site, long long nb, double (&G)[18]) {
+    for (int s = threadIdx.y; s < Ls; s += blockDim.y) {
+        const long long b = (long long)s * V;
+        double2 h[6], k[6];
+        half_spinor<MU, -1>(lam + 12 * (b + site), h);
+        half_spinor<MU, -1>(x + 12 * (b + nb), k);
+        outer_half(h, k, G);
+        half_spinor<MU, 1>(x + 12 * (b + site), h);
+        half_spinor<MU, 1>(lam + 12 * (b + nb), k);
+        outer_half(h, k, G);
+    }
 }
 
 // 4-d SU(3) link gradient G_mu(y) (3 x 3): Re(lam^dag dD x) = Re sum_ij conj(G_ij) dU_ij for any change
@@ -163,14 +186,18 @@ __device__ __forceinline__ void spin_proj4(const double2* __restrict__ v, int mu
 // with y = (1 - gamma_mu) x(y + mu), z = (1 + gamma_mu) x(y) (colour outer products over the spins a).
 // FORCE: the su(3) projection F = Pi(i U G^dag) (traceless Hermitian part), for which
 // Re(lam^dag dD x) = tr(H F) under U -> exp(i eps H) U.
+// grid.y = mu, a compile-time constant of each branch, so that gamma_mu is a choice of
+// components and signs: 192 FP64 instructions per (link, slice), 0.66 ms of the FP64 rate at
+// 12^3 x 24 x 12 (the memory floor is 35 us); measured 0.76 ms.  With gamma_mu looked up at run
+// time and all four spins multiplied out the kernel ran 3.20 ms.
 template <bool FORCE>
-__global__ void k_linkgrad_su3(const double2* __restrict__ U, const double2* __restrict__ lam,
-                               const double2* __restrict__ x, double2* __restrict__ out, int4 L, long long V, int Ls,
-                               int4 anti) {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= 4 * V) return;
-    const int mu = (int)(t / V);
-    const long long site = t % V;
+__global__ void __launch_bounds__(LINK_THREADS, 4)
+k_linkgrad_su3(const double2* __restrict__ U, const double2* __restrict__ lam, const double2* __restrict__ x,
+               double2* __restrict__ out, int4 L, long long V, int Ls, int4 anti) {
+    extern __shared__ double link_sh[];
+    const long long site = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const bool in = site < V;
+    const int mu = blockIdx.y;
     const int Lm = mu == 0 ? L.x : mu == 1 ? L.y : mu == 2 ? L.z : L.w;
     const long long stride = mu == 0 ? 1 : mu == 1 ? (long long)L.x : mu == 2 ? (long long)L.x * L.y
                                                                               : (long long)L.x * L.y * L.z;
@@ -178,35 +205,27 @@ __global__ void k_linkgrad_su3(const double2* __restrict__ U, const double2* __r
     const bool cross = c == Lm - 1;
     const long long nb = cross ? site - (long long)(Lm - 1) * stride : site + stride;
     const int am = mu == 0 ? anti.x : mu == 1 ? anti.y : mu == 2 ? anti.z : anti.w;
-    const double ph = (cross && am) ? -1.0 : 1.0;
-    double2 G[9];
+    const double ph = (cross && am) ? 0.5 : -0.5;
+    double G[18];
 #pragma unroll
-    for (int e = 0; e < 9; ++e) G[e] = make_double2(0.0, 0.0);
-    for (int s = 0; s < Ls; ++s) {
-        const long long b = (long long)s * V;
-        double2 y[12], z[12];
-        spin_proj4(x + 12 * (b + nb), mu, -1.0, y);
-        spin_proj4(x + 12 * (b + site), mu, +1.0, z);
-        const double2* l0 = lam + 12 * (b + site);
-        const double2* ln = lam + 12 * (b + nb);
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-#pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    const double2 li = l0[a * 3 + i], yj = y[a * 3 + j];      // lam_i conj(y_j)
-                    const double2 zi = z[a * 3 + i], mj = ln[a * 3 + j];      // z_i conj(lam'_j)
-                    G[i * 3 + j].x += li.x * yj.x + li.y * yj.y + zi.x * mj.x + zi.y * mj.y;
-                    G[i * 3 + j].y += li.y * yj.x - li.x * yj.y + zi.y * mj.x - zi.x * mj.y;
-                }
+    for (int e = 0; e < 18; ++e) G[e] = 0.0;
+    if (in) {
+        switch (mu) {
+            case 0: link_sum_su3<0>(lam, x, V, Ls, site, nb, G); break;
+            case 1: link_sum_su3<1>(lam, x, V, Ls, site, nb, G); break;
+            case 2: link_sum_su3<2>(lam, x, V, Ls, site, nb, G); break;
+            default: link_sum_su3<3>(lam, x, V, Ls, site, nb, G); break;
+        }
     }
+    sum_slice_groups<18>(G, link_sh);
+    if (!in || threadIdx.y != 0) return;
 #pragma unroll
-    for (int e = 0; e < 9; ++e) G[e] = make_double2(-0.5 * ph * G[e].x, -0.5 * ph * G[e].y);
+    for (int e = 0; e < 18; ++e) G[e] *= ph;
+    const long long t = mu * V + site;
     double2* o = out + 9 * t;
     if (!FORCE) {
 #pragma unroll
-        for (int e = 0; e < 9; ++e) o[e] = G[e];
+        for (int e = 0; e < 9; ++e) o[e] = make_double2(G[2 * e], G[2 * e + 1]);
         return;
     }
     // A = i U G^dag; F = (A + A^dag) / 2 - tr / 3
@@ -219,9 +238,10 @@ __global__ void k_linkgrad_su3(const double2* __restrict__ U, const double2* __r
             double re = 0.0, im = 0.0;       // sum_k U_ik conj(G_jk)
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                const double2 a = u[i * 3 + k], g = G[j * 3 + k];
-                re += a.x * g.x + a.y * g.y;
-                im += a.y * g.x - a.x * g.y;
+                const double2 a = u[i * 3 + k];
+                const double gx = G[2 * (j * 3 + k)], gy = G[2 * (j * 3 + k) + 1];
+                re += a.x * gx + a.y * gy;
+                im += a.y * gx - a.x * gy;
             }
             A[i * 3 + j] = make_double2(-im, re);    // times i
         }
@@ -235,6 +255,25 @@ __global__ void k_linkgrad_su3(const double2* __restrict__ U, const double2* __r
             if (i == j) f.x -= tr;
             o[i * 3 + j] = f;
         }
+}
+
+template <bool FORCE>
+static dwf_status launch_link(const Geom& G, const void* U, const void* lam, const void* x, void* out,
+                              cudaStream_t st) {
+    const bool su3 = G.nd == 4;
+    const int sp = link_slice_groups(su3 ? 4 * G.V : G.V, G.Ls);
+    const dim3 block(LINK_THREADS / sp, sp);
+    const dim3 grid((unsigned)((G.V + block.x - 1) / block.x), su3 ? 4u : 1u);
+    const size_t sh = (size_t)(sp - 1) * (su3 ? 18 : 4) * block.x * sizeof(double);
+    if (su3)
+        k_linkgrad_su3<FORCE><<<grid, block, sh, st>>>((const double2*)U, (const double2*)lam, (const double2*)x,
+                                                       (double2*)out, make_int4(G.L[0], G.L[1], G.L[2], G.L[3]), G.V,
+                                                       G.Ls, make_int4(G.anti[0], G.anti[1], G.anti[2], G.anti[3]));
+    else
+        k_linkgrad_u1_2d<FORCE><<<grid, block, sh, st>>>((const double2*)U, (const double2*)lam, (const double2*)x,
+                                                         (double*)out, G.L[0], G.V, G.Ls, G.anti[0], G.anti[1]);
+    DWF_CHECK_LAUNCH();
+    return DWF_OK;
 }
 
 }  // namespace dwf
@@ -283,21 +322,11 @@ dwf_status dwf_link_force(const dwf_geom* g, const void* U, const void* lam, con
     DWF_TRY(check_geom(g, &G));
     if (G.V == 0) return DWF_OK;
     if (!U || !lam || !x || !force) { set_error("NULL device pointer"); return DWF_ERR_ARG; }
-    const int thr = 256;
-    cudaStream_t st = as_stream(stream);
-    if (G.nd == 2 && G.group == DWF_U1) {
-        k_force_u1_2d<<<(unsigned)((G.V + thr - 1) / thr), thr, 0, st>>>(
-            (const double2*)U, (const double2*)lam, (const double2*)x, force, G.L[0], G.V, G.Ls, G.anti[0], G.anti[1]);
-    } else if (G.nd == 4 && G.group == DWF_SU3) {
-        k_linkgrad_su3<true><<<(unsigned)((4 * G.V + thr - 1) / thr), thr, 0, st>>>(
-            (const double2*)U, (const double2*)lam, (const double2*)x, (double2*)force,
-            make_int4(G.L[0], G.L[1], G.L[2], G.L[3]), G.V, G.Ls, make_int4(G.anti[0], G.anti[1], G.anti[2], G.anti[3]));
-    } else {
+    if (!(G.nd == 2 && G.group == DWF_U1) && !(G.nd == 4 && G.group == DWF_SU3)) {
         set_error("the link force is built for 2-d U(1) and 4-d SU(3)");
         return DWF_ERR_UNSUPPORTED;
     }
-    DWF_CHECK_LAUNCH();
-    return DWF_OK;
+    return launch_link<true>(G, U, lam, x, force, as_stream(stream));
 }
 
 dwf_status dwf_link_grad(const dwf_geom* g, const void* lam, const void* x, void* grad, void* stream) {
@@ -306,21 +335,11 @@ dwf_status dwf_link_grad(const dwf_geom* g, const void* lam, const void* x, void
     DWF_TRY(check_geom(g, &G));
     if (G.V == 0) return DWF_OK;
     if (!lam || !x || !grad) { set_error("NULL device pointer"); return DWF_ERR_ARG; }
-    const int thr = 256;
-    cudaStream_t st = as_stream(stream);
-    if (G.nd == 2 && G.group == DWF_U1) {
-        k_linkgrad_u1_2d<<<(unsigned)((G.V + thr - 1) / thr), thr, 0, st>>>(
-            (const double2*)lam, (const double2*)x, (double2*)grad, G.L[0], G.V, G.Ls, G.anti[0], G.anti[1]);
-    } else if (G.nd == 4 && G.group == DWF_SU3) {
-        k_linkgrad_su3<false><<<(unsigned)((4 * G.V + thr - 1) / thr), thr, 0, st>>>(
-            nullptr, (const double2*)lam, (const double2*)x, (double2*)grad,
-            make_int4(G.L[0], G.L[1], G.L[2], G.L[3]), G.V, G.Ls, make_int4(G.anti[0], G.anti[1], G.anti[2], G.anti[3]));
-    } else {
+    if (!(G.nd == 2 && G.group == DWF_U1) && !(G.nd == 4 && G.group == DWF_SU3)) {
         set_error("the link gradient is built for 2-d U(1) and 4-d SU(3)");
         return DWF_ERR_UNSUPPORTED;
     }
-    DWF_CHECK_LAUNCH();
-    return DWF_OK;
+    return launch_link<false>(G, nullptr, lam, x, grad, as_stream(stream));
 }
 
 }  // extern "C"
