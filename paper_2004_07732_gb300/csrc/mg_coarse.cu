@@ -687,30 +687,34 @@ __device__ __forceinline__ long long fine_idx(const TransferParams& p, int s, lo
     return 2 * (((((long long)(s >> 1)) * p.NB + (x >> 5)) * p.dof + d) * 32 + (x & 31)) + (s & 1);
 }
 
+// Aggregate of a site, and site l of an aggregate, in unsigned 32 bits: the links, near-null
+// vectors and prolongator of a hierarchy with 2^32 sites would take 500 GB.  The loops are unrolled
+// so that the parameter arrays are read with constant indexes.
 __device__ __forceinline__ long long agg_of(const TransferParams& p, long long site) {
-    long long xc = 0, stride = 1;
-    long long rem = site;
-    for (int mu = 0; mu < p.nd; ++mu) {
-        const int c = (int)(rem % p.L[mu]);
-        rem /= p.L[mu];
-        xc += (long long)(c / p.b[mu]) * stride;
-        stride *= p.Lc[mu];
-    }
+    unsigned xc = 0, stride = 1, rem = (unsigned)site;
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu)
+        if (mu < p.nd) {
+            const unsigned q = rem / (unsigned)p.L[mu], c = rem - q * (unsigned)p.L[mu];
+            rem = q;
+            xc += c / (unsigned)p.b[mu] * stride;
+            stride *= (unsigned)p.Lc[mu];
+        }
     return xc;
 }
 
 __device__ __forceinline__ long long agg_site(const TransferParams& p, long long xc, int l) {
-    long long site = 0, stride = 1;
-    long long rem = xc;
-    int lr = l;
-    for (int mu = 0; mu < p.nd; ++mu) {
-        const int c = (int)(rem % p.Lc[mu]);
-        rem /= p.Lc[mu];
-        const int lc = lr % p.b[mu];
-        lr /= p.b[mu];
-        site += (long long)(c * p.b[mu] + lc) * stride;
-        stride *= p.L[mu];
-    }
+    unsigned site = 0, stride = 1, rem = (unsigned)xc, lr = (unsigned)l;
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu)
+        if (mu < p.nd) {
+            const unsigned q = rem / (unsigned)p.Lc[mu], c = rem - q * (unsigned)p.Lc[mu];
+            rem = q;
+            const unsigned lq = lr / (unsigned)p.b[mu], lc = lr - lq * (unsigned)p.b[mu];
+            lr = lq;
+            site += (c * (unsigned)p.b[mu] + lc) * stride;
+            stride *= (unsigned)p.L[mu];
+        }
     return site;
 }
 
@@ -719,77 +723,165 @@ __device__ __forceinline__ int chir_dof(const TransferParams& p, int c, int cd) 
     return (2 * c + cd / p.ncol) * p.ncol + cd % p.ncol;
 }
 
-// grid.y = right-hand side (vectors back to back); skip[r]: per right-hand side
-__global__ void k_restrict(const float2* __restrict__ P, const float2* __restrict__ r, float2* __restrict__ out,
-                           TransferParams p, const int* skip) {
+// Restriction.  A group of J = nchd * nvec threads owns one (aggregate, chirality): thread
+// (cd, k) sums conj(P[x][c][cd][k]) r[x][cd] over the aggregate's sites x, whose J prolongator
+// values are one contiguous run that the group reads as such, all sites' loads in flight; the
+// cd sums meet in shared memory.  The two chiralities of an aggregate are neighbouring groups,
+// so every site's prolongator is read in one piece.  grid.y = right-hand side (vectors back to
+// back); skip[r]: per right-hand side.  Bound by the read of P (and by launch latency below a
+// few MB): with one thread per output, walking the sites one after the other through the index
+// divisions, 256^2 took 30 us and 12^3 x 24 (nvec 24) 132 us; the two transfers and two coarse
+// applies of a 256^2 hierarchy together went from 96.6 to 51.3 us.
+constexpr int RESTRICT_THREADS = 288;   // both chiralities of one aggregate at 4-d, nvec 24
+constexpr int RESTRICT_TABLE = 2048;    // aggregates up to this many sites keep their offsets in shared memory
+
+__global__ void __launch_bounds__(RESTRICT_THREADS)
+k_restrict(const float2* __restrict__ P, const float2* __restrict__ r, float2* __restrict__ out, TransferParams p,
+           const int* skip) {
     if (skip && skip[blockIdx.y]) return;
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long total = p.Vc * p.Ls_c * p.ncd;
-    if (t >= total) return;
+    __shared__ long long off[RESTRICT_TABLE];
+    __shared__ float2 red[RESTRICT_THREADS];
+    const int J = p.nchd * p.nvec;
+    const int G = blockDim.x / J;
+    const bool table = p.nb <= RESTRICT_TABLE;
+    if (table)
+        for (int l = threadIdx.x; l < p.nb; l += blockDim.x) off[l] = agg_site(p, 0, l);
+    __syncthreads();
+    const long long nc = p.Vc * p.Ls_c * p.ncd;
     r += (long long)blockIdx.y * p.V * p.Ls * p.dof;
-    out += (long long)blockIdx.y * total;
-    const int i = (int)(t % p.ncd);
-    const long long rest = t / p.ncd;
-    const long long xc = rest % p.Vc;
-    const int s = (int)(rest / p.Vc);
-    const int c = i / p.nvec, k = i % p.nvec;
+    out += (long long)blockIdx.y * nc;
+    const int j = threadIdx.x % J;
+    const int k = j % p.nvec, cd = j / p.nvec;
+    const long long g = (long long)blockIdx.x * G + threadIdx.x / J;
+    const int c = (int)(g & 1);
+    const long long xs = g >> 1;
+    const bool in = xs < p.Vc * (p.bulk ? p.Ls : 1);
+    const long long xc = xs % p.Vc;
+    // Phat_- P^dag P_- r_1 on coarse slice 1, Phat_+ P^dag P_+ r_Ls on coarse slice Lhat_s; bulk: every slice
+    const int sf = p.bulk ? (int)(xs / p.Vc) : (c == 1 ? 0 : p.Ls - 1);
     float2 acc = make_float2(0.f, 0.f);
-    int sf = -1;
-    if (c == 1 && s == 0) sf = 0;                 // Phat_- P^dag P_- r_1 on coarse slice 1
-    if (c == 0 && s == p.Ls_c - 1) sf = p.Ls - 1; // Phat_+ P^dag P_+ r_Ls on coarse slice Lhat_s
-    if (p.bulk) sf = s;                           // bulk: every slice
-    if (sf >= 0) {
+    if (in) {
+        const int d = chir_dof(p, c, cd);
+        const long long base = agg_site(p, xc, 0);
+        const float2* Pc = P + c * J + j;
+#pragma unroll 8
         for (int l = 0; l < p.nb; ++l) {
-            const long long x = agg_site(p, xc, l);
-            for (int cd = 0; cd < p.nchd; ++cd)
-                acc = cfma_conj(P[((x * 2 + c) * p.nchd + cd) * p.nvec + k], r[fine_idx(p, sf, x, chir_dof(p, c, cd))],
-                                acc);
+            const long long x = base + (table ? off[l] : agg_site(p, 0, l));
+            acc = cfma_conj(__ldg(Pc + x * 2 * J), __ldg(r + fine_idx(p, sf, x, d)), acc);
         }
     }
-    out[t] = acc;
+    if (p.nchd > 1) {
+        red[threadIdx.x] = acc;
+        __syncthreads();
+        if (cd == 0)
+            for (int q = 1; q < p.nchd; ++q) {
+                acc.x += red[threadIdx.x + q * p.nvec].x;
+                acc.y += red[threadIdx.x + q * p.nvec].y;
+            }
+    }
+    if (!in || cd != 0) return;
+    float2* o = out + xc * p.ncd + c * p.nvec + k;
+    if (p.bulk) {
+        o[sf * p.Vc * p.ncd] = acc;
+    } else {
+        const int wall = c == 1 ? 0 : p.Ls_c - 1;
+        for (int s = 0; s < p.Ls_c; ++s) o[s * p.Vc * p.ncd] = s == wall ? acc : make_float2(0.f, 0.f);
+    }
 }
 
-__global__ void k_prolong(const float2* __restrict__ P, const float2* __restrict__ e, float2* __restrict__ out,
-                          TransferParams p, const int* skip) {
-    if (skip && skip[blockIdx.y]) return;
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long total = p.V * p.Ls * p.dof;
-    if (t >= total) return;
-    e += (long long)blockIdx.y * p.Vc * p.Ls_c * p.ncd;
-    out += (long long)blockIdx.y * total;
-    // thread t writes element t of the output layout: (s, site, d) from the canonical or packed order
-    int d, s;
-    long long x;
-    if (!p.packed) {
-        d = (int)(t % p.dof);
-        const long long rest = t / p.dof;
-        x = rest % p.V;
-        s = (int)(rest / p.V);
+// sum_k P[k] e[k] over one prolongator row; V4: rows and e are 16-byte aligned and nvec is even
+template <bool V4>
+__device__ __forceinline__ float2 prolong_row(const float2* __restrict__ Pr, const float2* __restrict__ ev, int nvec) {
+    float2 acc = make_float2(0.f, 0.f);
+    if (V4) {
+#pragma unroll 4
+        for (int k = 0; k < nvec; k += 2) {
+            const float4 a = __ldg(reinterpret_cast<const float4*>(Pr + k));
+            const float4 b = __ldg(reinterpret_cast<const float4*>(ev + k));
+            acc = cfma(make_float2(a.x, a.y), make_float2(b.x, b.y), acc);
+            acc = cfma(make_float2(a.z, a.w), make_float2(b.z, b.w), acc);
+        }
     } else {
-        const int s1 = (int)(t & 1);
-        const long long q = t >> 1;
-        const int i = (int)(q & 31);
-        const long long q2 = q >> 5;
-        d = (int)(q2 % p.dof);
-        const long long q3 = q2 / p.dof;
-        x = (q3 % p.NB) * 32 + i;
-        s = (int)(q3 / p.NB) * 2 + s1;
+        for (int k = 0; k < nvec; ++k) acc = cfma(__ldg(Pr + k), __ldg(ev + k), acc);
+    }
+    return acc;
+}
+
+// Prolongation.  The first `wall_blocks` blocks of a row take one thread per (site, chirality,
+// dof): P_- P e_1 onto fine slice 1 and P_+ P e_{Lhat_s} onto slice Ls, with the zeros of the
+// other chirality there; the remaining blocks only store the zeros of the slices in between
+// (all of the output but two slices), as one contiguous range of zero_n complex values from
+// zero_0.  Bulk: no range of zeros, every slice is computed.  V4: the layout allows 16-byte
+// accesses (see prolong_wall).  Bound by the stores: 16.8 MB at 256^2 x 16, 64 MB at
+// 12^3 x 24 x 16; one thread per value with its index divisions took 34 us and 160 us.
+constexpr int PROLONG_ZERO = 16;   // complex values stored per thread of a zero block
+template <bool V4>
+__global__ void __launch_bounds__(256)
+k_prolong(const float2* __restrict__ P, const float2* __restrict__ e, float2* __restrict__ out, TransferParams p,
+          unsigned wall_blocks, long long zero_0, long long zero_n, const int* skip) {
+    if (skip && skip[blockIdx.y]) return;
+    e += (long long)blockIdx.y * p.Vc * p.Ls_c * p.ncd;
+    out += (long long)blockIdx.y * p.V * p.Ls * p.dof;
+    if (blockIdx.x >= wall_blocks) {
+        const long long b0 = (long long)(blockIdx.x - wall_blocks) * (256 * PROLONG_ZERO);
+        if (V4) {
+            float4* o = reinterpret_cast<float4*>(out + zero_0);
+#pragma unroll
+            for (int q = 0; q < PROLONG_ZERO / 2; ++q) {
+                const long long i = b0 / 2 + q * 256 + threadIdx.x;
+                if (i < zero_n / 2) o[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        } else {
+            for (int q = 0; q < PROLONG_ZERO; ++q) {
+                const long long i = b0 + q * 256 + threadIdx.x;
+                if (i < zero_n) out[zero_0 + i] = make_float2(0.f, 0.f);
+            }
+        }
+        return;
+    }
+    const long long t = (long long)blockIdx.x * 256 + threadIdx.x;
+    if (t >= p.V * p.dof) return;
+    // site fastest within a block of 32 sites in the packed layout, dof fastest in the canonical one
+    int d;
+    long long x;
+    if (p.packed) {
+        const long long q = t >> 5;
+        d = (int)(q % p.dof);
+        x = (q / p.dof) * 32 + (t & 31);
+    } else {
+        d = (int)(t % p.dof);
+        x = t / p.dof;
     }
     int c, cd;
     if (p.nd == 2) { c = d; cd = 0; }
     else { const int spin = d / p.ncol; c = spin / 2; cd = (spin % 2) * p.ncol + d % p.ncol; }
-    float2 acc = make_float2(0.f, 0.f);
-    int sc = -1;
-    if (c == 1 && s == 0) sc = 0;                 // P_- P e_1 on fine slice 1
-    if (c == 0 && s == p.Ls - 1) sc = p.Ls_c - 1; // P_+ P e_{Lhat_s} on fine slice Ls
-    if (p.bulk) sc = s;                           // bulk: every slice
-    if (sc >= 0) {
-        const long long xc = agg_of(p, x);
-        const float2* ev = e + ((long long)sc * p.Vc + xc) * p.ncd + c * p.nvec;
-        const float2* Pr = P + ((x * 2 + c) * p.nchd + cd) * p.nvec;
-        for (int k = 0; k < p.nvec; ++k) acc = cfma(Pr[k], ev[k], acc);
+    const float2* Pr = P + ((x * 2 + c) * p.nchd + cd) * p.nvec;
+    const float2* ev = e + agg_of(p, x) * p.ncd + c * p.nvec;
+    const float2 zero = make_float2(0.f, 0.f);
+    if (p.bulk) {
+        for (int s = 0; s < p.Ls; ++s)
+            out[fine_idx(p, s, x, d)] = prolong_row<V4>(Pr, ev + (long long)s * p.Vc * p.ncd, p.nvec);
+        return;
     }
-    out[t] = acc;
+    const float2 v = prolong_row<V4>(Pr, ev + (long long)(c == 1 ? 0 : p.Ls_c - 1) * p.Vc * p.ncd, p.nvec);
+    if (p.packed) {
+        // slice pairs (0, 1) and (Ls - 2, Ls - 1): one pair when Ls = 2
+        const float2 first = c == 1 ? v : zero, last = c == 0 ? v : zero;
+        if (p.Ls == 2) {
+            out[fine_idx(p, 0, x, d)] = first;
+            out[fine_idx(p, 1, x, d)] = last;
+        } else {
+            out[fine_idx(p, 0, x, d)] = first;
+            out[fine_idx(p, 1, x, d)] = zero;
+            out[fine_idx(p, p.Ls - 2, x, d)] = zero;
+            out[fine_idx(p, p.Ls - 1, x, d)] = last;
+        }
+    } else if (p.Ls == 1) {
+        out[fine_idx(p, 0, x, d)] = v;
+    } else {
+        out[fine_idx(p, 0, x, d)] = c == 1 ? v : zero;
+        out[fine_idx(p, p.Ls - 1, x, d)] = c == 0 ? v : zero;
+    }
 }
 
 static TransferParams transfer_params(const dwf_mg* h) {
@@ -824,10 +916,12 @@ dwf_status restrict_wall(const dwf_mg* h, const float2* r_fine, float2* r_coarse
                          int nrhs, bool packed) {
     TransferParams p = transfer_params(h);
     if (packed) { DWF_TRY(check_packed_transfer(p)); p.packed = 1; }
-    const long long total = p.Vc * p.Ls_c * p.ncd;
     if (nrhs < 1 || nrhs > 65535) { set_error("nrhs must be in [1, 65535]"); return DWF_ERR_ARG; }
-    k_restrict<<<dim3((unsigned)((total + 255) / 256), (unsigned)nrhs), 256, 0, st>>>(h->P32, r_fine, r_coarse, p,
-                                                                                       skip);
+    const int J = p.nchd * p.nvec;                       // at most 6 * 32
+    const int G = RESTRICT_THREADS / J;
+    const long long groups = 2 * p.Vc * (p.bulk ? p.Ls : 1);
+    k_restrict<<<dim3((unsigned)((groups + G - 1) / G), (unsigned)nrhs), G * J, 0, st>>>(h->P32, r_fine, r_coarse, p,
+                                                                                          skip);
     DWF_CHECK_LAUNCH();
     return DWF_OK;
 }
@@ -836,10 +930,20 @@ dwf_status prolong_wall(const dwf_mg* h, const float2* e_coarse, float2* e_fine,
                         int nrhs, bool packed) {
     TransferParams p = transfer_params(h);
     if (packed) { DWF_TRY(check_packed_transfer(p)); p.packed = 1; }
-    const long long total = p.V * p.Ls * p.dof;
     if (nrhs < 1 || nrhs > 65535) { set_error("nrhs must be in [1, 65535]"); return DWF_ERR_ARG; }
-    k_prolong<<<dim3((unsigned)((total + 255) / 256), (unsigned)nrhs), 256, 0, st>>>(h->P32, e_coarse, e_fine, p,
-                                                                                      skip);
+    const long long plane = p.V * p.dof;                 // one slice; a pair of slices in the packed layout is two
+    const unsigned wall_blocks = (unsigned)((plane + 255) / 256);
+    const int ends = packed ? 2 : 1;                     // slices the wall threads store at each end
+    const long long zero_0 = ends * plane;
+    const long long zero_n = p.bulk || p.Ls <= 2 * ends ? 0 : (p.Ls - 2 * ends) * plane;
+    const unsigned zero_blocks = (unsigned)((zero_n + 256 * PROLONG_ZERO - 1) / (256 * PROLONG_ZERO));
+    const dim3 grid(wall_blocks + zero_blocks, (unsigned)nrhs);
+    // 16-byte accesses: prolongator rows, coarse vectors and the zero range start on 16-byte boundaries (dof is
+    // even, so plane is) when nvec is even and the caller's vectors are aligned
+    if (p.nvec % 2 == 0 && aligned16(e_coarse) && aligned16(e_fine))
+        k_prolong<true><<<grid, 256, 0, st>>>(h->P32, e_coarse, e_fine, p, wall_blocks, zero_0, zero_n, skip);
+    else
+        k_prolong<false><<<grid, 256, 0, st>>>(h->P32, e_coarse, e_fine, p, wall_blocks, zero_0, zero_n, skip);
     DWF_CHECK_LAUNCH();
     return DWF_OK;
 }
