@@ -74,6 +74,8 @@ __device__ __forceinline__ void cadd4(float4& x, const float4 a, const float2 c)
     x.z += c.x * a.z - c.y * a.w; x.w += c.x * a.w + c.y * a.z;
 }
 
+static dim3 row_grid(long long n2, int nrhs, int cap = 1216);
+
 #define ROW_LOOP(i, n2) for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < (n2); i += (long long)gridDim.x * blockDim.x)
 
 // ---- element-wise kernels; n = complex values per right-hand side (even) ----
@@ -370,169 +372,386 @@ __global__ void __launch_bounds__(RED_THREADS) k_bmaxpy(float2* __restrict__ w, 
     }
 }
 
-// One GCR step of the coarse solve with a single classical Gram-Schmidt pass,
-// in one reduction pass and one element-wise pass.  The reduction reads the
-// image w = A p_k, the residual r and the orthogonalised images W_j (j < k)
-// once and sums d_j = <W_j, w>, |w|^2, <w, r> and |r|^2.  The W_j are mutually
-// orthogonal and r is orthogonal to every W_j, so with w' = w - sum_j c_j W_j:
-//   c_j = d_j / |W_j|^2,   |w'|^2 = |w|^2 - sum_j |d_j|^2 / |W_j|^2,
-//   alpha = <w', r> / |w'|^2 = <w, r> / |w'|^2,
-//   |r - alpha w'|^2 = |r|^2 - |<w, r>|^2 / |w'|^2,
-// and the element-wise pass forms w' and r - alpha w' without a reduction.
-// The residual norm is exact at every step (|r|^2 is summed afresh); only the
-// one-step prediction decides convergence.  A direction with |w'|^2 below
-// BSTEP_BREAK |w|^2 is not resolved by FP32 sums: its row stops (alpha = 0).
-constexpr int BSTEP_BLOCKS = 512;     // bound on the blocks per row of the reduction pass
+// ---------------------------------------------------------------------------
+// GCR in blocks of up to SB steps (cgs_passes = 1): the directions of a block are
+// p_0 = r, p_1 = A p_0, .., p_{m-1} = A p_{m-2}, which span the same Krylov space
+// as m single steps, so the block ends at the residual that m single steps end
+// at (the minimum over that space).  Its images w_i = A p_i are orthogonalised
+// together: one reduction pass reads every vector of the basis once for all of
+// the block and one element-wise pass writes the block's orthogonal images and the new
+// residual, where single steps pass over the basis twice per step.  8 steps
+// take 45 passes over a vector instead of 128, 16 steps 123 instead of 420.
+//
+// With W_j the orthogonal images so far (r is orthogonal to them), the reduction
+// sums d_ij = <W_j, w_i>, G_ab = <w_a, w_b>, <w_i, r> and |r|^2, and the rest is
+// algebra on scalars in FP64:
+//   c_ij = d_ij / |W_j|^2,   G'_ab = G_ab - sum_j conj(d_aj) d_bj / |W_j|^2,
+//   G' = L D L^H by elimination: w'_i = w_i - sum_j c_ij W_j - sum_{l<i} L_il w'_l,
+//   |w'_i|^2 = D_i,  <w'_i, r> = <w_i, r> - sum_{l<i} conj(L_il) <w'_l, r>,
+//   alpha_i = <w'_i, r> / D_i,   |r'|^2 = |r|^2 - sum_i |<w'_i, r>|^2 / D_i.
+// |r|^2 is summed afresh in every block; only the prediction for its end
+// decides convergence.  A direction with D_i below BSTEP_BREAK |w_i|^2 is not
+// resolved by FP32 sums: it and the rest of its block are dropped (alpha = 0),
+// and a block that loses its first direction ends that row's coarse solve.
+// SB = 4: the powers of A in a block have a Gram matrix of condition 4e4 on the
+// 2-d and 4-d operators (FP32 sums resolve it; 8 powers reach 4e10 and do not).
+// Against single steps: 256^2 x 16 gradient step (two solves to 1e-12) 1017 -> 630 ms,
+// 12^3 x 24 x 16 solve 1011 -> 614 ms, 14 sources on 64^2, 128^2, 256^2 1282 -> 764 ms, with the
+// same iteration counts.
+// ---------------------------------------------------------------------------
+constexpr int SB = 4;
 constexpr double BSTEP_BREAK = 1e-5;
+constexpr int BLK_Q0 = 25;            // Gram 4 + 2 * 6, <w_i, r> 2 * 4, |r|^2
+constexpr int BLK_KM = 12;            // basis vectors one thread takes together; more go SB to a group (grid.z)
+constexpr int BLK_GROUP = 10;         // blocks of a row whose partial sums meet first
+constexpr int BLK_GROUPS_MAX = 31;    // 304 blocks in groups of 10
+// quantity of d_ij: BLK_Q0 + 2 (SB j + i) (+ 1: Im)
 
-template <int KM>
-__global__ void __launch_bounds__(RED_THREADS) k_bstep_dots(float2* const* __restrict__ W, const float2* __restrict__ w,
-                                                            const float2* __restrict__ res, long long n, int k,
-                                                            double* __restrict__ part, unsigned* counters, BGcr* g,
-                                                            int* steps, int* done, const double* ref2, double tol2,
-                                                            int* iters, int maxit) {
-    constexpr int NQ = 2 * KM + 4;     // |w|^2, Re / Im <w, r>, |r|^2, then Re / Im d_j
-    const int r = blockIdx.y;
-    if (done[r]) return;
-    __shared__ const float4* Wp[KM];
-    __shared__ double sh[NQ][RED_THREADS / 32];
-    __shared__ double tot[NQ];
-    for (int j = threadIdx.x; j < k; j += blockDim.x) Wp[j] = reinterpret_cast<const float4*>(W[j] + r * n);
-    __syncthreads();
-    const float4* w4 = reinterpret_cast<const float4*>(w + r * n);
-    const float4* r4 = reinterpret_cast<const float4*>(res + r * n);
-    float re[KM], im[KM];
+// The sums over a warp of N quantities per lane (N a multiple of 32): afterwards v[q] of lane l,
+// q < N / 32, is the sum of quantity l N / 32 + q.  Every exchange halves the quantities a lane
+// still carries: N - N / 32 shuffles, where a tree per quantity takes 5 N.
+template <int N>
+__device__ __forceinline__ void warp_sums(float (&v)[N]) {
+    const int lane = threadIdx.x & 31;
+    int half = N / 2;
 #pragma unroll
-    for (int j = 0; j < KM; ++j) { re[j] = 0.f; im[j] = 0.f; }
-    float ww = 0.f, wr = 0.f, wi = 0.f, rr = 0.f;
-    ROW_LOOP(i, n >> 1) {
-        const float4 a = w4[i], b = r4[i];
+    for (int off = 16; off > 0; off >>= 1, half >>= 1) {
+        const bool up = lane & off;
 #pragma unroll
-        for (int j = 0; j < KM; ++j)
-            if (j < k) cdot4(Wp[j][i], a, re[j], im[j]);
-        ww += a.x * a.x + a.y * a.y + a.z * a.z + a.w * a.w;
-        cdot4(a, b, wr, wi);
-        rr += b.x * b.x + b.y * b.y + b.z * b.z + b.w * b.w;
+        for (int i = 0; i < N / 2; ++i)
+            if (i < half) {
+                const float send = up ? v[i] : v[i + half];
+                const float keep = up ? v[i + half] : v[i];
+                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+            }
     }
-    const int nq = 2 * k + 4;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // the tree over each warp in FP32, every sum across warps and blocks in FP64
-    float v[NQ];
-    v[0] = ww; v[1] = wr; v[2] = wi; v[3] = rr;
+}
+
+// The scalars of a block from the totals of its reduction (shared memory), by one warp: rows
+// k .. k + m - 1 of C, nrm and A, then |r'|^2 and, with `done`, the convergence test.  An FP64
+// instruction holds the SM's FP64 unit 16 clocks whether one lane or 32 take part, so the
+// elimination runs over the lanes: lane 8 a + b holds M_ab = G'_ab for b < SB and
+// M_a,SB = <w_a, r>, and step l subtracts conj(L_al) M_lb everywhere at once (one thread alone
+// took about 6 us).
+__device__ __forceinline__ void blk_scalars(const double* tot, int k, int m, BGcr& G, int* steps, int* done, double ref2,
+                                            double tol2, int* iters, int maxit) {
+    __shared__ double inv[BK_MAX];
+    __shared__ double2 cc[BK_MAX][SB];
+    const int lane = threadIdx.x & 31;
+    const int a = lane >> 3, b = lane & 7;
+    const int it0 = done ? *iters : 0;
+    if (lane < k) {                                              // k < BK_MAX = 32
+        const double nn = G.nrm[lane];
+        inv[lane] = nn > 0 ? 1.0 / nn : 0.0;
+    }
+    __syncwarp();
+    for (int e = lane; e < SB * k; e += 32) {
+        const int i = e % SB, j = e / SB;
+        const double2 c = make_double2(tot[BLK_Q0 + 2 * e] * inv[j], tot[BLK_Q0 + 2 * e + 1] * inv[j]);
+        cc[j][i] = c;
+        if (i < m) { G.C[k + i][j][0] = c.x; G.C[k + i][j][1] = c.y; }
+    }
+    __syncwarp();
+    double2 M = make_double2(0.0, 0.0);
+    if (b < SB) {
+        const int lo = a < b ? a : b, hi = a < b ? b : a;
+        if (a == b) M.x = tot[a];
+        else {
+            M.x = tot[4 + hi * (hi - 1) + 2 * lo];
+            M.y = (a < b ? 1.0 : -1.0) * tot[5 + hi * (hi - 1) + 2 * lo];
+        }
+        for (int j = 0; j < k; ++j) {
+            const double2 c = cc[j][a];
+            const double dx = tot[BLK_Q0 + 2 * (SB * j + b)], dy = tot[BLK_Q0 + 2 * (SB * j + b) + 1];
+            M.x -= c.x * dx; M.x -= c.y * dy;
+            M.y -= c.x * dy; M.y += c.y * dx;
+        }
+    } else if (b == SB) {
+        M = make_double2(tot[16 + 2 * a], tot[17 + 2 * a]);
+    }
+    const int left = done ? (maxit > it0 ? maxit - it0 : 1) : m;   // steps the iteration cap leaves
+    const int take = left < m ? left : m;
+    bool ok = true, first = true;
+    double fall = 0.0;                                           // of |r|^2: this lane's share
 #pragma unroll
-    for (int j = 0; j < KM; ++j) { v[4 + 2 * j] = re[j]; v[5 + 2 * j] = im[j]; }
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        if (q < nq) {                                             // block-uniform
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) v[q] += __shfl_down_sync(0xffffffffu, v[q], off);
-            if (lane == 0) sh[q][warp] = (double)v[q];
+    for (int l = 0; l < SB; ++l) {
+        if (l >= m) break;
+        const double d = __shfl_sync(0xffffffffu, M.x, 9 * l);
+        if (!(d > BSTEP_BREAK * tot[l])) { ok = false; if (l == 0) first = false; }
+        const bool use = ok && l < take;
+        const double id = use ? 1.0 / d : 0.0;
+        const double2 row = make_double2(__shfl_sync(0xffffffffu, M.x, 8 * l + b), __shfl_sync(0xffffffffu, M.y, 8 * l + b));
+        const double2 la = make_double2(__shfl_sync(0xffffffffu, M.x, 8 * l + a), __shfl_sync(0xffffffffu, M.y, 8 * l + a));
+        if (a == l) {                                            // this lane's M is M_lb
+            const double2 q = make_double2(M.x * id, M.y * id);
+            if (b < m && b > l) { G.C[k + b][k + l][0] = q.x; G.C[k + b][k + l][1] = q.y; }
+            if (b == SB) {
+                G.A[k + l][0] = q.x; G.A[k + l][1] = q.y;
+                fall = M.x * q.x + M.y * q.y;
+            }
+            if (b == l) G.nrm[k + l] = use ? d : 0.0;
+        } else if (a > l) {
+            const double lx = la.x * id, ly = la.y * id;         // L_al
+            M.x -= lx * row.x; M.x -= ly * row.y;
+            M.y -= lx * row.y; M.y += ly * row.x;
         }
     }
+    double rr = tot[24];
+#pragma unroll
+    for (int l = 0; l < SB; ++l) rr -= __shfl_sync(0xffffffffu, fall, 8 * l + SB);
+    if (lane != 0) return;
+    G.rr2 = rr;
+    if (steps) *steps = k + m;
+    if (done) {
+        *iters = it0 + take;
+        if (!first || rr <= tol2 * ref2 || it0 + take >= maxit) *done = 1;
+    }
+}
+
+// The images of a block before orthogonalisation: w_i
+struct BlkVecs {
+    const float2* w[SB];
+};
+
+// Grid (B, nrhs, groups of KM basis vectors), k = KM * groups: no guards in the loop, so that all
+// KM + 5 16-byte loads of an iteration are in flight before the first product (with a guard per
+// basis vector the loads went one by one: 687 us, now 248, for 12 basis vectors at 12^3 x 24 x 16).  Memory-bound at
+// fine sizes, at coarse sizes launch and tail.  The partial sums go to part as [block][quantity],
+// so that they are added up in contiguous runs.  done == nullptr: no convergence test (the smoother).
+template <int KM>
+__global__ void __launch_bounds__(RED_THREADS)
+k_blk_dots(float2* const* __restrict__ W, BlkVecs bv, const float2* __restrict__ res, long long n, int k, int m,
+           double* __restrict__ part, unsigned* counters, BGcr* g, const int* skip, int* steps, int* done,
+           const double* ref2, double tol2, int* iters, int maxit) {
+    constexpr int NQ = BLK_Q0 + 2 * SB * KM;
+    constexpr int NV = (NQ + 31) / 32 * 32;
+    const int r = blockIdx.y, j0 = blockIdx.z * KM;
+    if (skip && skip[r]) return;
+    __shared__ double sh[NV][RED_THREADS / 32 + 1];
+    const float4* Wp[KM + 1];
+#pragma unroll
+    for (int j = 0; j < KM; ++j) Wp[j] = reinterpret_cast<const float4*>(W[j0 + j] + r * n);
+    const float4* r4 = reinterpret_cast<const float4*>(res + r * n);
+    const float4* w4[SB];
+#pragma unroll
+    for (int i = 0; i < SB; ++i) w4[i] = i < m ? reinterpret_cast<const float4*>(bv.w[i] + r * n) : nullptr;
+    float v[NV];
+#pragma unroll
+    for (int q = 0; q < NV; ++q) v[q] = 0.f;
+    const bool gram = blockIdx.z == 0;
+    ROW_LOOP(x, n >> 1) {
+        float4 a[SB], b[KM + 1];
+#pragma unroll
+        for (int i = 0; i < SB; ++i) a[i] = i < m ? w4[i][x] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int j = 0; j < KM; ++j) b[j] = Wp[j][x];
+        if (gram) {
+            const float4 c = r4[x];
+#pragma unroll
+            for (int i = 0; i < SB; ++i) {
+                v[i] += a[i].x * a[i].x + a[i].y * a[i].y + a[i].z * a[i].z + a[i].w * a[i].w;
+                cdot4(a[i], c, v[16 + 2 * i], v[17 + 2 * i]);
+#pragma unroll
+                for (int l = 0; l < i; ++l) cdot4(a[l], a[i], v[4 + i * (i - 1) + 2 * l], v[5 + i * (i - 1) + 2 * l]);
+            }
+            v[24] += c.x * c.x + c.y * c.y + c.z * c.z + c.w * c.w;
+        }
+#pragma unroll
+        for (int j = 0; j < KM; ++j)
+#pragma unroll
+            for (int i = 0; i < SB; ++i)
+                cdot4(b[j], a[i], v[BLK_Q0 + 2 * (SB * j + i)], v[BLK_Q0 + 2 * (SB * j + i) + 1]);
+    }
+    // the tree over each warp in FP32, every sum across warps and blocks in FP64
+    warp_sums<NV>(v);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int q = 0; q < NV / 32; ++q) sh[lane * (NV / 32) + q][warp] = (double)v[q];
     __syncthreads();
+    const int nq = BLK_Q0 + 2 * SB * k;                          // quantities of the whole row
     const int B = gridDim.x;
-    double* pr = part + (size_t)r * BK_MAX * 2 * BMDOT_BLOCKS;       // [quantity][block]
-    for (int q = threadIdx.x; q < nq; q += blockDim.x) {
-        double s = 0.0;
-        for (int u = 0; u < RED_THREADS / 32; ++u) s += sh[q][u];
-        pr[(size_t)q * B + blockIdx.x] = s;
+    double* pr = part + (size_t)r * BK_MAX * 2 * BMDOT_BLOCKS;   // [block][quantity]
+    for (int q = threadIdx.x; q < NQ; q += blockDim.x) {
+        if (q < BLK_Q0 && !gram) continue;
+        double t = 0.0;
+#pragma unroll
+        for (int u = 0; u < RED_THREADS / 32; ++u) t += sh[q][u];
+        pr[(size_t)blockIdx.x * nq + (q < BLK_Q0 ? q : q + 2 * SB * j0)] = t;
         __threadfence();
     }
     __syncthreads();
-    if (!grid_last_block(counters + (size_t)r * BK_MAX * CROW)) return;
+    // Blocks meet twice: the last of each group of BLK_GROUP adds the group's partials up (in order), and the last
+    // group's last block adds the groups: one SM alone would spend 2 us and more on the FP64 sums of 128 blocks.
+    const unsigned ngroups = (B + BLK_GROUP - 1) / BLK_GROUP, grp = blockIdx.x / BLK_GROUP;
+    const int rows = min(BLK_GROUP, B - (int)grp * BLK_GROUP);
+    unsigned* cnt = counters + (size_t)r * BK_MAX * CROW;         // [ngroups] then the top one, 128 bytes apart
+    __shared__ bool last;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(cnt + grp * RED_CSTRIDE, 1u) == (unsigned)rows * gridDim.z - 1;
+    }
+    __syncthreads();
+    if (!last) return;
     __threadfence();
-    for (int q = warp; q < nq; q += RED_THREADS / 32) {
-        double s = 0.0;
-        for (int b = lane; b < B; b += 32) s += __ldcg(pr + (size_t)q * B + b);
+    constexpr int NT = BLK_Q0 + 2 * SB * BK_MAX;
+    __shared__ double tot[NT];
+    double* gr = pr + (size_t)grp * BLK_GROUP * nq;              // the group's sums replace its first row
+    for (int q = threadIdx.x; q < nq; q += blockDim.x) {
+        double t = 0.0;
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
-        if (lane == 0) tot[q] = s;
+        for (int u = 0; u < BLK_GROUP; ++u) t += u < rows ? __ldcg(gr + (size_t)u * nq + q) : 0.0;
+        if (ngroups == 1) tot[q] = t;
+        else gr[q] = t;
+        __threadfence();
     }
     __syncthreads();
-    if (threadIdx.x != 0) return;
-    BGcr& G = g[r];
-    double proj = 0.0;
-    for (int j = 0; j < k; ++j) {
-        const double nn = G.nrm[j], dr = tot[4 + 2 * j], di = tot[5 + 2 * j];
-        const double cr = nn > 0 ? dr / nn : 0.0, ci = nn > 0 ? di / nn : 0.0;
-        G.coef[j][0] = cr; G.coef[j][1] = ci;
-        G.C[k][j][0] = cr; G.C[k][j][1] = ci;
-        if (nn > 0) proj += (dr * dr + di * di) / nn;
+    if (ngroups > 1) {
+        if (threadIdx.x == 0) {
+            cnt[grp * RED_CSTRIDE] = 0u;
+            __threadfence();
+            last = atomicAdd(cnt + BLK_GROUPS_MAX * RED_CSTRIDE, 1u) == ngroups - 1;
+            if (last) cnt[BLK_GROUPS_MAX * RED_CSTRIDE] = 0u;
+        }
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        for (int q = threadIdx.x; q < nq; q += blockDim.x) {
+            double t = 0.0;
+#pragma unroll 8
+            for (unsigned u = 0; u < ngroups; ++u) t += __ldcg(pr + (size_t)u * BLK_GROUP * nq + q);
+            tot[q] = t;
+        }
+        __syncthreads();
+    } else if (threadIdx.x == 0) {
+        cnt[grp * RED_CSTRIDE] = 0u;
     }
-    const double wp = tot[0] - proj;
-    const bool ok = wp > BSTEP_BREAK * tot[0];
-    const double ar = ok ? tot[1] / wp : 0.0, ai = ok ? tot[2] / wp : 0.0;
-    const double rn = ok ? tot[3] - (tot[1] * tot[1] + tot[2] * tot[2]) / wp : tot[3];
-    G.nrm[k] = ok ? wp : 0.0;
-    G.alpha[0] = ar; G.alpha[1] = ai;
-    G.A[k][0] = ar; G.A[k][1] = ai;
-    G.rr2 = rn;
-    steps[r] = k + 1;
-    iters[r] += 1;
-    if (!ok || rn <= tol2 * ref2[r] || iters[r] >= maxit) done[r] = 1;
+    if (warp == 0)
+        blk_scalars(tot, k, m, g[r], steps ? steps + r : nullptr, done ? done + r : nullptr, ref2 ? ref2[r] : 0.0, tol2,
+                    iters ? iters + r : nullptr, maxit);
 }
 
-static void launch_bstep_dots(dim3 grid, float2* const* W, const float2* w, const float2* res, long long n, int k,
-                              double* part, unsigned* counters, BGcr* g, int* steps, int* done, const double* ref2,
-                              double tol2, int* iters, int maxit, cudaStream_t st) {
-#define DWF_BSTEP(KM) k_bstep_dots<KM><<<grid, RED_THREADS, 0, st>>>(W, w, res, n, k, part, counters, g, steps, done, \
-                                                                     ref2, tol2, iters, maxit)
-    if (k <= 4)       DWF_BSTEP(4);
-    else if (k <= 8)  DWF_BSTEP(8);
-    else if (k <= 16) DWF_BSTEP(16);
-    else              DWF_BSTEP(32);
-#undef DWF_BSTEP
+static void launch_blk_dots(float2* const* W, const BlkVecs& bv, const float2* res, long long n, int nrhs, int k, int m,
+                            double* part, unsigned* counters, BGcr* g, const int* skip, int* steps, int* done,
+                            const double* ref2, double tol2, int* iters, int maxit, cudaStream_t st) {
+    // about 4 float4 per thread, at most two blocks per SM (one where the sums leave registers for no more), and no
+    // more than the row's partial sums have room for
+    const int nq = BLK_Q0 + 2 * SB * k, km = k <= BLK_KM ? k : SB;
+    long long B = ((n >> 1) + 4 * RED_THREADS - 1) / (4 * RED_THREADS);
+    const long long cap = km <= 4 ? 304 : 152, room = (long long)BK_MAX * 2 * BMDOT_BLOCKS / nq;
+    if (B > cap) B = cap;
+    if (B > room) B = room;
+    if (B < 1) B = 1;
+    const dim3 grid((unsigned)B, (unsigned)nrhs, (unsigned)(km > 0 ? k / km : 1));
+#define DWF_BLK(KM) k_blk_dots<KM><<<grid, RED_THREADS, 0, st>>>(W, bv, res, n, k, m, part, counters, g, skip, steps, \
+                                                                 done, ref2, tol2, iters, maxit)
+    if (km == 0)      DWF_BLK(0);
+    else if (km == 4) DWF_BLK(4);
+    else if (km == 8) DWF_BLK(8);
+    else              DWF_BLK(12);
+#undef DWF_BLK
 }
 
-// The element-wise pass of the step: w' = w - sum_{j<k} coef_j W_j (stored in
-// place) and rout = rin - alpha w'.  Rows whose solve ended at this step skip.
-__global__ void __launch_bounds__(RED_THREADS) k_bstep_update(float2* __restrict__ w, float2* const* __restrict__ W,
-                                                              const BGcr* g, int k, const float2* __restrict__ rin,
-                                                              float2* __restrict__ rout, long long n,
-                                                              const int* skip) {
+// The element-wise pass of a block: w'_i into Wout[i] (STORE: a later block needs them) and
+// r' = r - sum_i alpha_i w'_i, or with rsub the difference rsub - r' (the image of the smoother's
+// whole correction), into rout.  w'_i may overwrite w_i.
+struct BlkOut {
+    float2* w[SB];
+};
+template <bool STORE>
+__global__ void __launch_bounds__(RED_THREADS)
+k_blk_update(float2* const* __restrict__ W, BlkVecs bv, BlkOut bo, const BGcr* g, int k, int m,
+             const float2* __restrict__ rin, const float2* __restrict__ rsub, float2* __restrict__ rout, long long n,
+             const int* skip) {
     const int r = blockIdx.y;
-    if (skip[r]) return;
-    __shared__ float2 c[BK_MAX];
+    if (skip && skip[r]) return;
+    __shared__ float2 c[SB][BK_MAX];                             // c_ij (j < k) and L_il (j = k + l)
+    __shared__ float2 al[SB];
     __shared__ const float4* Wp[BK_MAX];
-    for (int j = threadIdx.x; j < k; j += blockDim.x) {
-        c[j] = make_float2((float)g[r].coef[j][0], (float)g[r].coef[j][1]);
-        Wp[j] = reinterpret_cast<const float4*>(W[j] + r * n);
+    const BGcr& G = g[r];
+    for (int e = threadIdx.x; e < SB * (k + SB); e += blockDim.x) {
+        const int i = e % SB, j = e / SB;
+        if (i < m && j < k + i) c[i][j] = make_float2((float)G.C[k + i][j][0], (float)G.C[k + i][j][1]);
     }
+    if (threadIdx.x < m) al[threadIdx.x] = make_float2((float)G.A[k + threadIdx.x][0], (float)G.A[k + threadIdx.x][1]);
+    for (int j = threadIdx.x; j < k; j += blockDim.x) Wp[j] = reinterpret_cast<const float4*>(W[j] + r * n);
     __syncthreads();
-    const float2 al = make_float2((float)g[r].alpha[0], (float)g[r].alpha[1]);
-    float4* w4 = reinterpret_cast<float4*>(w + r * n);
-    const float4* a4 = reinterpret_cast<const float4*>(rin + r * n);
+    const float4* r4 = reinterpret_cast<const float4*>(rin + r * n);
+    const float4* s4 = rsub ? reinterpret_cast<const float4*>(rsub + r * n) : nullptr;
     float4* o4 = reinterpret_cast<float4*>(rout + r * n);
-    ROW_LOOP(i, n >> 1) {
-        float4 wi = w4[i];
-        const float4 ri0 = a4[i];
-        int j = 0;
-        for (; j + 3 < k; j += 4) {
-            const float4 b0 = Wp[j][i], b1 = Wp[j + 1][i], b2 = Wp[j + 2][i], b3 = Wp[j + 3][i];
-            csub4(wi, b0, c[j]); csub4(wi, b1, c[j + 1]); csub4(wi, b2, c[j + 2]); csub4(wi, b3, c[j + 3]);
+    const float4* w4[SB];
+    float4* q4[SB];
+#pragma unroll
+    for (int i = 0; i < SB; ++i) {
+        w4[i] = i < m ? reinterpret_cast<const float4*>(bv.w[i] + r * n) : nullptr;
+        q4[i] = STORE && i < m ? reinterpret_cast<float4*>(bo.w[i] + r * n) : nullptr;
+    }
+    ROW_LOOP(x, n >> 1) {
+        float4 a[SB];
+#pragma unroll
+        for (int i = 0; i < SB; ++i) a[i] = i < m ? w4[i][x] : make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 rr = r4[x];
+        float4 ss = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (s4) ss = s4[x];
+        for (int j = 0; j < k; j += 4) {                         // k is a multiple of SB = 4
+            const float4 b0 = Wp[j][x], b1 = Wp[j + 1][x], b2 = Wp[j + 2][x], b3 = Wp[j + 3][x];
+#pragma unroll
+            for (int i = 0; i < SB; ++i)
+                if (i < m) {
+                    csub4(a[i], b0, c[i][j]); csub4(a[i], b1, c[i][j + 1]);
+                    csub4(a[i], b2, c[i][j + 2]); csub4(a[i], b3, c[i][j + 3]);
+                }
         }
-        for (; j < k; ++j) csub4(wi, Wp[j][i], c[j]);
-        if (k > 0) w4[i] = wi;
-        float4 ri = ri0;
-        csub4(ri, wi, al);
-        o4[i] = ri;
+#pragma unroll
+        for (int i = 0; i < SB; ++i)
+            if (i < m) {
+#pragma unroll
+                for (int l = 0; l < i; ++l) csub4(a[i], a[l], c[i][k + l]);
+                if (STORE) q4[i][x] = a[i];
+                csub4(rr, a[i], al[i]);
+            }
+        if (s4) rr = make_float4(ss.x - rr.x, ss.y - rr.y, ss.z - rr.z, ss.w - rr.w);
+        o4[x] = rr;
     }
 }
 
-// y of the deferred solution update for the first m steps: (I + C)^T y = A,
-// y_j = A_j - sum_{k>j} C[k][j] y_k (one thread, FP64)
-__device__ __forceinline__ void back_substitute(const BGcr& g, int m, float2* y) {
-    double yr[BK_MAX], yi[BK_MAX];
-    for (int j = m - 1; j >= 0; --j) {
-        double a = g.A[j][0], b = g.A[j][1];
-        for (int k = j + 1; k < m; ++k) {
-            const double cr = g.C[k][j][0], ci = g.C[k][j][1];
-            a -= cr * yr[k] - ci * yi[k];
-            b -= cr * yi[k] + ci * yr[k];
-        }
-        yr[j] = a; yi[j] = b;
-        y[j] = make_float2((float)a, (float)b);
+// One block of GCR steps k .. k + m - 1: the raw images are in P[k + 1] .. P[k + m - 1] and
+// Q[k + m - 1], the residual in P[k]; Q[k] .. Q[k + m - 1] receive the orthogonal images (when
+// `store`) and rout the new residual (with rsub: rsub minus it).
+static dwf_status bblock(BGcr* g, float2* const* P, float2* const* Q, float2* const* dQ, int k, int m, bool store,
+                         const float2* rsub, float2* rout, long long n, int nrhs, double* part, unsigned* counters,
+                         const int* skip, int* steps, int* done, const double* ref2, double tol2, int* iters,
+                         int maxit, cudaStream_t st) {
+    BlkVecs bv{};
+    BlkOut bo{};
+    for (int i = 0; i < m; ++i) {
+        bv.w[i] = i + 1 < m ? P[k + i + 1] : Q[k + m - 1];
+        bo.w[i] = Q[k + i];
     }
+    launch_blk_dots(dQ, bv, P[k], n, nrhs, k, m, part, counters, g, skip, steps, done, ref2, tol2, iters, maxit, st);
+    const dim3 eg = row_grid(n >> 1, nrhs);
+    if (store) k_blk_update<true><<<eg, RED_THREADS, 0, st>>>(dQ, bv, bo, g, k, m, P[k], rsub, rout, n, skip);
+    else       k_blk_update<false><<<eg, RED_THREADS, 0, st>>>(dQ, bv, bo, g, k, m, P[k], rsub, rout, n, skip);
+    DWF_CHECK_LAUNCH();
+    return DWF_OK;
+}
+
+// y of the deferred solution update for the first m <= 32 steps: (I + C)^T y = A,
+// y_j = A_j - sum_{k>j} C[k][j] y_k, by one warp in FP64 (lane j holds y_j; one thread alone
+// took 7 us for 16 steps, at the start of every block of the combination)
+__device__ __forceinline__ void back_substitute(const BGcr& g, int m, float2* y) {
+    const int j = threadIdx.x;
+    if (j >= 32) return;
+    double a = 0.0, b = 0.0;
+    if (j < m) { a = g.A[j][0]; b = g.A[j][1]; }
+    for (int k = m - 1; k > 0; --k) {
+        const double yr = __shfl_sync(0xffffffffu, a, k), yi = __shfl_sync(0xffffffffu, b, k);
+        if (j < k) {
+            const double cr = g.C[k][j][0], ci = g.C[k][j][1];
+            a -= cr * yr - ci * yi;
+            b -= cr * yi + ci * yr;
+        }
+    }
+    if (j < m) y[j] = make_float2((float)a, (float)b);
 }
 
 // out += sum_{j<m} y_j P_j (FP32), m = nsteps[r] or m_fixed when nsteps is
@@ -546,7 +765,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_bcombine32(float2* __restrict__
     const int m = nsteps ? nsteps[r] : m_fixed;
     __shared__ float2 y[BK_MAX];
     __shared__ const float4* Pp[BK_MAX];
-    if (threadIdx.x == 0 && m > 0) back_substitute(g[r], m, y);
+    if (m > 0) back_substitute(g[r], m, y);
     for (int j = threadIdx.x; j < m; j += blockDim.x) Pp[j] = reinterpret_cast<const float4*>(P[j] + r * n);
     __syncthreads();
     float4* o4 = reinterpret_cast<float4*>(out + r * n);
@@ -556,7 +775,12 @@ __global__ void __launch_bounds__(RED_THREADS) k_bcombine32(float2* __restrict__
     ROW_LOOP(i, n >> 1) {
         if (m > 0) {
             float4 x = o4[i];
-            for (int j = 0; j < m; ++j) cadd4(x, Pp[j][i], y[j]);
+            int j = 0;
+            for (; j + 3 < m; j += 4) {
+                const float4 b0 = Pp[j][i], b1 = Pp[j + 1][i], b2 = Pp[j + 2][i], b3 = Pp[j + 3][i];
+                cadd4(x, b0, y[j]); cadd4(x, b1, y[j + 1]); cadd4(x, b2, y[j + 2]); cadd4(x, b3, y[j + 3]);
+            }
+            for (; j < m; ++j) cadd4(x, Pp[j][i], y[j]);
             o4[i] = x;
         }
         if (wout) {
@@ -575,7 +799,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_bcombine64(double2* __restrict_
     if (m <= 0) return;
     __shared__ float2 y[BK_MAX];
     __shared__ const float4* Zp[BK_MAX];
-    if (threadIdx.x == 0) back_substitute(g[r], m, y);
+    back_substitute(g[r], m, y);
     for (int j = threadIdx.x; j < m; j += blockDim.x) Zp[j] = reinterpret_cast<const float4*>(Z[j] + r * n);
     __syncthreads();
     const double sc = s[r];
@@ -597,7 +821,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_bcombine64_pk(double2* __restri
     if (m <= 0) return;
     __shared__ float2 y[BK_MAX];
     __shared__ const float4* Zp[BK_MAX];
-    if (threadIdx.x == 0) back_substitute(g[0], m, y);
+    back_substitute(g[0], m, y);
     for (int j = threadIdx.x; j < m; j += blockDim.x) Zp[j] = reinterpret_cast<const float4*>(Z[j]);
     __syncthreads();
     const double sc = s[0];
@@ -776,7 +1000,7 @@ struct BSolver {
     long long l3_solves = 0;     // and coarsest solves
 };
 
-static dim3 row_grid(long long n2, int nrhs, int cap = 1216) {
+static dim3 row_grid(long long n2, int nrhs, int cap) {
     long long b = (n2 + 255) / 256;
     if (b < 1) b = 1;
     if (b > cap) b = cap;
@@ -852,29 +1076,32 @@ static dwf_status bcoarse_cycle(BSolver& s) {
     DWF_CHECK_CUDA(cudaMemsetAsync(v.csteps, 0, s.nrhs * sizeof(int), s.st));
     k_bcopy<<<eg, 256, 0, s.st>>>(v.Zc[0], v.crr, n, v.cdone);
     DWF_CHECK_LAUNCH();
-    for (int k = 0; k < KC; ++k) {
-        if (s.nrhs == 1) {
-            // one column: the shared-memory tile stencil has the shorter latency
-            DWF_TRY(coarse_dwf_apply(h, v.Zc[k], v.ct, h->mf, false, v.cdone, s.st));
-            DWF_TRY(coarse_dwf_apply(h, v.ct, v.Wc[k], 1.0, true, v.cdone, s.st));
-        } else {
-            DWF_TRY(coarse_apply_multi_tc(h, s.nrhs, v.Zc[k], v.ct, h->mf, false, v.cdone, s.st));
-            DWF_TRY(coarse_apply_multi_tc(h, s.nrhs, v.ct, v.Wc[k], 1.0, true, v.cdone, s.st));
+    const bool blocks = h->prm.cgs_passes == 1;
+    for (int k = 0; k < KC;) {
+        const int m = !blocks ? 1 : KC - k < SB ? KC - k : SB;
+        for (int i = 0; i < m; ++i) {
+            float2* out = i + 1 < m ? v.Zc[k + i + 1] : v.Wc[k + m - 1];
+            if (s.nrhs == 1) {
+                // one column: the shared-memory tile stencil has the shorter latency
+                DWF_TRY(coarse_dwf_apply(h, v.Zc[k + i], v.ct, h->mf, false, v.cdone, s.st));
+                DWF_TRY(coarse_dwf_apply(h, v.ct, out, 1.0, true, v.cdone, s.st));
+            } else {
+                DWF_TRY(coarse_apply_multi_tc(h, s.nrhs, v.Zc[k + i], v.ct, h->mf, false, v.cdone, s.st));
+                DWF_TRY(coarse_apply_multi_tc(h, s.nrhs, v.ct, out, 1.0, true, v.cdone, s.st));
+            }
         }
-        float2* rnext = k + 1 < KC ? v.Zc[k + 1] : v.crr;
-        if (h->prm.cgs_passes == 1) {
-            // one reduction pass and one element-wise pass per step
-            const dim3 dg((unsigned)(rg.x < BSTEP_BLOCKS ? rg.x : BSTEP_BLOCKS), (unsigned)s.nrhs);
-            launch_bstep_dots(dg, v.dptr + 5 * BK_MAX, v.Wc[k], v.Zc[k], n, k, v.mpart, v.mcount, v.cgcr, v.csteps,
-                              v.cdone, v.cref2, tol2, v.citers, h->prm.coarse_maxiter, s.st);
-            k_bstep_update<<<eg, RED_THREADS, 0, s.st>>>(v.Wc[k], v.dptr + 5 * BK_MAX, v.cgcr, k, v.Zc[k], rnext, n,
-                                                         v.cdone);
+        float2* rnext = k + m < KC ? v.Zc[k + m] : v.crr;
+        if (blocks) {
+            DWF_TRY(bblock(v.cgcr, v.Zc, v.Wc, v.dptr + 5 * BK_MAX, k, m, k + m < KC, nullptr, rnext, n, s.nrhs, v.mpart,
+                           v.mcount, v.cdone, v.csteps, v.cdone, v.cref2, tol2, v.citers, h->prm.coarse_maxiter,
+                           s.st));
         } else {
             DWF_TRY(borthogonalise(s, v.cgcr, v.Wc, k, v.Zc[k], n, v.dptr + 5 * BK_MAX, v.csteps, v.cdone));
             k_bres_update<<<rg, RED_THREADS, 0, s.st>>>(v.Zc[k], rnext, v.Wc[k], v.cgcr, n, v.red, v.cdone, v.cdone,
                                                         v.cref2, tol2, v.citers, h->prm.coarse_maxiter);
         }
         DWF_CHECK_LAUNCH();
+        k += m;
     }
     k_bcombine32<<<eg, RED_THREADS, 0, s.st>>>(v.ec, v.dptr + 4 * BK_MAX, v.cgcr, v.csteps, 0, n, nullptr, nullptr,
                                                nullptr, nullptr);
@@ -946,8 +1173,8 @@ static dwf_status bcoarse_solve(BSolver& s, int* citers_out) {
     return DWF_OK;
 }
 
-// z = M(r) and w = A z for every right-hand side with idone == 0.  The
-// smoother's step j keeps its residual in Ps[j] and writes the next one to
+// z = M(r) and w = A z for every right-hand side with idone == 0.  With two
+// Gram-Schmidt passes the smoother's step j keeps its residual in Ps[j] and writes the next one to
 // Ps[j + 1] (rs_ after the last step); z += sum_j y_j Ps[j] and w = r - rs_
 // come out of one final pass.
 static dwf_status bprecondition(BSolver& s, const float2* res, float2* zout, float2* wout, int* citers_out) {
@@ -972,6 +1199,23 @@ static dwf_status bprecondition(BSolver& s, const float2* res, float2* zout, flo
     DWF_TRY(bapply_A(s, zout, v.ps, v.idone));
     k_bsub32<<<eg, 256, 0, s.st>>>(v.Ps[0], res, v.ps, n, v.idone);
     DWF_CHECK_LAUNCH();
+    if (h->prm.cgs_passes == 1) {
+        // blocks of steps; the last one leaves w = r - rs_ in place of the residual rs_
+        for (int j = 0; j < S;) {
+            const int m = S - j < SB ? S - j : SB;
+            for (int i = 0; i < m; ++i)
+                DWF_TRY(bapply_A(s, v.Ps[j + i], i + 1 < m ? v.Ps[j + i + 1] : v.Qs[j + m - 1], v.idone));
+            const bool last = j + m == S;
+            DWF_TRY(bblock(v.smooth, v.Ps, v.Qs, v.dptr + 3 * BK_MAX, j, m, !last, last ? res : nullptr,
+                           last ? wout : v.Ps[j + m], n, s.nrhs, v.mpart, v.mcount, v.idone, nullptr, nullptr, nullptr,
+                           0.0, nullptr, 0, s.st));
+            j += m;
+        }
+        k_bcombine32<<<eg, RED_THREADS, 0, s.st>>>(zout, v.dptr + 2 * BK_MAX, v.smooth, nullptr, S, n, nullptr, nullptr,
+                                                   nullptr, v.idone);
+        DWF_CHECK_LAUNCH();
+        return DWF_OK;
+    }
     const dim3 rg((unsigned)red_grid4(n), (unsigned)s.nrhs);
     for (int j = 0; j < S; ++j) {
         DWF_TRY(bapply_A(s, v.Ps[j], v.Qs[j], v.idone));
