@@ -313,37 +313,11 @@ __device__ __forceinline__ double tile_site(const TileSmemT<BT>& sm, float2* __r
 
 constexpr unsigned long long TILE_WAIT_NS = 2000000000ULL;   // 2 s
 
-template <class BT>
-__global__ void __launch_bounds__(TILE_THREADS) k_coarse_tile(const BT* __restrict__ B, const float2* __restrict__ in,
-                                                              float2* __restrict__ out, CoarseParams p, bool dag,
-                                                              const int* skip, int* status) {
-    if (skip && *skip) return;
-    extern __shared__ __align__(128) unsigned char tile_raw[];
-    TileSmemT<BT>& sm = *reinterpret_cast<TileSmemT<BT>*>(tile_raw);
-    const int ntx = (p.Lc[0] + TILE_X - 1) / TILE_X;
-    const int x0 = (blockIdx.x % ntx) * TILE_X, y0 = (blockIdx.x / ntx) * TILE_Y;
-    if (threadIdx.x == 0) mbar_init(&sm.mbar, 1);
-    __syncthreads();
-    tile_issue_blocks(sm, B, p, x0, y0);
-    tile_stage<false, BT>(sm, in, p, x0, y0);
-    __syncthreads();
-    if (!mbar_wait_bounded(&sm.mbar, 0, TILE_WAIT_NS)) {
-        if (threadIdx.x == 0) atomicExch(status, 2);
-        mbar_wait_bounded(&sm.mbar, 0, TILE_WAIT_NS);     // let the copies land before the block exits
-        return;
-    }
-    tile_site(sm, out, p, x0, y0, p.mf, dag);
-}
-
 static bool tile_ok(const CoarseParams& p) { return p.nd == 2 && p.ncd == 16 && p.Ls_c <= 4; }
 
 static dwf_status site_init_attributes();
 
 dwf_status coarse_init_attributes() {
-    DWF_CHECK_CUDA(cudaFuncSetAttribute(k_coarse_tile<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)sizeof(TileSmemT<float2>)));
-    DWF_CHECK_CUDA(cudaFuncSetAttribute(k_coarse_tile<__half2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)sizeof(TileSmemT<__half2>)));
     return site_init_attributes();
 }
 
@@ -355,6 +329,128 @@ __global__ void __launch_bounds__(256) k_coarse_dwf(const float2* __restrict__ B
     if (xc >= p.Vc) return;
     if (NCD == 16 && p.Ls_c <= 4) warp_site16<false>(B, in, out, p, xc, p.mf, dag, threadIdx.x & 31);
     else warp_site_apply<NCD, false>(B, in, out, p, xc, p.mf, dag, threadIdx.x & 31);
+}
+
+// ---------------------------------------------------------------------------
+// One vector, 2-d, 16 coarse dof, Ls_c <= 4: one warp per coarse site, everything straight from
+// global memory.  Lane 4 g + q holds the columns 2 g, 2 g + 1 and the rows 4 q .. 4 q + 3 of a
+// block, so a block arrives as two 16-byte loads per lane (FP16 storage) and its inputs as one
+// per slice (broadcast over q), nothing is staged or waited for, and every FP32 multiply-add of the block is done
+// once: 640 per lane and site.  The 4 rows x 4 slices of partial sums then fold over the 8
+// lanes g in three exchanges that each halve what a lane carries, which leaves slice lane / 8 and
+// two adjacent rows in a lane: one 16-byte store.  The adjoint uses sigma_3 (Dhat_W^dag =
+// sigma_3 Dhat_W sigma_3): the sign of the chirality - columns goes onto a lane's sums.
+// Bound by FP32 issue and the L2 round trips of five directions (the 21 MB of blocks of a
+// 64^2 lattice stay in L2).  Staging blocks and inputs in shared memory (8 sites per thread block,
+// bulk copies, every block element converted twice) took 12.5 us at 64^2 x 4; 256^2 x 16
+// gradient step 630 -> 522 ms.
+// ---------------------------------------------------------------------------
+constexpr int W16_WARPS = 4;
+
+// rows 4 q .. 4 q + 3 of one block column
+__device__ __forceinline__ void ld_rows4(const __half2* p, float2 (&y)[4]) {
+    const uint4 u = __ldg(reinterpret_cast<const uint4*>(p));
+    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+    for (int r = 0; r < 4; ++r) y[r] = __half22float2(*reinterpret_cast<const __half2*>(&w[r]));
+}
+__device__ __forceinline__ void ld_rows4(const float2* p, float2 (&y)[4]) {
+    const float4 a = __ldg(reinterpret_cast<const float4*>(p)), b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+    y[0] = make_float2(a.x, a.y); y[1] = make_float2(a.z, a.w);
+    y[2] = make_float2(b.x, b.y); y[3] = make_float2(b.z, b.w);
+}
+// two adjacent complex values; V4: 16-byte aligned
+template <bool V4>
+__device__ __forceinline__ float4 ld_pair(const float2* p) {
+    if (V4) return __ldg(reinterpret_cast<const float4*>(p));
+    const float2 a = __ldg(p), b = __ldg(p + 1);
+    return make_float4(a.x, a.y, b.x, b.y);
+}
+
+template <class BT, bool V4>
+__global__ void __launch_bounds__(W16_WARPS * 32, 5)
+k_coarse_w16(const BT* __restrict__ B, const float2* __restrict__ in, float2* __restrict__ out, CoarseParams p,
+             bool dag, const int* skip) {
+    if (skip && *skip) return;
+    const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+    const int xc = blockIdx.x * W16_WARPS + (threadIdx.x >> 5);
+    if (xc >= p.Vc) return;                              // whole warps; no block-wide barrier below
+    const int L0 = p.Lc[0], L1 = p.Lc[1], y0 = xc / L0, x0 = xc - y0 * L0;
+    const int nb[5] = {xc, x0 + 1 == L0 ? xc - x0 : xc + 1, x0 == 0 ? xc + L0 - 1 : xc - 1,
+                       y0 + 1 == L1 ? x0 : xc + L0, y0 == 0 ? xc + (L1 - 1) * L0 : xc - L0};
+    const long long slice = p.Vc * 16;
+    const BT* Bl = B + (long long)xc * (5 * 256) + 2 * g * 16 + 4 * q;
+    float2 acc[4][4];                                    // [slice][row]
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) acc[s][r] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int dir = 0; dir < 5; ++dir) {
+        const float2* v = in + (long long)nb[dir] * 16 + 2 * g;
+        float4 a[4];
+#pragma unroll
+        for (int s = 0; s < 4; ++s) a[s] = s < p.Ls_c ? ld_pair<V4>(v + s * slice) : make_float4(0.f, 0.f, 0.f, 0.f);
+        float2 ya[4], yb[4];
+        ld_rows4(Bl + dir * 256, ya);
+        ld_rows4(Bl + dir * 256 + 16, yb);
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                acc[s][r] = cfma(ya[r], make_float2(a[s].x, a[s].y), acc[s][r]);
+                acc[s][r] = cfma(yb[r], make_float2(a[s].z, a[s].w), acc[s][r]);
+            }
+    }
+    // fold over g: bit 4 of the lane keeps slices 0, 1 or 2, 3, bit 3 one of the two, bit 2 rows 0, 1 or 2, 3
+    const float sg = dag && g >= 4 ? -1.f : 1.f;
+    const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
+    float2 h2[2][4], h1[4], h0[2];
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const float2 keep = b4 ? acc[s + 2][r] : acc[s][r], send = b4 ? acc[s][r] : acc[s + 2][r];
+            // the partner's columns have the other chirality: each side signs its own sums
+            h2[s][r].x = sg * keep.x + __shfl_xor_sync(0xffffffffu, sg * send.x, 16);
+            h2[s][r].y = sg * keep.y + __shfl_xor_sync(0xffffffffu, sg * send.y, 16);
+        }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const float2 keep = b3 ? h2[1][r] : h2[0][r], send = b3 ? h2[0][r] : h2[1][r];
+        h1[r].x = keep.x + __shfl_xor_sync(0xffffffffu, send.x, 8);
+        h1[r].y = keep.y + __shfl_xor_sync(0xffffffffu, send.y, 8);
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const float2 keep = b2 ? h1[r + 2] : h1[r], send = b2 ? h1[r] : h1[r + 2];
+        h0[r].x = keep.x + __shfl_xor_sync(0xffffffffu, send.x, 4);
+        h0[r].y = keep.y + __shfl_xor_sync(0xffffffffu, send.y, 4);
+    }
+    const int s = lane >> 3, row = 4 * q + (b2 ? 2 : 0);
+    if (s >= p.Ls_c) return;
+    const int c = row / p.nvec;                          // nvec = 8: both rows have one chirality
+    const float si = dag && c == 1 ? -1.f : 1.f;
+    const bool from_below = dag ? (c == 1) : (c == 0);
+    const int sh = from_below ? (s > 0 ? s - 1 : p.Ls_c - 1) : (s < p.Ls_c - 1 ? s + 1 : 0);
+    const float sc = from_below ? (s > 0 ? 1.f : -p.mf) : (s < p.Ls_c - 1 ? 1.f : -p.mf);
+    const float2* me = in + (long long)xc * 16 + row;
+    const float4 self = ld_pair<V4>(me + s * slice), hv = ld_pair<V4>(me + sh * slice);
+    const float4 o = make_float4(si * h0[0].x + self.x + sc * hv.x, si * h0[0].y + self.y + sc * hv.y,
+                                 si * h0[1].x + self.z + sc * hv.z, si * h0[1].y + self.w + sc * hv.w);
+    float2* op = out + s * slice + (long long)xc * 16 + row;
+    if (V4) *reinterpret_cast<float4*>(op) = o;
+    else { op[0] = make_float2(o.x, o.y); op[1] = make_float2(o.z, o.w); }
+}
+
+template <class BT>
+static void launch_w16(const void* B, const float2* in, float2* out, const CoarseParams& p, bool dag, const int* skip,
+                       cudaStream_t st) {
+    const unsigned grid = (unsigned)((p.Vc + W16_WARPS - 1) / W16_WARPS);
+    if (aligned16(in) && aligned16(out))
+        k_coarse_w16<BT, true><<<grid, W16_WARPS * 32, 0, st>>>((const BT*)B, in, out, p, dag, skip);
+    else
+        k_coarse_w16<BT, false><<<grid, W16_WARPS * 32, 0, st>>>((const BT*)B, in, out, p, dag, skip);
 }
 
 // ---------------------------------------------------------------------------
@@ -597,13 +693,8 @@ dwf_status coarse_dwf_apply(const dwf_mg* h, const float2* in, float2* out, doub
     const unsigned grid = (unsigned)((p.Vc * 32 + thr - 1) / thr);
     const float2* B = dagger ? h->Yd32 : h->Y32;
     if (tile_ok(p)) {
-        const int ntiles = ((p.Lc[0] + TILE_X - 1) / TILE_X) * ((p.Lc[1] + TILE_Y - 1) / TILE_Y);
-        if (h->ytile_half)
-            k_coarse_tile<__half2><<<ntiles, TILE_THREADS, sizeof(TileSmemT<__half2>), st>>>(
-                (const __half2*)h->Ytile, in, out, p, dagger, skip, h->status + 1);
-        else
-            k_coarse_tile<float2><<<ntiles, TILE_THREADS, sizeof(TileSmemT<float2>), st>>>(
-                (const float2*)h->Ytile, in, out, p, dagger, skip, h->status + 1);
+        if (h->ytile_half) launch_w16<__half2>(h->Ytile, in, out, p, dagger, skip, st);
+        else               launch_w16<float2>(h->Ytile, in, out, p, dagger, skip, st);
     } else if (h->Ymma && p.ncd == 48 && p.ndir == 9 && p.Ls_c <= 4) {
         const unsigned grid1 = (unsigned)((p.Vc + CM_WARPS - 1) / CM_WARPS);
         k_coarse_mma<<<grid1, CM_WARPS * 32, 0, st>>>((const uint4*)h->Ymma, in, out, p, dagger, skip);
