@@ -10,7 +10,6 @@
 
 #include "mg.cuh"
 #include "async_copy.cuh"
-#include "mma_tf32.cuh"
 
 namespace dwf {
 
@@ -317,7 +316,10 @@ static bool tile_ok(const CoarseParams& p) { return p.nd == 2 && p.ncd == 16 && 
 
 static dwf_status site_init_attributes();
 
+static dwf_status mma_init_attributes();
+
 dwf_status coarse_init_attributes() {
+    DWF_TRY(mma_init_attributes());
     return site_init_attributes();
 }
 
@@ -562,99 +564,228 @@ __global__ void __launch_bounds__(512) k_coarse_site(const BT* __restrict__ B, c
 // ---------------------------------------------------------------------------
 // Tensor-core form of the 48-dof stencil (4-d, FP16 blocks, Ls_c <= 4).  One
 // warp per coarse site.  Per direction the complex product Y v over the Ls_c
-// slices is the real product of A = [Re Y; Im Y] (96 x 48, FP16, exact in
-// TF32) with B = [Re v | Im v] (48 x 2 Ls_c): C = A B holds Re Y Re v, Re Y Im v
-// (rows < 48) and Im Y Re v, Im Y Im v (rows >= 48), so
-// Re(Y v) = C[i][Re] - C[48 + i][Im] and Im(Y v) = C[48 + i][Re] + C[i][Im].
-// B column n = 4 part + s; the FP32 inputs are split into TF32 high and low
-// parts multiplied separately (FP32-level accuracy).  A streams from HBM in
-// fragment order (one coalesced 16-byte load per lane per row tile and column
-// tile pair, no shared-memory staging), so many warps per SM keep enough bytes
-// in flight; the products accumulate over the 9 directions in registers.
+// slices is the real product of A = [Re Y; Im Y] (96 x 48, FP16 as stored)
+// with B (48 x 8), column 2 s the real and 2 s + 1 the imaginary part of
+// slice s: C = A B holds Re Y Re v, Re Y Im v (rows < 48) and Im Y Re v, Im Y Im v
+// (rows >= 48) of one slice in one lane, so
+// Re(Y v) = C[i][Re] - C[48 + i][Im] and Im(Y v) = C[48 + i][Re] + C[i][Im]
+// are sums of its own accumulators.
+//
+// Inputs: a slice's 48 values are scaled by a power of two to below 2^14 and
+// split into two FP16 parts of 11 bits each (22 bits, what a TF32 high / low
+// pair keeps too), so that mma.m16n8k16 takes the blocks as they are stored:
+// half the products of the TF32 form and no conversion of a block.  The
+// products of one direction accumulate in FP32; directions are added up in
+// FP32 with the scale taken back.
+//
+// Only the self block and the four forward blocks of a site are stored: the
+// kernel is gamma_5-hermitian, so the backward block of x is
+// sigma_3 Y_+mu(x - mu)^dag sigma_3 of its neighbour's forward block, which that
+// neighbour's warp reads too: once from HBM, then from L2 (the farthest
+// neighbour, one coarse t-slice away, is 23 MB of blocks behind at 8^3 x 16).
+// A block lies in memory as 8 x 8 tiles, and ldmatrix reads it from shared
+// memory as it is or transposed; sigma_3 and the conjugate are signs of the
+// inputs and of the sums.
+//
+// Each warp brings the block of direction d + 1 into the other half of its
+// shared-memory ring by one bulk copy while it multiplies that of direction
+// d: 9.2 KB per warp, 12 warps per SM.  Bound by the block bytes (L2 to SM:
+// 83 KB per site; HBM: 46 KB): 33 us at 6^3 x 12 sites x 4 slices and 81 us at 8^3 x 16
+// (8.4 TB/s of block bytes), where nine stored blocks and TF32 products took 44 and 114 us.
 // ---------------------------------------------------------------------------
 constexpr int CM_WARPS = 4;
-__device__ __forceinline__ uint32_t f16_bits_to_f32(uint32_t w, int hi) {
-    return __float_as_uint(__half2float(__ushort_as_half((unsigned short)(hi ? (w >> 16) : (w & 0xffffu)))));
+constexpr int CM_BLOCKS = 5;                             // stored blocks per site: self, +mu
+constexpr unsigned CM_BLOCK_BYTES = 96 * 48 * sizeof(__half);
+struct CmSmem {
+    unsigned char ring[2][CM_BLOCK_BYTES];               // [row tile 12][column tile 6][8][8] halves
+    unsigned long long bar[2];
+    unsigned long long pad[14];                          // the next warp's ring on a 128-byte line
+};
+
+// four 8 x 8 tiles of halves: lane l gives the address of row l % 8 of tile l / 8
+template <bool TRANS>
+__device__ __forceinline__ void ldmatrix4(uint32_t (&a)[4], uint32_t addr) {
+    if (TRANS)
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]) : "r"(addr) : "memory");
+    else
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void mma_f16(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+                 "{%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-__global__ void __launch_bounds__(CM_WARPS * 32, 3) k_coarse_mma(const uint4* __restrict__ Ym,
+// This lane's inputs of one direction: column g = 2 s + part, dof 8 j + 2 t and 8 j + 2 t + 1 (j < 6)
+template <bool V4>
+__device__ __forceinline__ void cm_load(float (&v)[6][2], const float2* vin, bool colv, int part) {
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+        const float4 u = colv ? ld_pair<V4>(vin + 8 * j) : make_float4(0.f, 0.f, 0.f, 0.f);
+        v[j][0] = part ? u.y : u.x;
+        v[j][1] = part ? u.w : u.z;
+    }
+}
+// B fragments: hi[kt][h] and lo[kt][h] hold dof 16 kt + 8 h + 2 t, + 1; chirality - dof change sign with
+// `neg`.  Returns what undoes the scale of this lane's slice.
+__device__ __forceinline__ float cm_split(uint32_t (&hi)[3][2], uint32_t (&lo)[3][2], const float (&v)[6][2], bool neg) {
+    float m = 0.f;
+#pragma unroll
+    for (int j = 0; j < 6; ++j) m = fmaxf(m, fmaxf(fabsf(v[j][0]), fabsf(v[j][1])));
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));    // the slice's values: lanes t, and part
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 4));
+    // 2^(13 - exponent of m): |v| scaled < 2^14; tiny slices are left where 2^113 brings them
+    const int e = max((int)(__float_as_uint(m) >> 23), 27);
+    const float scale = __uint_as_float((unsigned)(127 + 13 + 127 - e) << 23);
+    const float back = __uint_as_float((unsigned)(e - 13) << 23);
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+        const float sc = neg && j >= 3 ? -scale : scale;
+        const float a = v[j][0] * sc, b = v[j][1] * sc;
+        const __half2 h = __floats2half2_rn(a, b);
+        const float2 f = __half22float2(h);
+        const __half2 l = __floats2half2_rn(a - f.x, b - f.y);
+        hi[j >> 1][j & 1] = *reinterpret_cast<const uint32_t*>(&h);
+        lo[j >> 1][j & 1] = *reinterpret_cast<const uint32_t*>(&l);
+    }
+    return back;
+}
+
+template <bool V4>
+__global__ void __launch_bounds__(CM_WARPS * 32, 3) k_coarse_mma(const unsigned char* __restrict__ Ym,
                                                                  const float2* __restrict__ in,
                                                                  float2* __restrict__ out, CoarseParams p, bool dag,
-                                                                 const int* skip) {
+                                                                 const int* skip, int* status) {
     if (skip && *skip) return;
-    __shared__ float Ps[CM_WARPS][96][9];
+    extern __shared__ __align__(128) unsigned char cm_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    CmSmem& sm = reinterpret_cast<CmSmem*>(cm_raw)[warp];
     const int xc = blockIdx.x * CM_WARPS + warp;
     if (xc >= p.Vc) return;                              // whole warps; no block-wide barrier below
     const int Ls_c = p.Ls_c;
     const long long slice = p.Vc * 48;
-    const int part = g >> 2, sB = g & 3;                 // B column n = g
+    const int part = g & 1, sB = g >> 1;                 // B column g
     const bool colv = sB < Ls_c;
-    float acc[6][2][4];
-#pragma unroll
-    for (int mt = 0; mt < 6; ++mt)
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) acc[mt][h][q] = 0.f;
-    const uint4* A = Ym + (long long)xc * (9 * 3 * 6 * 32) + lane;
-#pragma unroll 1
-    for (int dir = 0; dir < 9; ++dir) {
-        // L2 prefetch of the next direction's 18 fragment rows (one lane per 128-byte line)
-        if (dir + 1 < 9 && (lane & 7) == 0) {
-#pragma unroll
-            for (int q = 0; q < 18; ++q) asm volatile("prefetch.global.L2 [%0];" ::"l"(A + ((dir + 1) * 18 + q) * 32));
-        }
-        const int nb = coarse_nb32(p, xc, dir);
-        const float* vin = reinterpret_cast<const float*>(in + (colv ? sB : 0) * slice + (long long)nb * 48) + part;
-#pragma unroll
-        for (int kp = 0; kp < 3; ++kp) {
-            uint4 a[6];
-#pragma unroll
-            for (int mt = 0; mt < 6; ++mt) a[mt] = __ldg(A + ((dir * 3 + kp) * 6 + mt) * 32);
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int kt = 2 * kp + h;                 // input dof 8 kt .. 8 kt + 7
-                float b0 = colv ? __ldg(vin + 2 * (8 * kt + t)) : 0.f;
-                float b1 = colv ? __ldg(vin + 2 * (8 * kt + t + 4)) : 0.f;
-                if (dag && kt >= 3) { b0 = -b0; b1 = -b1; }   // sigma_3 on the chirality - inputs
-                uint32_t bh[2], bl[2];
-                split_tf32(b0, bh[0], bl[0]);
-                split_tf32(b1, bh[1], bl[1]);
-#pragma unroll
-                for (int mt = 0; mt < 6; ++mt) {
-                    const uint32_t w0 = h ? a[mt].z : a[mt].x, w1 = h ? a[mt].w : a[mt].y;
-                    const uint32_t af[4] = {f16_bits_to_f32(w0, 0), f16_bits_to_f32(w0, 1), f16_bits_to_f32(w1, 0),
-                                            f16_bits_to_f32(w1, 1)};
-                    mma_tf32(acc[mt][0], af, bh);
-                    mma_tf32(acc[mt][1], af, bl);
-                }
-            }
-        }
-    }
-    // C fragment: c0 (g, 2t), c1 (g, 2t + 1), c2 (g + 8, 2t), c3 (g + 8, 2t + 1)
-#pragma unroll
-    for (int mt = 0; mt < 6; ++mt)
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            Ps[warp][mt * 16 + g + ((q & 2) ? 8 : 0)][2 * t + (q & 1)] = acc[mt][0][q] + acc[mt][1][q];
+    const float2* vb = in + (colv ? sB : 0) * slice + 2 * t;
+    // steps: the self block, the four forward hops, the four backward hops (the neighbour's forward block)
+    constexpr int STEPS = 2 * CM_BLOCKS - 1;
+    // (lane d finds the neighbour of step d: its index divisions are done once per site)
+    const int mine = coarse_nb32(p, xc, lane == 0 || lane >= STEPS ? 0 : lane < CM_BLOCKS ? 2 * lane - 1 : 2 * (lane - CM_BLOCKS) + 2);
+    auto neighbour = [&](int d) { return __shfl_sync(0xffffffffu, mine, d); };
+    auto issue = [&](int d, int nb) {
+        if (lane != 0) return;
+        const long long blk = d < CM_BLOCKS ? (long long)xc * CM_BLOCKS + d : (long long)nb * CM_BLOCKS + d - CM_BLOCKS + 1;
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        mbar_expect_tx(&sm.bar[d & 1], CM_BLOCK_BYTES);
+        bulk_g2s(sm.ring[d & 1], Ym + blk * CM_BLOCK_BYTES, CM_BLOCK_BYTES, &sm.bar[d & 1]);
+    };
+    if (lane == 0) { mbar_init(&sm.bar[0], 1); mbar_init(&sm.bar[1], 1); }
     __syncwarp();
-    const int nvec = p.nvec;
-    for (int idx = lane; idx < 48 * Ls_c; idx += 32) {
-        const int s = idx / 48, r = idx % 48;
-        const float re = Ps[warp][r][s] - Ps[warp][48 + r][4 + s];
-        const float im = Ps[warp][48 + r][s] + Ps[warp][r][4 + s];
-        const float si = (dag && r >= nvec) ? -1.f : 1.f;  // sigma_3 on the output
-        const float2 self = __ldg(in + s * slice + (long long)xc * 48 + r);
-        const int c = r / nvec;
-        const bool from_below = dag ? (c == 1) : (c == 0);
-        int sh;
-        float sc = 1.f;
-        if (from_below) { if (s > 0) sh = s - 1; else { sh = Ls_c - 1; sc = -p.mf; } }
-        else            { if (s < Ls_c - 1) sh = s + 1; else { sh = 0; sc = -p.mf; } }
-        const float2 hv = __ldg(in + sh * slice + (long long)xc * 48 + r);
-        out[s * slice + (long long)xc * 48 + r] = make_float2(si * re + self.x + sc * hv.x, si * im + self.y + sc * hv.y);
+    issue(0, xc);
+    issue(1, xc);
+    float acc[3][4];                                     // rows 16 m + g (re, im), 16 m + g + 8 (re, im) of slice t
+#pragma unroll
+    for (int m = 0; m < 3; ++m)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[m][q] = 0.f;
+    const int r8 = lane & 7, i8 = (lane >> 3) & 1, i16 = lane >> 4;
+    float v[6][2];
+    cm_load<V4>(v, vb + (long long)xc * 48, colv, part);
+#pragma unroll 1
+    for (int d = 0; d < STEPS; ++d) {
+        const bool fwd = d < CM_BLOCKS;
+        uint32_t hi[3][2], lo[3][2];
+        // sigma_3 on the inputs: of the adjoint operator, and of a backward block
+        float back = cm_split(hi, lo, v, dag != !fwd);
+        back = __shfl_sync(0xffffffffu, back, 8 * t);    // the scale of slice t, this lane's columns of C
+        if (d + 1 < STEPS) cm_load<V4>(v, vb + (long long)neighbour(d + 1) * 48, colv, part);
+        if (!__all_sync(0xffffffffu, mbar_wait_bounded(&sm.bar[d & 1], (d >> 1) & 1, TILE_WAIT_NS))) {
+            if (lane == 0) atomicExch(status, 2);
+            // let the copies land before the warp exits
+            mbar_wait_bounded(&sm.bar[d & 1], (d >> 1) & 1, TILE_WAIT_NS);
+            if (d + 1 < STEPS) mbar_wait_bounded(&sm.bar[(d + 1) & 1], ((d + 1) >> 1) & 1, TILE_WAIT_NS);
+            return;
+        }
+        const uint32_t ring = smem_u32(sm.ring[d & 1]);
+        float C[6][4];
+#pragma unroll
+        for (int m = 0; m < 6; ++m)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) C[m][q] = 0.f;
+        if (fwd) {
+            // tiles (row 2 m, 2 m + 1) x (column 2 kt, 2 kt + 1)
+            const uint32_t base = ring + (i8 * 6 + i16) * 128 + r8 * 16;
+#pragma unroll
+            for (int kt = 0; kt < 3; ++kt) {
+                uint32_t a[6][4];
+#pragma unroll
+                for (int m = 0; m < 6; ++m) ldmatrix4<false>(a[m], base + (12 * m + 2 * kt) * 128);
+#pragma unroll
+                for (int m = 0; m < 6; ++m) mma_f16(C[m], a[m], hi[kt]);
+#pragma unroll
+                for (int m = 0; m < 6; ++m) mma_f16(C[m], a[m], lo[kt]);
+            }
+#pragma unroll
+            for (int m = 0; m < 3; ++m)
+#pragma unroll
+                for (int q = 0; q < 4; q += 2) {
+                    acc[m][q] = fmaf(back, C[m][q] - C[m + 3][q + 1], acc[m][q]);
+                    acc[m][q + 1] = fmaf(back, C[m][q + 1] + C[m + 3][q], acc[m][q + 1]);
+                }
+        } else {
+            // outputs 16 m .. are columns (tiles 2 m, 2 m + 1), inputs 16 kt .. rows (tiles 2 kt, 2 kt + 1) of Re Y and Im Y
+            const uint32_t base = ring + (i16 * 6 + i8) * 128 + r8 * 16;
+#pragma unroll
+            for (int kt = 0; kt < 3; ++kt) {
+                uint32_t a[6][4];
+#pragma unroll
+                for (int m = 0; m < 6; ++m) ldmatrix4<true>(a[m], base + (12 * (kt + (m < 3 ? 0 : 3)) + 2 * (m % 3)) * 128);
+#pragma unroll
+                for (int m = 0; m < 6; ++m) mma_f16(C[m], a[m], hi[kt]);
+#pragma unroll
+                for (int m = 0; m < 6; ++m) mma_f16(C[m], a[m], lo[kt]);
+            }
+#pragma unroll
+            for (int m = 0; m < 3; ++m)
+#pragma unroll
+                for (int q = 0; q < 4; q += 2) {
+                    // conj(Y): Re + Im parts; sigma_3 on outputs 8 (2 m + q / 2) and up
+                    const float sb = 2 * m + q / 2 >= 3 ? -back : back;
+                    acc[m][q] = fmaf(sb, C[m][q] + C[m + 3][q + 1], acc[m][q]);
+                    acc[m][q + 1] = fmaf(sb, C[m][q + 1] - C[m + 3][q], acc[m][q + 1]);
+                }
+        }
+        __syncwarp();                                    // every lane has read this half of the ring
+        if (d + 2 < STEPS) issue(d + 2, neighbour(d + 2));
     }
+    const int s = t;
+    if (s >= Ls_c) return;
+#pragma unroll
+    for (int m = 0; m < 3; ++m)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int r = 16 * m + 8 * h + g;
+            const int c = r >= 24;
+            const float si = dag && c ? -1.f : 1.f;      // sigma_3 on the output
+            const bool from_below = dag ? (c == 1) : (c == 0);
+            const int sh = from_below ? (s > 0 ? s - 1 : Ls_c - 1) : (s < Ls_c - 1 ? s + 1 : 0);
+            const float sc = from_below ? (s > 0 ? 1.f : -p.mf) : (s < Ls_c - 1 ? 1.f : -p.mf);
+            const float2* me = in + (long long)xc * 48 + r;
+            const float2 self = __ldg(me + s * slice), hv = __ldg(me + sh * slice);
+            out[s * slice + (long long)xc * 48 + r] = make_float2(si * acc[m][2 * h] + self.x + sc * hv.x,
+                                                                  si * acc[m][2 * h + 1] + self.y + sc * hv.y);
+        }
+}
+
+static dwf_status mma_init_attributes() {
+    const int sh = (int)(CM_WARPS * sizeof(CmSmem));
+    DWF_CHECK_CUDA(cudaFuncSetAttribute(k_coarse_mma<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sh));
+    DWF_CHECK_CUDA(cudaFuncSetAttribute(k_coarse_mma<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sh));
+    return DWF_OK;
 }
 
 constexpr size_t SITE_SMEM_MAX = 200 * 1024;
@@ -697,7 +828,11 @@ dwf_status coarse_dwf_apply(const dwf_mg* h, const float2* in, float2* out, doub
         else               launch_w16<float2>(h->Ytile, in, out, p, dagger, skip, st);
     } else if (h->Ymma && p.ncd == 48 && p.ndir == 9 && p.Ls_c <= 4) {
         const unsigned grid1 = (unsigned)((p.Vc + CM_WARPS - 1) / CM_WARPS);
-        k_coarse_mma<<<grid1, CM_WARPS * 32, 0, st>>>((const uint4*)h->Ymma, in, out, p, dagger, skip);
+        constexpr size_t sh = CM_WARPS * sizeof(CmSmem);
+        if (aligned16(in))
+            k_coarse_mma<true><<<grid1, CM_WARPS * 32, sh, st>>>((const unsigned char*)h->Ymma, in, out, p, dagger, skip, h->status + 1);
+        else
+            k_coarse_mma<false><<<grid1, CM_WARPS * 32, sh, st>>>((const unsigned char*)h->Ymma, in, out, p, dagger, skip, h->status + 1);
     } else if (site_ok(p, h->ytile_half)) {
         const int threads = p.ncd * p.Ls_c;
         if (h->ytile_half)

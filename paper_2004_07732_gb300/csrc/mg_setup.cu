@@ -275,7 +275,7 @@ __device__ __forceinline__ float2 gamma4(int mu, int a, int b) {
 constexpr int GAL4_THREADS = 256;
 constexpr int GAL4_MAXE = 16;           // Y entries per thread: ncd^2 <= 16 * 256 (ncd <= 64)
 
-// One block per (coarse site, direction): Y_dir = sum_x P(x)^dag Q(x) with
+// One block per (coarse site, self or forward direction): Y_dir = sum_x P(x)^dag Q(x) with
 // Q(x) = sum over the hops from x that land in the aggregate of xc + dir (and
 // the diagonal for dir 0) of D_W(x, y) P(y).  P(x) is 12 x ncd, block diagonal
 // in chirality (rows of spins 2c, 2c+1 feed columns c*nvec ...).
@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(GAL4_THREADS) k_galerkin_4d(const double2* __r
     float2* Q = Px + 12 * nvec;         // [12][ncd]
     __shared__ float Ul[9][2];
     const long long xc = blockIdx.x;
-    const int dir = blockIdx.y;
+    const int dir = blockIdx.y == 0 ? 0 : 2 * (int)blockIdx.y - 1;   // self and forward hops (k_backward_blocks: the rest)
     const int nb = ai.b[0] * ai.b[1] * ai.b[2] * ai.b[3];
     const int nent = ncd * ncd;
     float2 acc[GAL4_MAXE];
@@ -427,26 +427,41 @@ __global__ void k_blocks_to_f16(const double2* __restrict__ Y, __half2* __restri
     }
 }
 
-// Blocks of the 48-dof coarse operator in the fragment order of k_coarse_mma:
-// the real form A = [Re Y; Im Y] (96 x 48) of each direction's block, cut in
-// 6 row tiles of 16 and 6 column tiles of 8.  Per coarse site, direction d,
-// column-tile pair kp and row tile mt, lane l = 4 g + t holds eight halves: the
-// m16n8k8 A fragment {A(g, t), A(g + 8, t), A(g, t + 4), A(g + 8, t + 4)} of
-// column tile 2 kp, then that of column tile 2 kp + 1.  FP16 rounding as in
+// Blocks of the 48-dof coarse operator as k_coarse_mma reads them: the real
+// form A = [Re Y; Im Y] (96 x 48) of the self block and the four forward blocks
+// of a site (the backward ones are their adjoints), each as [row tile 12]
+// [column tile 6] tiles of 8 x 8 halves, row-major.  FP16 rounding as in
 // k_blocks_to_f16.
 __global__ void k_blocks_to_mma(const double2* __restrict__ Y, __half* __restrict__ Ym, long long nsites) {
-    constexpr int per_site = 9 * 3 * 6 * 32 * 8;
-    const long long n = nsites * per_site;
+    constexpr int per_block = 96 * 48;
+    const long long n = nsites * 5 * per_block;
     for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
-        const long long site = t / per_site;
-        const int r = (int)(t % per_site);
-        const int e = r & 7, lane = (r >> 3) & 31, f = r >> 8;     // f = (dir 3 + kp) 6 + mt
-        const int mt = f % 6, kp = (f / 6) % 3, dir = f / 18;
-        const int g = lane >> 2, tq = lane & 3, kt = 2 * kp + (e >> 2), q = e & 3;
-        const int row = mt * 16 + g + ((q & 1) ? 8 : 0);
-        const int col = kt * 8 + tq + ((q & 2) ? 4 : 0);
+        const long long sb = t / per_block, site = sb / 5;
+        const int r = (int)(t % per_block), blk = (int)(sb % 5);
+        const int dir = blk == 0 ? 0 : 2 * blk - 1;                // self, then the forward hops
+        const int tile = r >> 6;
+        const int row = (tile / 6) * 8 + ((r >> 3) & 7), col = (tile % 6) * 8 + (r & 7);
         const double2 v = Y[((site * 9 + dir) * 48 + row % 48) * 48 + col];
         Ym[t] = __double2half(row < 48 ? v.x : v.y);
+    }
+}
+
+// The backward blocks of a 4-d Galerkin kernel from the forward ones of the neighbours behind:
+// Dhat_W^dag = sigma_3 Dhat_W sigma_3 gives Y_-mu(x) = sigma_3 Y_+mu(x - mu)^dag sigma_3.
+__global__ void k_backward_blocks(double2* __restrict__ Y, AggIndex ai, int nvec, long long Vc) {
+    const int ncd = 2 * nvec;
+    const long long bsz = (long long)ncd * ncd, n = Vc * 4 * bsz;
+    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x) {
+        const int e = (int)(t % bsz), row = e / ncd, col = e % ncd;
+        const long long rest = t / bsz, xc = rest >> 2;
+        const int mu = (int)(rest & 3);
+        long long stride = 1;
+        for (int nu = 0; nu < mu; ++nu) stride *= ai.Lc[nu];
+        const int c = (int)((xc / stride) % ai.Lc[mu]);
+        const long long back = c == 0 ? xc + (ai.Lc[mu] - 1) * stride : xc - stride;
+        const double2 v = Y[(back * 9 + 1 + 2 * mu) * bsz + (long long)col * ncd + row];
+        const double sg = (row < nvec) == (col < nvec) ? 1.0 : -1.0;
+        Y[(xc * 9 + 2 + 2 * mu) * bsz + e] = make_double2(sg * v.x, -sg * v.y);
     }
 }
 
@@ -556,10 +571,12 @@ static dwf_status setup_impl(dwf_mg* h, const void* U, const void* starts) {
             return DWF_ERR_UNSUPPORTED;
         }
         const size_t sh = (size_t)(12 * m.nvec * 2 + 12 * m.ncd) * sizeof(float2);
-        dim3 grid((unsigned)m.Vc, 9);
+        dim3 grid((unsigned)m.Vc, 5);
         k_galerkin_4d<<<grid, GAL4_THREADS, sh, st>>>((const double2*)h->U64, h->P32, h->Y64, ai, m.nvec, G.V,
                                                       (float)((double)G.nd - h->M5),
                                                       make_int4(G.anti[0], G.anti[1], G.anti[2], G.anti[3]));
+        DWF_CHECK_LAUNCH();
+        k_backward_blocks<<<ew_grid(m.Vc * 4 * m.ncd * m.ncd), 256, 0, st>>>(h->Y64, ai, m.nvec, m.Vc);
         DWF_CHECK_LAUNCH();
     }
     k_blocks_to_f32<<<ew_grid(nblk * m.ncd * m.ncd), 256, 0, st>>>(h->Y64, h->Y32, nblk, m.ncd);
@@ -571,8 +588,8 @@ static dwf_status setup_impl(dwf_mg* h, const void* U, const void* starts) {
         DWF_CHECK_LAUNCH();
         h->ytile_half = 1;
         if (m.ncd == 48 && m.ndir == 9 && m.Ls_c <= 4) {
-            DWF_TRY(mg_alloc(h, &h->Ymma, nblk * m.ncd * m.ncd * sizeof(__half2)));
-            k_blocks_to_mma<<<ew_grid(nblk * m.ncd * m.ncd * 2), 256, 0, st>>>(h->Y64, (__half*)h->Ymma, m.Vc);
+            DWF_TRY(mg_alloc(h, &h->Ymma, m.Vc * 5 * m.ncd * m.ncd * sizeof(__half2)));
+            k_blocks_to_mma<<<ew_grid(m.Vc * 5 * m.ncd * m.ncd * 2), 256, 0, st>>>(h->Y64, (__half*)h->Ymma, m.Vc);
             DWF_CHECK_LAUNCH();
         }
     } else {
