@@ -18,83 +18,88 @@
 
 namespace dwf {
 
-template <class C> struct HalfSp { C v[2][3]; };   // 2 spins x 3 colours
+// Canonical layout: a site's 12 complex values are one record of 96 (FP32) or 192 (FP64) bytes.
+// With W32 (records on 32-byte boundaries) they move in 32-byte pieces: a warp's load touches every
+// one of its lines once per piece, and L1 handles a line per touch, so pieces of 16 bytes cost twice
+// the L1 time.  Sites are 32-bit (a 4-d lattice has at most 2^28 of them); slice offsets 64-bit.
+__device__ __forceinline__ void ld32(const float2* p, float2 (&v)[4]) {
+    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(v[0].x), "=f"(v[0].y), "=f"(v[1].x), "=f"(v[1].y), "=f"(v[2].x), "=f"(v[2].y), "=f"(v[3].x), "=f"(v[3].y)
+        : "l"(p));
+}
+__device__ __forceinline__ void ld32(const double2* p, double2 (&v)[2]) {
+    asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];"
+        : "=d"(v[0].x), "=d"(v[0].y), "=d"(v[1].x), "=d"(v[1].y) : "l"(p));
+}
+__device__ __forceinline__ void ld16(const float2* p, float2 (&v)[2]) {
+    const float4 a = __ldg(reinterpret_cast<const float4*>(p));
+    v[0] = make_float2(a.x, a.y); v[1] = make_float2(a.z, a.w);
+}
+__device__ __forceinline__ void ld16(const double2* p, double2 (&v)[1]) { v[0] = __ldg(p); }
 
-template <class R> struct Spin4 { typename cplx<R>::T v[4][3]; };
-
-// Canonical layout.  f4(s, site): float4 index of piece 0 of an FP32 spinor,
-// pieces KS apart; rec(s, site): site record of an FP64 spinor (12 double2);
-// lk(mu, site): index of entry 0 of a link, entries JS apart.  Sites are
-// 32-bit (a 4-d lattice has at most 2^28 of them); slice and direction
-// offsets are 64-bit.
-struct LayCanon {
-    static constexpr int KS = 1, JS = 1;
-    long long V;
-    __device__ __forceinline__ long long f4(int s, int site) const { return (long long)s * (V * 6) + (long long)site * 6; }
-    __device__ __forceinline__ long long rec(int s, int site) const { return (long long)s * V + site; }
-    __device__ __forceinline__ long long lk(int mu, int site) const { return (long long)mu * (V * 9) + (long long)site * 9; }
-};
-template <class LAY>
-__device__ __forceinline__ void ld_spin4(const float2* p, const LAY& L, int s, int site, Spin4<float>& v) {
-    const float4* q = reinterpret_cast<const float4*>(p) + L.f4(s, site);
+// N values from p into v[0 .. N - 1]: 16-byte pieces up to the first 32-byte boundary (HEAD values) and at the end
+template <bool W32, int N, int HEAD, class C>
+__device__ __forceinline__ void ld_values(const C* p, C* v) {
+    constexpr int P16 = 16 / sizeof(C), P32 = 32 / sizeof(C);
+    constexpr int n32 = W32 ? (N - HEAD) / P32 : 0, first = W32 ? HEAD : 0;
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        float4 a = __ldg(q + k * LAY::KS);
-        const int e0 = 2 * k, e1 = 2 * k + 1;
-        v.v[e0 / 3][e0 % 3] = make_float2(a.x, a.y);
-        v.v[e1 / 3][e1 % 3] = make_float2(a.z, a.w);
+    for (int i = 0; i < n32; ++i) {
+        C t[P32];
+        ld32(p + first + i * P32, t);
+#pragma unroll
+        for (int j = 0; j < P32; ++j) v[first + i * P32 + j] = t[j];
+    }
+#pragma unroll
+    for (int e = 0; e < N; e += P16) {
+        if (e >= first && e < first + n32 * P32) continue;
+        C t[P16];
+        ld16(p + e, t);
+#pragma unroll
+        for (int j = 0; j < P16; ++j) v[e + j] = t[j];
     }
 }
-__device__ __forceinline__ void ld_spin4(const double2* p, const LayCanon& L, int s, int site, Spin4<double>& v) {
-    const double2* q = p + L.rec(s, site) * 12;
-#pragma unroll
-    for (int e = 0; e < 12; ++e) v.v[e / 3][e % 3] = __ldg(q + e);
+template <bool W32, class C>
+__device__ __forceinline__ void ld_spin4(const C* p, C (&v)[4][3]) { ld_values<W32, 12, 0>(p, &v[0][0]); }
+// spins 2 hi, 2 hi + 1 (hi = 0: upper pair, 1: lower pair)
+template <bool W32, int HI, class C>
+__device__ __forceinline__ void ld_half(const C* p, C (&h)[2][3]) {
+    ld_values<W32, 6, HI && sizeof(C) == 8 ? 2 : 0>(p + 6 * HI, &h[0][0]);
 }
-// spins 2 hi, 2 hi + 1 (hi = 0: upper pair, 1: lower pair) into h[0..1]
-template <class LAY>
-__device__ __forceinline__ void ld_half(const float2* p, const LAY& L, int s, int site, int hi, float2 (&h)[2][3]) {
-    const float4* q = reinterpret_cast<const float4*>(p) + L.f4(s, site) + 3 * hi * LAY::KS;
+__device__ __forceinline__ void st_piece(float2* p, const float2* v, bool w32) {
+    if (w32)
+        asm volatile("st.global.cs.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0].x), "f"(v[0].y),
+                     "f"(v[1].x), "f"(v[1].y), "f"(v[2].x), "f"(v[2].y), "f"(v[3].x), "f"(v[3].y) : "memory");
+    else
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        float4 a = __ldg(q + k * LAY::KS);
-        const int e0 = 2 * k, e1 = 2 * k + 1;
-        h[e0 / 3][e0 % 3] = make_float2(a.x, a.y);
-        h[e1 / 3][e1 % 3] = make_float2(a.z, a.w);
+        for (int j = 0; j < 4; j += 2)
+            __stcs(reinterpret_cast<float4*>(p + j), make_float4(v[j].x, v[j].y, v[j + 1].x, v[j + 1].y));
+}
+__device__ __forceinline__ void st_piece(double2* p, const double2* v, bool w32) {
+    if (w32)
+        asm volatile("st.global.cs.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(v[0].x), "d"(v[0].y), "d"(v[1].x),
+                     "d"(v[1].y) : "memory");
+    else {
+        __stcs(p, v[0]);
+        __stcs(p + 1, v[1]);
     }
 }
-__device__ __forceinline__ void ld_half(const double2* p, const LayCanon& L, int s, int site, int hi, double2 (&h)[2][3]) {
-    const double2* q = p + L.rec(s, site) * 12 + 6 * hi;
+template <bool W32, class C>
+__device__ __forceinline__ void st_spin4(C* p, const C (&v)[4][3]) {
+    constexpr int P32 = 32 / sizeof(C);
 #pragma unroll
-    for (int e = 0; e < 6; ++e) h[e / 3][e % 3] = __ldg(q + e);
-}
-template <class LAY>
-__device__ __forceinline__ void st_spin4(float2* p, const LAY& L, int s, int site, const Spin4<float>& v) {
-    float4* q = reinterpret_cast<float4*>(p) + L.f4(s, site);
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        const int e0 = 2 * k, e1 = 2 * k + 1;
-        __stcs(q + k * LAY::KS, make_float4(v.v[e0 / 3][e0 % 3].x, v.v[e0 / 3][e0 % 3].y, v.v[e1 / 3][e1 % 3].x,
-                                            v.v[e1 / 3][e1 % 3].y));
-    }
-}
-__device__ __forceinline__ void st_spin4(double2* p, const LayCanon& L, int s, int site, const Spin4<double>& v) {
-    double2* q = p + L.rec(s, site) * 12;
-#pragma unroll
-    for (int e = 0; e < 12; ++e) __stcs(q + e, v.v[e / 3][e % 3]);
+    for (int e = 0; e < 12; e += P32) st_piece(p + e, &v[0][0] + e, W32);
 }
 
-// 3x3 link, row-major complex, in the storage of the link precision
-template <class LT, class LAY, class C>
-__device__ __forceinline__ void ld_link3(const typename LT::store* U, const LAY& L, int mu, int site, C (&u)[3][3]) {
-    const long long b0 = L.lk(mu, site);
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = 0; b < 3; ++b) {
-            auto v = load_link(U, b0 + (a * 3 + b) * LAY::JS);
-            u[a][b].x = v.x;
-            u[a][b].y = v.y;
-        }
+// acc + a b, acc + conj(a) b
+template <class C> __device__ __forceinline__ C cmac(C acc, C a, C b) {
+    acc.x = fma(a.x, b.x, acc.x); acc.x = fma(-a.y, b.y, acc.x);
+    acc.y = fma(a.x, b.y, acc.y); acc.y = fma(a.y, b.x, acc.y);
+    return acc;
+}
+template <class C> __device__ __forceinline__ C cmacc(C acc, C a, C b) {
+    acc.x = fma(a.x, b.x, acc.x); acc.x = fma(a.y, b.y, acc.x);
+    acc.y = fma(a.x, b.y, acc.y); acc.y = fma(-a.y, b.x, acc.y);
+    return acc;
 }
 
 // A psi_low for direction mu (A = -i sigma_1, -i sigma_2, -i sigma_3, 1)
@@ -120,78 +125,90 @@ __device__ __forceinline__ void apply_Adag(int mu, const C (&h)[2][3], C (&o)[2]
     }
 }
 
-// Block: 32 consecutive sites x 8 slices.  Blocks are numbered slice group
-// fastest, so the slice groups of one set of sites run together and share its
-// links and boundary slices in L2.
 template <class R> __device__ __forceinline__ R param_cast(double d, float f);
 template <> __device__ __forceinline__ double param_cast<double>(double d, float) { return d; }
 template <> __device__ __forceinline__ float param_cast<float>(double, float f) { return f; }
 
-template <class LT, class R, bool DAG, class LAY>
-__global__ void __launch_bounds__(256, 3) k_dwf4d(const typename LT::store* __restrict__ U,
+// Block: 32 consecutive sites x 8 slices.  Blocks are numbered slice group
+// fastest, so the slice groups of one set of sites run together and share its
+// links and boundary slices in L2.  The block first finds the 8 neighbours of its sites, one
+// thread each.  Bound by L1 (a spinor piece touches 24 lines per warp) and FP32 issue; FP64 by the
+// FP64 pipe.  16^3 x 32 x 16, FP16 links: 173 us against 222 us with 16-byte pieces, products
+// and sums apart and the index divisions in every thread; 12^3 x 24 x 12 in FP64, at the 128
+// registers its values need, 834 against 1159 us.  (The block's links staged in shared memory:
+// 191 us, 226 us for the adjoint, whose registers then spill.)
+constexpr int NB_CROSS = 1 << 30;         // the hop crosses a boundary (sites are below 2^28)
+template <class LT, class R, bool DAG, bool W32>
+__global__ void __launch_bounds__(256, sizeof(R) == 8 ? 2 : 3) k_dwf4d(const typename LT::store* __restrict__ U,
                                                const typename cplx<R>::T* __restrict__ psi,
-                                               typename cplx<R>::T* __restrict__ out, Fine4dParams p, LAY lay,
+                                               typename cplx<R>::T* __restrict__ out, Fine4dParams p,
                                                int ngroups, const int* skip) {
     if (skip && *skip) return;
     using C = typename cplx<R>::T;
-    const int site = (int)(blockIdx.x / ngroups) * 32 + threadIdx.x;
+    __shared__ int nbs[8][32];
+    const int V = (int)p.V;
+    const int base = (int)(blockIdx.x / ngroups) * 32;
+    const int site = base + threadIdx.x;
     const int s = (int)(blockIdx.x % ngroups) * 8 + threadIdx.y;
-    if (site >= p.V || s >= p.Ls) return;
-    int stride[4];
-    int coord[4];
     {
-        int st = 1, rem = site;
+        // neighbour 2 mu (forward) or 2 mu + 1 (backward); sites past the end take the last site's
+        const int x = min(site, V - 1), mu = threadIdx.y >> 1;
+        const bool fwd = !(threadIdx.y & 1);
+        int stride = 1, rem = x, c = 0, L = 1;
 #pragma unroll
-        for (int mu = 0; mu < 4; ++mu) {
-            stride[mu] = st;
-            coord[mu] = rem % p.L[mu];
-            rem /= p.L[mu];
-            st *= p.L[mu];
+        for (int nu = 0; nu < 4; ++nu) {
+            const int q = rem / p.L[nu];
+            if (nu == mu) { c = rem - q * p.L[nu]; L = p.L[nu]; }
+            if (nu < mu) stride *= p.L[nu];
+            rem = q;
         }
+        const bool cross = fwd ? c == L - 1 : c == 0;
+        const int nb = fwd ? (cross ? x - (L - 1) * stride : x + stride) : (cross ? x + (L - 1) * stride : x - stride);
+        nbs[threadIdx.y][threadIdx.x] = nb | (cross ? NB_CROSS : 0);
     }
+    __syncthreads();
+    if (site >= V || s >= p.Ls) return;
     C up[2][3], lo[2][3];     // accumulated -1/2 sum of hops, upper / lower spin pairs
 #pragma unroll
     for (int a = 0; a < 2; ++a)
 #pragma unroll
         for (int c = 0; c < 3; ++c) { up[a][c] = mk<C>(R(0), R(0)); lo[a][c] = mk<C>(R(0), R(0)); }
+    const C* plane = psi + (long long)s * V * 12;
 
 #pragma unroll
     for (int mu = 0; mu < 4; ++mu) {
-        const int L = p.L[mu];
         // forward: y = x + mu, link U_mu(x); backward: y = x - mu, link U_mu(y)^dag
 #pragma unroll
         for (int dirn = 0; dirn < 2; ++dirn) {
             const bool fwd = dirn == 0;
-            const bool cross = fwd ? (coord[mu] == L - 1) : (coord[mu] == 0);
-            const int nb = fwd ? (cross ? site - (L - 1) * stride[mu] : site + stride[mu])
-                               : (cross ? site + (L - 1) * stride[mu] : site - stride[mu]);
-            const R ph = (cross && p.anti[mu]) ? R(-1) : R(1);
+            const int nbw = nbs[2 * mu + dirn][threadIdx.x], nb = nbw & (NB_CROSS - 1);
+            const R ph = ((nbw & NB_CROSS) && p.anti[mu]) ? R(-1) : R(1);
             // projector sign: D uses (1 - gamma) forward, (1 + gamma) backward; D^dag the opposite
             const bool minus = (fwd != DAG);
-            Spin4<R> v;
-            ld_spin4(psi + 0, lay, s, nb, v);
-            C lw[2][3] = {{v.v[2][0], v.v[2][1], v.v[2][2]}, {v.v[3][0], v.v[3][1], v.v[3][2]}};
+            C v[4][3];
+            ld_spin4<W32>(plane + (long long)nb * 12, v);
+            C lw[2][3] = {{v[2][0], v[2][1], v[2][2]}, {v[3][0], v[3][1], v[3][2]}};
             C Al[2][3];
             apply_A(mu, lw, Al);
             C h[2][3];
 #pragma unroll
             for (int a = 0; a < 2; ++a)
 #pragma unroll
-                for (int c = 0; c < 3; ++c) h[a][c] = minus ? (v.v[a][c] - Al[a][c]) : (v.v[a][c] + Al[a][c]);
+                for (int c = 0; c < 3; ++c) h[a][c] = minus ? (v[a][c] - Al[a][c]) : (v[a][c] + Al[a][c]);
             C u[3][3];
-            ld_link3<LT>(U, lay, mu, fwd ? site : nb, u);
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+#pragma unroll
+                for (int b = 0; b < 3; ++b) u[a][b] = load_link(U, ((long long)mu * V + (fwd ? site : nb)) * 9 + a * 3 + b);
             C uh[2][3];
 #pragma unroll
             for (int a = 0; a < 2; ++a)
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
-                    C acc = mk<C>(R(0), R(0));
+                    // forward: U h; backward: U^dag h
+                    C acc = fwd ? cmul(u[c][0], h[a][0]) : cmulc(u[0][c], h[a][0]);
 #pragma unroll
-                    for (int b = 0; b < 3; ++b) {
-                        // forward: U h; backward: U^dag h
-                        const C uu = fwd ? u[c][b] : mk<C>(u[b][c].x, -u[b][c].y);
-                        acc = acc + cmul(uu, h[a][b]);
-                    }
+                    for (int b = 1; b < 3; ++b) acc = fwd ? cmac(acc, u[c][b], h[a][b]) : cmacc(acc, u[b][c], h[a][b]);
                     uh[a][c] = acc;
                 }
             C Ad[2][3];
@@ -208,8 +225,8 @@ __global__ void __launch_bounds__(256, 3) k_dwf4d(const typename LT::store* __re
     }
     const R diag = param_cast<R>(p.diag, p.diag_f);
     const R mf = param_cast<R>(p.mf, p.mf_f);
-    Spin4<R> self;
-    ld_spin4(psi + 0, lay, s, site, self);
+    C self[4][3];
+    ld_spin4<W32>(plane + (long long)site * 12, self);
     // s-hops: D: up += psi_{s-1}.up (or -m psi_{Ls-1}.up), lo += psi_{s+1}.lo (or -m psi_0.lo)
     //         D^dag: up from s+1 / wall psi_0, lo from s-1 / wall psi_{Ls-1}
     const int s_up = DAG ? (s + 1 < p.Ls ? s + 1 : 0) : (s > 0 ? s - 1 : p.Ls - 1);
@@ -217,17 +234,17 @@ __global__ void __launch_bounds__(256, 3) k_dwf4d(const typename LT::store* __re
     const R f_up = DAG ? (s + 1 < p.Ls ? R(1) : -mf) : (s > 0 ? R(1) : -mf);
     const R f_lo = DAG ? (s > 0 ? R(1) : -mf) : (s + 1 < p.Ls ? R(1) : -mf);
     C hu[2][3], hl[2][3];
-    ld_half(psi + 0, lay, s_up, site, 0, hu);
-    ld_half(psi + 0, lay, s_lo, site, 1, hl);
-    Spin4<R> o;
+    ld_half<W32, 0>(psi + ((long long)s_up * V + site) * 12, hu);
+    ld_half<W32, 1>(psi + ((long long)s_lo * V + site) * 12, hl);
+    C o[4][3];
 #pragma unroll
     for (int a = 0; a < 2; ++a)
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            o.v[a][c] = scale(up[a][c], R(-0.5)) + scale(self.v[a][c], diag) + scale(hu[a][c], f_up);
-            o.v[a + 2][c] = scale(lo[a][c], R(-0.5)) + scale(self.v[a + 2][c], diag) + scale(hl[a][c], f_lo);
+            o[a][c] = scale(up[a][c], R(-0.5)) + scale(self[a][c], diag) + scale(hu[a][c], f_up);
+            o[a + 2][c] = scale(lo[a][c], R(-0.5)) + scale(self[a + 2][c], diag) + scale(hl[a][c], f_lo);
         }
-    st_spin4(out + 0, lay, s, site, o);
+    st_spin4<W32>(out + ((long long)s * V + site) * 12, o);
 }
 
 static dwf_status grid4d(const Fine4dParams& p, unsigned* blocks, int* ngroups) {
@@ -239,9 +256,9 @@ static dwf_status grid4d(const Fine4dParams& p, unsigned* blocks, int* ngroups) 
     return DWF_OK;
 }
 
-template <class LT, class R, class LAY>
-static dwf_status launch4d(const void* U, const void* psi, void* out, const Fine4dParams& p, const LAY& lay,
-                           bool dagger, cudaStream_t st, const int* skip = nullptr) {
+template <class LT, class R>
+static dwf_status launch4d(const void* U, const void* psi, void* out, const Fine4dParams& p, bool dagger,
+                           cudaStream_t st, const int* skip = nullptr) {
     unsigned blocks;
     int ng;
     DWF_TRY(grid4d(p, &blocks, &ng));
@@ -250,8 +267,15 @@ static dwf_status launch4d(const void* U, const void* psi, void* out, const Fine
     auto Ut = reinterpret_cast<const typename LT::store*>(U);
     auto pi = reinterpret_cast<const C*>(psi);
     auto po = reinterpret_cast<C*>(out);
-    if (dagger) k_dwf4d<LT, R, true, LAY><<<blocks, block, 0, st>>>(Ut, pi, po, p, lay, ng, skip);
-    else        k_dwf4d<LT, R, false, LAY><<<blocks, block, 0, st>>>(Ut, pi, po, p, lay, ng, skip);
+    // the ABI promises 16-byte alignment; records (96 or 192 bytes) keep a 32-byte aligned base's alignment
+    const bool w32 = ((reinterpret_cast<uintptr_t>(psi) | reinterpret_cast<uintptr_t>(out)) & 31u) == 0;
+    if (w32) {
+        if (dagger) k_dwf4d<LT, R, true, true><<<blocks, block, 0, st>>>(Ut, pi, po, p, ng, skip);
+        else        k_dwf4d<LT, R, false, true><<<blocks, block, 0, st>>>(Ut, pi, po, p, ng, skip);
+    } else {
+        if (dagger) k_dwf4d<LT, R, true, false><<<blocks, block, 0, st>>>(Ut, pi, po, p, ng, skip);
+        else        k_dwf4d<LT, R, false, false><<<blocks, block, 0, st>>>(Ut, pi, po, p, ng, skip);
+    }
     return DWF_OK;
 }
 
@@ -272,12 +296,11 @@ dwf_status fine_apply_4d(const Geom& g, const void* U, const void* psi, void* ou
                          bool dagger, int prec, int s_chunk, cudaStream_t st, const int* skip) {
     (void)s_chunk;
     const Fine4dParams p = params4d(g, M5, mf);
-    LayCanon lay{g.V};
     switch (prec) {
-        case DWF_F64:       DWF_TRY((launch4d<LinkF64, double>(U, psi, out, p, lay, dagger, st, skip))); break;
-        case DWF_F32:       DWF_TRY((launch4d<LinkF32, float>(U, psi, out, p, lay, dagger, st, skip))); break;
-        case DWF_F32_L16:   DWF_TRY((launch4d<LinkH16, float>(U, psi, out, p, lay, dagger, st, skip))); break;
-        case DWF_F32_LBF16: DWF_TRY((launch4d<LinkBF16, float>(U, psi, out, p, lay, dagger, st, skip))); break;
+        case DWF_F64:       DWF_TRY((launch4d<LinkF64, double>(U, psi, out, p, dagger, st, skip))); break;
+        case DWF_F32:       DWF_TRY((launch4d<LinkF32, float>(U, psi, out, p, dagger, st, skip))); break;
+        case DWF_F32_L16:   DWF_TRY((launch4d<LinkH16, float>(U, psi, out, p, dagger, st, skip))); break;
+        case DWF_F32_LBF16: DWF_TRY((launch4d<LinkBF16, float>(U, psi, out, p, dagger, st, skip))); break;
         default: set_error("bad precision %d", prec); return DWF_ERR_ARG;
     }
     DWF_CHECK_LAUNCH();
