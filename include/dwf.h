@@ -359,7 +359,8 @@ typedef struct {
                              1, 2, 4 column tiles per warp; 5 = tcgen05 with one (site, column
                              tile) per thread block; 6 = the tcgen05 form with the data
                              operand in tensor memory wherever eligible (fixed forms, for
-                             testing each one)                                                 */
+                             testing each one).  With FP16 blocks, one column tile (2) takes the data
+                             as scaled FP16 high and low parts in place of TF32 ones           */
     int transfer;         /* 0 (default): the truncated wall transfer of Eq. TruncProjectInterpolate;
                              1: the bulk transfer the paper compares it with (Sec. 4.1), P^dag /
                              P on every slice, which needs Ls_c = Ls                           */

@@ -60,7 +60,7 @@ __device__ __forceinline__ float2 block_val(const float2* p) { return __ldg(p); 
 __device__ __forceinline__ float2 block_val(const __half2* p) { return __half22float2(__ldg(p)); }
 
 // BT = float2: FP32 blocks, split into TF32 high and low parts (three products
-// per term).  BT = __half2: FP16 blocks, exact in TF32 (same 11-bit
+// per term).  BT = __half2 (from two column tiles per warp on): FP16 blocks, exact in TF32 (same 11-bit
 // significand), so only the vectors are split (two products per term).
 template <int NT, class BT>
 __global__ void __launch_bounds__(256, 2) k_coarse_tc(const BT* __restrict__ Y, const float2* __restrict__ in,
@@ -172,6 +172,212 @@ __global__ void __launch_bounds__(256, 2) k_coarse_tc(const BT* __restrict__ Y, 
                 out[rb + (long long)s * p.cs] = make_float2(hr + self.x + sc * hv.x, hi + self.y + sc * hv.y);
             }
         }
+}
+
+// ---------------------------------------------------------------------------
+// FP16 blocks, one column tile of 8 at a time (form 1).  A block of 16 warps owns a 4 x 4 tile of
+// coarse sites, one warp per site, and walks a range of column tiles:
+//   * the inputs of the tile's 32 sites (16 and their outer neighbours, without the corners) for 8
+//     columns are read once, in whole lines, while the previous 8 columns are multiplied, so that
+//     every input is read and converted twice in all instead of five times; the identity and the
+//     s-hops read their FP32 values from shared memory too;
+//   * each (site, column) is scaled by a power of two to below 2^14 and split into two FP16 parts (22
+//     bits, what a TF32 high / low pair keeps), in shared memory as the 8 x 8 tiles that
+//     ldmatrix hands to mma.m16n8k16 as B; the blocks are the A operand as stored, in
+//     registers for all five directions, with no conversion and half the products of TF32;
+//   * a direction's products accumulate in FP32 and are added up in FP32 with the scale taken back.
+// Per warp, direction and column tile: 2 ldmatrix, 8 mma, 8 multiply-adds; with the conversion and the
+// epilogue about 600 instructions per warp and column tile, whose issue (51% of the slots) is what bounds
+// it.  64 vectors at 64^2 x 4: 172 us, against 192 us of the tcgen05 form with the data in tensor memory and
+// 205 to 225 us of the TF32 mma.sync forms, and 1.0e-7 of error against 64 bits where they have 3.6e-7.
+// (Loading 64 bytes per thread and the s-hops from global memory: 211 us, L1 at 80%; one block per tile of
+// sites, 1.7 rounds of them: no change.)
+// ---------------------------------------------------------------------------
+constexpr int CF_TX = 4, CF_TY = 4, CF_SITES = CF_TX * CF_TY, CF_HALO = CF_SITES + 2 * CF_TX + 2 * CF_TY;
+constexpr int CF_THREADS = 32 * CF_SITES;
+constexpr int CF_ITEMS = CF_HALO * 8 * 8 / CF_THREADS;   // 16-byte pieces of the inputs per thread and column tile
+constexpr int CF_TILE = 192;     // bytes between 8 x 8 tiles: the two tiles a warp stores to at once share no bank
+constexpr int CF_ROW = 144;      // bytes between FP32 rows: the columns that a warp reads at once share no bank
+static_assert(CF_HALO == 32 && CF_THREADS == 512, "the loading threads' places");
+struct CfSmem {
+    // per site 8 tiles of [column 8][dof 8] halves: high parts Re 0-7, Re 8-15, Im 0-7, Im 8-15, then the low parts
+    unsigned char v[2][CF_HALO][8 * CF_TILE];
+    unsigned char raw[2][CF_SITES][8 * CF_ROW];          // the tile's own inputs in FP32, [column][dof]
+    float back[2][CF_HALO][8];                           // what undoes the scale, per (site, column)
+};
+
+__device__ __forceinline__ void cf_ldmatrix(uint32_t (&a)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void cf_mma(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+                 "{%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// c = A b
+__device__ __forceinline__ void cf_mma0(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+                 "{%10,%10,%10,%10};"
+                 : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+}
+__device__ __forceinline__ uint32_t cf_pack(__half a, __half b) {
+    const __half2 h = __halves2half2(a, b);
+    return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+// One block per SM; block b takes the steps [b per_block, (b + 1) per_block) of the list of (tile of
+// sites, column tile), column tiles fastest, so that every block has the same number of them.
+__global__ void __launch_bounds__(CF_THREADS, 1)
+k_coarse_f16(const __half2* __restrict__ Y, const float2* __restrict__ in, float2* __restrict__ out, TcParams p,
+             long long steps, long long per_block, unsigned inv_Ls, const int* __restrict__ skip_rhs) {
+    extern __shared__ __align__(128) unsigned char cf_raw[];
+    CfSmem& sm = *reinterpret_cast<CfSmem*>(cf_raw);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+    const int ntx = (p.Lc0 + CF_TX - 1) / CF_TX;
+    const int ngroups = (p.ncols + 7) / 8;
+    // right-hand side of a column: exact below 2^32 / Ls_c columns (inv_Ls = ceil(2^32 / Ls_c))
+    auto rhs_of = [&](int col) { return p.Ls_c == 1 ? col : (int)__umulhi((unsigned)col, inv_Ls); };
+    const long long step1 = min(steps, ((long long)blockIdx.x + 1) * per_block);
+    for (long long step = (long long)blockIdx.x * per_block; step < step1;) {
+    const int tile = (int)(step / ngroups), first = (int)(step - (long long)tile * ngroups);
+    const int g1 = (int)min((long long)ngroups, first + (step1 - step));
+    step += g1 - first;
+    const int x0 = (tile % ntx) * CF_TX, y0 = (tile / ntx) * CF_TY;
+    // the first group of columns from cg on that has a right-hand side to work on (block-uniform)
+    auto live = [&](int cg) {
+        for (; cg < g1; ++cg) {
+            if (!skip_rhs) return cg;
+            const int r1 = rhs_of(min(8 * cg + 7, p.ncols - 1));
+            for (int r = rhs_of(8 * cg); r <= r1; ++r)
+                if (!skip_rhs[r]) return cg;
+        }
+        return g1;
+    };
+    int cg = live(first);
+    if (cg >= g1) continue;
+    // loading: 8 threads take the 128 bytes of a (site, column); this thread's piece of column ln, and the sites
+    // 8 i + threadIdx.x / 64.  Sites of the halo: the tile, then x = -1, x = 4 (4 each), y = -1, y = 4
+    const int lc = threadIdx.x & 7, ln = (threadIdx.x >> 3) & 7, l0 = threadIdx.x >> 6;
+    long long src[CF_ITEMS];
+#pragma unroll
+    for (int i = 0; i < CF_ITEMS; ++i) {
+        const int lh = 8 * i + l0;
+        const int hx = lh < 16 ? lh & 3 : lh < 20 ? -1 : lh < 24 ? CF_TX : lh & 3;
+        const int hy = lh < 16 ? lh >> 2 : lh < 24 ? lh & 3 : lh < 28 ? -1 : CF_TY;
+        const int gx = (x0 + hx + p.Lc0) % p.Lc0, gy = (y0 + hy + p.Lc1) % p.Lc1;
+        src[i] = ((long long)gy * p.Lc0 + gx) * p.ss + 2 * lc;
+    }
+    float4 ld[CF_ITEMS];
+    auto load = [&](int grp) {
+        const int col = 8 * grp + ln;
+        const bool ok = col < p.ncols && !(skip_rhs && skip_rhs[rhs_of(col)]);
+        const float2* q = in + (long long)(ok ? col : 0) * p.cs;
+#pragma unroll
+        for (int i = 0; i < CF_ITEMS; ++i)
+            ld[i] = ok ? __ldg(reinterpret_cast<const float4*>(q + src[i])) : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    auto convert = [&](int buf) {
+#pragma unroll
+        for (int i = 0; i < CF_ITEMS; ++i) {
+            const int lh = 8 * i + l0;
+            const float4 u = ld[i];
+            float m = fmaxf(fmaxf(fabsf(u.x), fabsf(u.y)), fmaxf(fabsf(u.z), fabsf(u.w)));
+            m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
+            m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
+            m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 4));
+            // 2^(13 - exponent of m); tiny columns are left where 2^113 brings them
+            const int e = max((int)(__float_as_uint(m) >> 23), 27);
+            float scale = __uint_as_float((unsigned)(127 + 13 + 127 - e) << 23);
+            if (lc == 0) sm.back[buf][lh][ln] = __uint_as_float((unsigned)(e - 13) << 23);
+            if (p.dag && lc >= 4) scale = -scale;        // sigma_3 on the chirality - inputs
+            const float re0 = u.x * scale, im0 = u.y * scale, re1 = u.z * scale, im1 = u.w * scale;
+            const __half2 hr = __floats2half2_rn(re0, re1), hi = __floats2half2_rn(im0, im1);
+            const float2 fr = __half22float2(hr), fi = __half22float2(hi);
+            unsigned char* d = sm.v[buf][lh] + (lc >> 2) * CF_TILE + ln * 16 + (lc & 3) * 4;
+            *reinterpret_cast<__half2*>(d) = hr;
+            *reinterpret_cast<__half2*>(d + 2 * CF_TILE) = hi;
+            *reinterpret_cast<__half2*>(d + 4 * CF_TILE) = __floats2half2_rn(re0 - fr.x, re1 - fr.y);
+            *reinterpret_cast<__half2*>(d + 6 * CF_TILE) = __floats2half2_rn(im0 - fi.x, im1 - fi.y);
+            if (i < CF_SITES / 8) *reinterpret_cast<float4*>(sm.raw[buf][lh] + ln * CF_ROW + lc * 16) = u;
+        }
+    };
+    load(cg);
+    // multiplying: this warp's site and the halo places of its neighbours
+    const int wx = warp & 3, wy = warp >> 2;
+    const bool mine = x0 + wx < p.Lc0 && y0 + wy < p.Lc1;
+    const long long xc = mine ? (long long)(y0 + wy) * p.Lc0 + x0 + wx : 0;
+    const int place[5] = {warp, wx < 3 ? warp + 1 : 20 + wy, wx > 0 ? warp - 1 : 16 + wy, wy < 3 ? warp + 4 : 28 + wx,
+                          wy > 0 ? warp - 4 : 24 + wx};
+    uint32_t yr[5][4], yi[5][4];                         // A fragments of Re Y and Im Y
+#pragma unroll
+    for (int d = 0; d < 5; ++d) {
+        const __half2* Yb = Y + (xc * 5 + d) * 256;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {                    // rows g + 8 (q & 1), columns 2 t + 8 (q >> 1), + 1
+            const __half2* a = Yb + (2 * t + 8 * (q >> 1)) * 16 + g + 8 * (q & 1);
+            const __half2 a0 = __ldg(a), a1 = __ldg(a + 16);
+            yr[d][q] = cf_pack(__low2half(a0), __low2half(a1));
+            yi[d][q] = cf_pack(__high2half(a0), __high2half(a1));
+        }
+    }
+    convert(0);
+    __syncthreads();
+    for (int buf = 0; cg < g1; buf ^= 1) {
+        const int next = live(cg + 1);
+        if (next < g1) load(next);
+        if (mine) {
+            float re[4] = {0.f, 0.f, 0.f, 0.f}, im[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int d = 0; d < 5; ++d) {
+                const uint32_t addr = smem_u32(sm.v[buf][place[d]]) + (lane >> 3) * CF_TILE + (lane & 7) * 16;
+                uint32_t bh[4], bl[4];                   // Re 0-7, Re 8-15, Im 0-7, Im 8-15
+                cf_ldmatrix(bh, addr);
+                cf_ldmatrix(bl, addr + 4 * CF_TILE);
+                const float2 sc = *reinterpret_cast<const float2*>(&sm.back[buf][place[d]][2 * t]);
+                const uint32_t ny[4] = {yi[d][0] ^ 0x80008000u, yi[d][1] ^ 0x80008000u, yi[d][2] ^ 0x80008000u,
+                                        yi[d][3] ^ 0x80008000u};
+                float c0[4], c1[4];
+                cf_mma0(c0, yr[d], bh[0], bh[1]); cf_mma0(c1, yi[d], bh[0], bh[1]);
+                cf_mma(c0, ny, bh[2], bh[3]);    cf_mma(c1, yr[d], bh[2], bh[3]);
+                cf_mma(c0, yr[d], bl[0], bl[1]); cf_mma(c1, yi[d], bl[0], bl[1]);
+                cf_mma(c0, ny, bl[2], bl[3]);    cf_mma(c1, yr[d], bl[2], bl[3]);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    re[q] = fmaf(q & 1 ? sc.y : sc.x, c0[q], re[q]);
+                    im[q] = fmaf(q & 1 ? sc.y : sc.x, c1[q], im[q]);
+                }
+            }
+            // lane: rows g and g + 8 of columns 2 t, 2 t + 1; the identity and the chiral hops along s in FP32
+#pragma unroll
+            for (int w = 0; w < 2; ++w) {
+                const int col = 8 * cg + 2 * t + w;
+                const int r = rhs_of(col), s = col - r * p.Ls_c;
+                if (col >= p.ncols || (skip_rhs && skip_rhs[r])) continue;
+                float2* op = out + (long long)col * p.cs + xc * p.ss + g;
+                const unsigned char* row = sm.raw[buf][warp] + g * 8;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float so = p.dag && h ? -1.f : 1.f;
+                    const bool below = p.dag ? h == 1 : h == 0;
+                    const int sh = below ? (s > 0 ? s - 1 : p.Ls_c - 1) : (s < p.Ls_c - 1 ? s + 1 : 0);
+                    const float f = below ? (s > 0 ? 1.f : -p.mf) : (s < p.Ls_c - 1 ? 1.f : -p.mf);
+                    const float2 self = *reinterpret_cast<const float2*>(row + (2 * t + w) * CF_ROW + 64 * h);
+                    const int hc = r * p.Ls_c + sh - 8 * cg;     // the hop's column in this tile, if it is there
+                    const float2 hv = hc >= 0 && hc < 8 ? *reinterpret_cast<const float2*>(row + hc * CF_ROW + 64 * h)
+                                                        : __ldg(in + (long long)(col - s + sh) * p.cs + xc * p.ss + g + 8 * h);
+                    op[8 * h] = make_float2(so * re[2 * h + w] + self.x + f * hv.x,
+                                            so * im[2 * h + w] + self.y + f * hv.y);
+                }
+            }
+        }
+        if (next < g1) convert(buf ^ 1);
+        __syncthreads();
+        cg = next;
+    }
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1129,6 +1335,7 @@ static dwf_status tc_device_init(int* sms_out) {
                                             (int)sizeof(UpSmem)));
         DWF_CHECK_CUDA(cudaFuncSetAttribute(k_coarse_umma_t<UT_NG, UT_NR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             (int)sizeof(UtSmem<UT_NG, UT_NR>)));
+        DWF_CHECK_CUDA(cudaFuncSetAttribute(k_coarse_f16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CfSmem)));
         int sms = 0;
         DWF_CHECK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         if (sms <= 0) { set_error("no multiprocessors reported"); return DWF_ERR_CUDA; }
@@ -1177,6 +1384,20 @@ static dwf_status launch_form(const dwf_mg* h, int form, const TcParams& p, cons
         DWF_CHECK_LAUNCH();
         return DWF_OK;
     }
+    if (form == 1 && h->ytile_half) {
+        int sms = 0;
+        DWF_TRY(tc_device_init(&sms));
+        const long long tiles = (long long)((p.Lc0 + CF_TX - 1) / CF_TX) * ((p.Lc1 + CF_TY - 1) / CF_TY);
+        const long long steps = tiles * ((p.ncols + 7) / 8);
+        if (tiles > 0x7fffffffLL) { set_error("coarse batch too large for one launch"); return DWF_ERR_ARG; }
+        const long long per = (steps + sms - 1) / sms;
+        if (per < 1) return DWF_OK;
+        const unsigned inv_Ls = p.Ls_c > 1 ? (unsigned)(((1ULL << 32) + p.Ls_c - 1) / p.Ls_c) : 0u;
+        k_coarse_f16<<<(unsigned)((steps + per - 1) / per), CF_THREADS, sizeof(CfSmem), st>>>(
+            (const __half2*)h->Ytile, in, out, p, steps, per, inv_Ls, skip_rhs);
+        DWF_CHECK_LAUNCH();
+        return DWF_OK;
+    }
     const int NT = form;
     const long long warps = p.Vc * ((p.ncols + 8 * NT - 1) / (8 * NT));
     const long long blocks = (warps * 32 + 255) / 256;
@@ -1186,7 +1407,7 @@ static dwf_status launch_form(const dwf_mg* h, int form, const TcParams& p, cons
         k_coarse_tc<N, __half2><<<(unsigned)blocks, 256, 0, st>>>((const __half2*)h->Ytile, in, out, p, skip_rhs);   \
     else                                                                                                               \
         k_coarse_tc<N, float2><<<(unsigned)blocks, 256, 0, st>>>(h->Y32, in, out, p, skip_rhs);
-    if (NT == 1) { DWF_TC_LAUNCH(1) }
+    if (NT == 1) k_coarse_tc<1, float2><<<(unsigned)blocks, 256, 0, st>>>(h->Y32, in, out, p, skip_rhs);
     else if (NT == 2) { DWF_TC_LAUNCH(2) }
     else { DWF_TC_LAUNCH(4) }
 #undef DWF_TC_LAUNCH
