@@ -957,22 +957,22 @@ __device__ __forceinline__ int chir_dof(const TransferParams& p, int c, int cd) 
 // back); skip[r]: per right-hand side.  Bound by the read of P (and by launch latency below a
 // few MB): with one thread per output, walking the sites one after the other through the index
 // divisions, 256^2 took 30 us and 12^3 x 24 (nvec 24) 132 us; the two transfers and two coarse
-// applies of a 256^2 hierarchy together went from 96.6 to 51.3 us.
+// applies of a 256^2 hierarchy together went from 96.6 to 51.3 us (and from 42.9 to 35.7 later, with
+// eight sites' loads before the first product and 32-bit offsets).
 constexpr int RESTRICT_THREADS = 288;   // both chiralities of one aggregate at 4-d, nvec 24
 constexpr int RESTRICT_TABLE = 2048;    // aggregates up to this many sites keep their offsets in shared memory
 
-__global__ void __launch_bounds__(RESTRICT_THREADS)
+__global__ void __launch_bounds__(RESTRICT_THREADS, 2)
 k_restrict(const float2* __restrict__ P, const float2* __restrict__ r, float2* __restrict__ out, TransferParams p,
            const int* skip) {
     if (skip && skip[blockIdx.y]) return;
-    __shared__ long long off[RESTRICT_TABLE];
+    __shared__ unsigned off[RESTRICT_TABLE];
     __shared__ float2 red[RESTRICT_THREADS];
     const int J = p.nchd * p.nvec;
     const int G = blockDim.x / J;
     const bool table = p.nb <= RESTRICT_TABLE;
     if (table)
-        for (int l = threadIdx.x; l < p.nb; l += blockDim.x) off[l] = agg_site(p, 0, l);
-    __syncthreads();
+        for (int l = threadIdx.x; l < p.nb; l += blockDim.x) off[l] = (unsigned)agg_site(p, 0, l);
     const long long nc = p.Vc * p.Ls_c * p.ncd;
     r += (long long)blockIdx.y * p.V * p.Ls * p.dof;
     out += (long long)blockIdx.y * nc;
@@ -982,18 +982,28 @@ k_restrict(const float2* __restrict__ P, const float2* __restrict__ r, float2* _
     const int c = (int)(g & 1);
     const long long xs = g >> 1;
     const bool in = xs < p.Vc * (p.bulk ? p.Ls : 1);
-    const long long xc = xs % p.Vc;
+    const long long xc = p.bulk ? xs % p.Vc : xs;
     // Phat_- P^dag P_- r_1 on coarse slice 1, Phat_+ P^dag P_+ r_Ls on coarse slice Lhat_s; bulk: every slice
     const int sf = p.bulk ? (int)(xs / p.Vc) : (c == 1 ? 0 : p.Ls - 1);
     float2 acc = make_float2(0.f, 0.f);
+    const int d = chir_dof(p, c, cd);
+    const long long base = in ? agg_site(p, xc, 0) : 0;
+    const float2* Pc = P + c * J + j;
+    __syncthreads();
     if (in) {
-        const int d = chir_dof(p, c, cd);
-        const long long base = agg_site(p, xc, 0);
-        const float2* Pc = P + c * J + j;
-#pragma unroll 8
-        for (int l = 0; l < p.nb; ++l) {
-            const long long x = base + (table ? off[l] : agg_site(p, 0, l));
-            acc = cfma_conj(__ldg(Pc + x * 2 * J), __ldg(r + fine_idx(p, sf, x, d)), acc);
+        // eight sites' loads before the first product
+        for (int l0 = 0; l0 < p.nb; l0 += 8) {
+            float2 a[8], b[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int l = min(l0 + q, p.nb - 1);
+                const long long x = base + (table ? off[l] : (unsigned)agg_site(p, 0, l));
+                a[q] = __ldg(Pc + x * 2 * J);
+                b[q] = __ldg(r + fine_idx(p, sf, x, d));
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (l0 + q < p.nb) acc = cfma_conj(a[q], b[q], acc);
         }
     }
     if (p.nchd > 1) {
