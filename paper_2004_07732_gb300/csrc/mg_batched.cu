@@ -20,6 +20,7 @@
 // side (and per basis vector for the Gram-Schmidt dots of vectors that fit in
 // L2; larger vectors take all basis vectors in one pass over w), so the rows
 // finish independently and each result is summed in a fixed order.
+#include <algorithm>
 #include <chrono>
 #include <mutex>
 #include <string.h>
@@ -923,6 +924,7 @@ struct BatchedState {
     double* hvals = nullptr;          // pinned: bn2, rn2, rA2, ref2, scale, rn [6][cap]
     cudaGraphExec_t gfirst = nullptr, gcycle = nullptr;
     int gnrhs = 0;                    // right-hand sides the graphs were captured for
+    int cycles = 1;                   // restart cycles the last coarse solve took (launched ahead of the first check)
     ~BatchedState() {
         if (gfirst) cudaGraphExecDestroy(gfirst);
         if (gcycle) cudaGraphExecDestroy(gcycle);
@@ -1157,19 +1159,27 @@ static dwf_status bcoarse_solve(BSolver& s, int* citers_out) {
         DWF_TRY(bcapture(s, false, &bs->gcycle));
         bs->gnrhs = s.nrhs;
     }
+    // As many restart cycles as the last solve took are launched before the host looks: a check costs about 25 us
+    // (the copy, the wait and the next launch), and a cycle past the end about as much (every kernel of it
+    // returns at once), while consecutive solves take 3 or 4 cycles each: 256^2 x 16 gradient step 522 -> 494 ms.
     int* hcd = bs->hflags + 2 * bs->cap;
     int launched = 0;
     for (;;) {
-        DWF_CHECK_CUDA(cudaGraphLaunch(launched == 0 ? bs->gfirst : bs->gcycle, s.st));
-        launched += h->prm.coarse_restart;
+        const int n = launched == 0 ? bs->cycles : 1;
+        for (int i = 0; i < n && (launched == 0 || launched < h->prm.coarse_maxiter); ++i) {
+            DWF_CHECK_CUDA(cudaGraphLaunch(launched == 0 ? bs->gfirst : bs->gcycle, s.st));
+            launched += h->prm.coarse_restart;
+        }
         DWF_CHECK_CUDA(cudaMemcpyAsync(hcd, v.cdone, s.nrhs * sizeof(int), cudaMemcpyDeviceToHost, s.st));
+        DWF_CHECK_CUDA(cudaMemcpyAsync(citers_out, v.citers, s.nrhs * sizeof(int), cudaMemcpyDeviceToHost, s.st));
         DWF_CHECK_CUDA(cudaStreamSynchronize(s.st));
         bool all = true;
         for (int r = 0; r < s.nrhs; ++r) all = all && hcd[r];
         if (all || launched >= h->prm.coarse_maxiter) break;
     }
-    DWF_CHECK_CUDA(cudaMemcpyAsync(citers_out, v.citers, s.nrhs * sizeof(int), cudaMemcpyDeviceToHost, s.st));
-    DWF_CHECK_CUDA(cudaStreamSynchronize(s.st));
+    int most = 1;
+    for (int r = 0; r < s.nrhs; ++r) most = std::max(most, citers_out[r]);
+    bs->cycles = (most + h->prm.coarse_restart - 1) / h->prm.coarse_restart;
     return DWF_OK;
 }
 
