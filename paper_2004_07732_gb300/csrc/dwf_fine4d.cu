@@ -131,13 +131,12 @@ template <> __device__ __forceinline__ float param_cast<float>(double, float f) 
 
 // Block: 32 consecutive sites x 8 slices.  Blocks are numbered slice group
 // fastest, so the slice groups of one set of sites run together and share its
-// links and boundary slices in L2.  The block first finds the 8 neighbours of its sites, one
-// thread each.  Bound by L1 (a spinor piece touches 24 lines per warp) and FP32 issue; FP64 by the
-// FP64 pipe.  16^3 x 32 x 16, FP16 links: 173 us against 222 us with 16-byte pieces, products
-// and sums apart and the index divisions in every thread; 12^3 x 24 x 12 in FP64, at the 128
-// registers its values need, 834 against 1159 us.  (The block's links staged in shared memory:
-// 191 us, 226 us for the adjoint, whose registers then spill.)
-constexpr int NB_CROSS = 1 << 30;         // the hop crosses a boundary (sites are below 2^28)
+// links and boundary slices in L2.  Bound by L1 (a spinor piece touches 24 lines per warp) and FP32
+// issue; FP64 by the FP64 pipe.  16^3 x 32 x 16, FP16 links: 162 us against 222 us with 16-byte
+// pieces and products and sums apart; 12^3 x 24 x 12 in FP64, at the 128 registers its values need,
+// 834 against 1159 us.  (One table of neighbours per block in shared memory: 173 us, its barrier
+// costs more than the divisions; the block's links in shared memory too: 191 us, and 226 us for
+// the adjoint, whose registers then spill.)
 template <class LT, class R, bool DAG, bool W32>
 __global__ void __launch_bounds__(256, sizeof(R) == 8 ? 2 : 3) k_dwf4d(const typename LT::store* __restrict__ U,
                                                const typename cplx<R>::T* __restrict__ psi,
@@ -145,29 +144,24 @@ __global__ void __launch_bounds__(256, sizeof(R) == 8 ? 2 : 3) k_dwf4d(const typ
                                                int ngroups, const int* skip) {
     if (skip && *skip) return;
     using C = typename cplx<R>::T;
-    __shared__ int nbs[8][32];
     const int V = (int)p.V;
     const int base = (int)(blockIdx.x / ngroups) * 32;
     const int site = base + threadIdx.x;
     const int s = (int)(blockIdx.x % ngroups) * 8 + threadIdx.y;
-    {
-        // neighbour 2 mu (forward) or 2 mu + 1 (backward); sites past the end take the last site's
-        const int x = min(site, V - 1), mu = threadIdx.y >> 1;
-        const bool fwd = !(threadIdx.y & 1);
-        int stride = 1, rem = x, c = 0, L = 1;
-#pragma unroll
-        for (int nu = 0; nu < 4; ++nu) {
-            const int q = rem / p.L[nu];
-            if (nu == mu) { c = rem - q * p.L[nu]; L = p.L[nu]; }
-            if (nu < mu) stride *= p.L[nu];
-            rem = q;
-        }
-        const bool cross = fwd ? c == L - 1 : c == 0;
-        const int nb = fwd ? (cross ? x - (L - 1) * stride : x + stride) : (cross ? x + (L - 1) * stride : x - stride);
-        nbs[threadIdx.y][threadIdx.x] = nb | (cross ? NB_CROSS : 0);
-    }
-    __syncthreads();
     if (site >= V || s >= p.Ls) return;
+    int stride[4];
+    int coord[4];
+    {
+        int st = 1, rem = site;
+#pragma unroll
+        for (int mu = 0; mu < 4; ++mu) {
+            const int q = rem / p.L[mu];
+            stride[mu] = st;
+            coord[mu] = rem - q * p.L[mu];
+            rem = q;
+            st *= p.L[mu];
+        }
+    }
     C up[2][3], lo[2][3];     // accumulated -1/2 sum of hops, upper / lower spin pairs
 #pragma unroll
     for (int a = 0; a < 2; ++a)
@@ -181,8 +175,11 @@ __global__ void __launch_bounds__(256, sizeof(R) == 8 ? 2 : 3) k_dwf4d(const typ
 #pragma unroll
         for (int dirn = 0; dirn < 2; ++dirn) {
             const bool fwd = dirn == 0;
-            const int nbw = nbs[2 * mu + dirn][threadIdx.x], nb = nbw & (NB_CROSS - 1);
-            const R ph = ((nbw & NB_CROSS) && p.anti[mu]) ? R(-1) : R(1);
+            const int L = p.L[mu];
+            const bool cross = fwd ? (coord[mu] == L - 1) : (coord[mu] == 0);
+            const int nb = fwd ? (cross ? site - (L - 1) * stride[mu] : site + stride[mu])
+                               : (cross ? site + (L - 1) * stride[mu] : site - stride[mu]);
+            const R ph = (cross && p.anti[mu]) ? R(-1) : R(1);
             // projector sign: D uses (1 - gamma) forward, (1 + gamma) backward; D^dag the opposite
             const bool minus = (fwd != DAG);
             C v[4][3];
