@@ -81,8 +81,8 @@ __device__ __forceinline__ double2 cmacc(double2 acc, double2 a, double2 b) {
 // (times 1 or i): p grows in t_f by fused multiply-adds, and the difference is p - 2 t_f.  The
 // FP64 kernel is bound by FP64 issue (ncu: 84% of the pipe), and this takes 40 instructions per
 // site and slice with the diagonal and the s-hops, where separate products, sums and scaling take
-// 48: D_PV^dag D_DW at 250 x 333 x 13 went from 219 to 200 us, at the same error against 64 bits
-// (1.5e-16).  The sums stay trees and the large diagonal term comes last: started from the diagonal
+// 48: D_PV^dag D_DW at 250 x 333 x 13 went from 219 to 200 us (186 with the present walk), at the
+// same error against 64 bits (1.5e-16).  The sums stay trees and the large diagonal term comes last: started from the diagonal
 // term, one chain of multiply-adds has an error of 2.0e-16.
 template <bool DAG>
 __device__ __forceinline__ Sp2<double> hop2d_fused(const Sp2<double>& xf, const Sp2<double>& xb, const Sp2<double>& yf,
@@ -239,10 +239,11 @@ k_dwf2d_multi(const typename LT::store* __restrict__ U, const Sp2<R>* __restrict
     dwf2d_site<LT, R, DAG, 1>(U, psi + off, out + off, p, site, s0, min(s0 + p.s_chunk, p.Ls));
 }
 
-// Threads per block.  A lattice with fewer than a block of 256 for each of the 152 SMs is spread over
-// more of them in blocks of 64: in FP64 one block of 256 keeps its SM's FP64 unit busy for 3 us
-// per slice while others idle (32^2 x 8 in FP64: 7.9 -> 5.4 us a call).
-static int block_threads(long long threads) { return threads < 152LL * 256 ? 64 : 256; }
+// Threads per block.  Fewer threads than 256 for each of the 152 SMs are spread over more SMs in blocks
+// of 64: in FP64 one block of 256 keeps its SM's FP64 unit busy for 3 us per slice while others
+// idle (32^2 x 8 in FP64: 7.9 -> 5.4 us a call).  Otherwise blocks of 128, which end more evenly
+// than ones of 256 (512 x 256 x 16: 17.0 against 18.6 us).
+static int block_threads(long long threads) { return threads < 152LL * 256 ? 64 : 128; }
 
 template <class LT, class R>
 static void launch2d_multi(const void* U, const void* psi, void* out, const Fine2dParams& p, int nrhs,
@@ -321,14 +322,17 @@ static void launch2d(const void* U, const void* psi, void* out, const Fine2dPara
     else        k_dwf2d<LT, R, false, PF><<<grid, threads, 0, st>>>(Ut, pi, po, p);
 }
 
-int choose_s_chunk(long long V, int Ls) {
-    // enough threads to fill 152 SMs x 2048 threads several times over; a
-    // longer chunk keeps more of the s-window reuse (fewer boundary re-reads)
-    const long long target = 152LL * 2048LL * 2LL;
+// Slices per thread.  A longer walk re-reads fewer boundary planes and loads the links less often, a
+// shorter one gives the SMs more threads: the walk is halved until there are 512 threads per SM
+// in FP32 (256^2 x 16, FP16 links: 10.3 us with 8 slices, 12.4 with 2; 512 x 256 x 16: 17.0 with 16,
+// 20.6 with 4) and 2048 in FP64, which is bound by issue and wants its SMs evenly loaded (D_PV^dag
+// D_DW at 250 x 333 x 13: 181 us with 4 slices, 193 with 2, 210 with 1).
+static int choose_s_chunk(long long V, int Ls, bool f64) {
+    const long long target = 152LL * (f64 ? 2048 : 512);
     long long nchunks = (target + V - 1) / V;
     if (nchunks < 1) nchunks = 1;
     if (nchunks > Ls) nchunks = Ls;
-    int chunk = (int)((Ls + nchunks - 1) / nchunks);
+    const int chunk = (int)((Ls + nchunks - 1) / nchunks);
     return chunk < 1 ? 1 : chunk;
 }
 
@@ -356,7 +360,7 @@ dwf_status fine_apply_2d_range(const Geom& g, const void* U, const void* psi, vo
     p.anti1 = g.anti[1];
     p.diag = (double)g.nd - M5 + 1.0;
     p.mf = mf;
-    p.s_chunk = s_chunk > 0 ? s_chunk : choose_s_chunk(g.V, s_hi - s_lo);
+    p.s_chunk = s_chunk > 0 ? s_chunk : choose_s_chunk(g.V, s_hi - s_lo, prec == DWF_F64);
     switch (prec) {
         case DWF_F64:      launch2d<LinkF64, double>(U, psi, out, p, dagger, st); break;
         case DWF_F32:      launch2d<LinkF32, float>(U, psi, out, p, dagger, st); break;
@@ -381,7 +385,7 @@ dwf_status fine_apply_2d_multi(const Geom& g, const void* U, const void* psi, vo
     p.anti1 = g.anti[1];
     p.diag = (double)g.nd - M5 + 1.0;
     p.mf = mf;
-    p.s_chunk = choose_s_chunk(g.V * nrhs, g.Ls);
+    p.s_chunk = choose_s_chunk(g.V * nrhs, g.Ls, prec == DWF_F64);
     p.s_base = 0;
     p.s_end = g.Ls;
     switch (prec) {

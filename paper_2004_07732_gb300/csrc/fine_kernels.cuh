@@ -26,8 +26,6 @@ struct Fine4dParams {
     int s_chunk;
 };
 
-int choose_s_chunk(long long V, int Ls);
-
 // One right-hand side of a batched 2-d apply: its lattice, links and vectors,
 // and the first virtual block of its range (blocks of 256 sites).
 constexpr int BATCH_MAX = 256;
