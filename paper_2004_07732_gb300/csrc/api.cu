@@ -166,6 +166,8 @@ dwf_status dwf_apply_batched(int nrhs, const dwf_geom* geoms, const void* const*
             p.anti0 = G.anti[0]; p.anti1 = G.anti[1];
             p.diag = (double)G.nd - M5 + 1.0;
             p.mf = mf;
+            p.diag_f = (float)p.diag;
+            p.mf_f = (float)mf;
             p.s_chunk = G.Ls;
             p.s_base = 0;
             p.s_end = G.Ls;

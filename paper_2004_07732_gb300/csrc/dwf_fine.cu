@@ -41,7 +41,8 @@ __device__ __forceinline__ typename cplx<R>::T ld_comp(const Sp2<R>* p, long lon
 }
 
 // Wilson hopping term -1/2 sum_mu [ (1 -+ gamma_mu) U psi(x+mu) + (1 +- gamma_mu) U^dag psi(x-mu) ]
-// (upper signs: D_W; lower: D_W^dag = gamma_5 D_W gamma_5).
+// (upper signs: D_W; lower: D_W^dag = gamma_5 D_W gamma_5), for links that come with the -1/2 in
+// them (exact).
 template <class R, bool DAG>
 __device__ __forceinline__ Sp2<R> hop2d(const Sp2<R>& xf, const Sp2<R>& xb, const Sp2<R>& yf, const Sp2<R>& yb,
                                         typename cplx<R>::T u0f, typename cplx<R>::T u0b,
@@ -64,8 +65,8 @@ __device__ __forceinline__ Sp2<R> hop2d(const Sp2<R>& xf, const Sp2<R>& xb, cons
         s1 = (t0f - t0b) + times_i(t1f - t1b);
     }
     Sp2<R> o;
-    o.c0 = scale(s0, R(-0.5));
-    o.c1 = scale(s1, R(-0.5));
+    o.c0 = s0;
+    o.c1 = s1;
     return o;
 }
 
@@ -76,8 +77,7 @@ __device__ __forceinline__ double2 cmacc(double2 acc, double2 a, double2 b) {
     return acc;
 }
 
-// The same in FP64, for links that come with the -1/2 in them (exact).  With t_f, t_b the
-// transported half spinors of a direction, the two components take p = t_f + t_b and t_b - t_f
+// The same in FP64.  With t_f, t_b the transported half spinors of a direction, the two components take p = t_f + t_b and t_b - t_f
 // (times 1 or i): p grows in t_f by fused multiply-adds, and the difference is p - 2 t_f.  The
 // FP64 kernel is bound by FP64 issue (ncu: 84% of the pipe), and this takes 40 instructions per
 // site and slice with the diagonal and the s-hops, where separate products, sums and scaling take
@@ -114,87 +114,71 @@ __device__ __forceinline__ void st_sp_cs(Sp2<double>* p, long long i, const Sp2<
     __stcs(q + 1, s.c1);
 }
 
-// PF = prefetch depth of the s-window: while slice s is computed, the loads of
-// psi_{s+1} .. psi_{s+PF} at this site are already in flight.
+template <class R> __device__ __forceinline__ R param_cast(double d, float f);
+template <> __device__ __forceinline__ double param_cast<double>(double d, float) { return d; }
+template <> __device__ __forceinline__ float param_cast<float>(double, float f) { return f; }
+
 // One site, slices [s0, s1): the body shared by the single-lattice kernel and
-// the batched (many right-hand sides, mixed lattices) kernel.
-template <class LT, class R, bool DAG, int PF>
+// the batched (many right-hand sides, mixed lattices) kernel.  While slice s is computed, the load
+// of psi_{s+2} at this site is in flight and psi_{s+4} on its way to L2.  Every stream has a
+// pointer of its own that moves by a plane: with the addresses formed from slice and site, 152
+// instructions per slice kept the FP32 kernel at 72% issue.  1024^2 x 16, FP16 links: 96.8 us
+// against 98.3 (5.6 TB/s; without the L2 prefetch 112, one plane nearer or two farther 102 and
+// 101); 256^2 x 16 9.4 against 10.3; FP64 D_PV^dag D_DW at 250 x 333 x 13 180 against 186.  UNROLL 2
+// saves the window's moves; the batched kernel is the faster without (151 against 158 us).
+template <class LT, class R, bool DAG, int UNROLL>
 __device__ __forceinline__ void dwf2d_site(const typename LT::store* __restrict__ U, const Sp2<R>* __restrict__ psi,
                                            Sp2<R>* __restrict__ out, const Fine2dParams& p, long long site, int s0,
                                            int s1) {
     using C = typename cplx<R>::T;
     const long long V = p.V;
     const int Lx = p.L0;
-    const int x = (int)(site % Lx);
-    const long long yrow = site - x;  // y * Lx
+    const int x = V <= 0xffffffffLL ? (int)((unsigned)site % (unsigned)Lx) : (int)(site % Lx);
     const int Ls = p.Ls;
 
-    // neighbour sites with periodic wrap
-    const long long xf_site = (x == Lx - 1) ? yrow : site + 1;
-    const long long xb_site = (x == 0) ? yrow + Lx - 1 : site - 1;
-    const long long yf_site = (site + Lx >= V) ? site + Lx - V : site + Lx;
-    const long long yb_site = (site - Lx < 0) ? site - Lx + V : site - Lx;
+    // neighbour sites with periodic wrap, relative to this one
+    const bool xe = x == Lx - 1, xs = x == 0, ye = site + Lx >= V, ys = site - Lx < 0;
+    const long long dxf = xe ? 1 - Lx : 1, dxb = xs ? Lx - 1 : -1;
+    const long long dyf = ye ? Lx - V : Lx, dyb = ys ? V - Lx : -Lx;
 
-    // links, loaded once for all s (antiperiodic boundaries flip the hop sign)
-    C u0f = load_link(U, site);
-    C u1f = load_link(U, V + site);
-    C u0b = load_link(U, xb_site);
-    C u1b = load_link(U, V + yb_site);
-    if (p.anti0) {
-        if (x == Lx - 1) u0f = scale(u0f, R(-1));
-        if (x == 0) u0b = scale(u0b, R(-1));
-    }
-    if (p.anti1) {
-        if (site + Lx >= V) u1f = scale(u1f, R(-1));
-        if (site - Lx < 0) u1b = scale(u1b, R(-1));
-    }
-    constexpr bool FUSED = sizeof(R) == 8;     // hop2d_fused
-    if constexpr (FUSED) {
-        u0f = scale(u0f, -0.5); u0b = scale(u0b, -0.5);
-        u1f = scale(u1f, -0.5); u1b = scale(u1b, -0.5);
-    }
-    const R diag = R(p.diag);
-    const R mf = R(p.mf);
+    // links, loaded once for all s, with the hops' -1/2 (antiperiodic boundaries flip the hop sign)
+    const C u0f = scale(load_link(U, site), p.anti0 && xe ? R(0.5) : R(-0.5));
+    const C u1f = scale(load_link(U, V + site), p.anti1 && ye ? R(0.5) : R(-0.5));
+    const C u0b = scale(load_link(U, site + dxb), p.anti0 && xs ? R(0.5) : R(-0.5));
+    const C u1b = scale(load_link(U, V + site + dyb), p.anti1 && ys ? R(0.5) : R(-0.5));
+    const R diag = param_cast<R>(p.diag, p.diag_f);
+    const R mf = param_cast<R>(p.mf, p.mf_f);
     // component fed from below (s-1) and from above (s+1):
     //   D:     out.c0 += psi_{s-1}.c0, out.c1 += psi_{s+1}.c1
     //   D^dag: out.c0 += psi_{s+1}.c0, out.c1 += psi_{s-1}.c1
     const int cb = DAG ? 1 : 0;   // component taken from s-1
     const int ca = DAG ? 0 : 1;   // component taken from s+1
     const int slast = s1 < Ls ? s1 : Ls - 1;   // last plane the window needs
+    const bool lead = (threadIdx.x & (128 / sizeof(Sp2<R>) - 1)) == 0;   // one lane per 128-byte line
 
-    // win[0] = psi_s, win[k] = psi_{s+k} (loads in flight)
-    Sp2<R> win[PF + 1];
-#pragma unroll
-    for (int k = 0; k <= PF; ++k)
-        if (s0 + k <= slast) win[k] = ld_sp(psi, (long long)(s0 + k) * V + site);
-    C below = (s0 > 0) ? ld_comp(psi, (long long)(s0 - 1) * V + site, cb)
-                       : scale(ld_comp(psi, (long long)(Ls - 1) * V + site, cb), -mf);
-    C wall0 = (s0 == 0) ? (ca == 0 ? win[0].c0 : win[0].c1) : C();
+    const Sp2<R>* pc = psi + ((long long)s0 * V + site);
+    Sp2<R> cur = ld_sp(pc, 0), next = cur;
+    if (s0 + 1 <= slast) next = ld_sp(pc + V, 0);
+    C below = (s0 > 0) ? ld_comp(pc - V, 0, cb) : scale(ld_comp(psi, (long long)(Ls - 1) * V + site, cb), -mf);
+    const C wall0 = (s0 == 0) ? (ca == 0 ? cur.c0 : cur.c1) : C();
+    const Sp2<R>*pxf = pc + dxf, *pxb = pc + dxb, *pyf = pc + dyf, *pyb = pc + dyb, *pn = pc + 2 * V;
+    Sp2<R>* po = out + ((long long)s0 * V + site);
 
+#pragma unroll UNROLL
     for (int s = s0; s < s1; ++s) {
-        const long long base = (long long)s * V;
+        const Sp2<R> nb_xf = ld_sp(pxf, 0), nb_xb = ld_sp(pxb, 0), nb_yf = ld_sp(pyf, 0), nb_yb = ld_sp(pyb, 0);
         C above;
         if (s + 1 < Ls) {
-            above = (ca == 0) ? win[1].c0 : win[1].c1;
+            above = (ca == 0) ? next.c0 : next.c1;
         } else {
-            C w = (s0 == 0) ? wall0 : ld_comp(psi, site, ca);
+            const C w = (s0 == 0) ? wall0 : ld_comp(psi, site, ca);
             above = scale(w, -mf);
         }
-        Sp2<R> nb_xf = ld_sp(psi, base + xf_site);
-        Sp2<R> nb_xb = ld_sp(psi, base + xb_site);
-        Sp2<R> nb_yf = ld_sp(psi, base + yf_site);
-        Sp2<R> nb_yb = ld_sp(psi, base + yb_site);
-        const Sp2<R> cur = win[0];
-        // advance the window and start the load of psi_{s+PF+1}
-#pragma unroll
-        for (int k = 0; k < PF; ++k) win[k] = win[k + 1];
-        if (s + PF + 1 <= slast) win[PF] = ld_sp(psi, (long long)(s + PF + 1) * V + site);
-        // L2 prefetch two planes beyond the window, one lane per 128-byte line:
-        // more bytes in flight without the registers of a deeper window
-        if (s + PF + 3 <= slast && (threadIdx.x & (128 / sizeof(Sp2<R>) - 1)) == 0)
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(psi + (long long)(s + PF + 3) * V + site));
+        Sp2<R> over = next;
+        if (s + 2 <= slast) over = ld_sp(pn, 0);
+        if (lead && s + 4 <= slast) asm volatile("prefetch.global.L2 [%0];" ::"l"(pn + 2 * V));
         Sp2<R> o;
-        if constexpr (FUSED) {
+        if constexpr (sizeof(R) == 8) {
             o = hop2d_fused<DAG>(nb_xf, nb_xb, nb_yf, nb_yb, u0f, u0b, u1f, u1b);
             const C in0 = cb == 0 ? below : above, in1 = cb == 0 ? above : below;
             o.c0.x = fma(diag, cur.c0.x, o.c0.x) + in0.x; o.c0.y = fma(diag, cur.c0.y, o.c0.y) + in0.y;
@@ -206,27 +190,31 @@ __device__ __forceinline__ void dwf2d_site(const typename LT::store* __restrict_
             if (cb == 0) { o.c0 = o.c0 + below; o.c1 = o.c1 + above; }
             else         { o.c1 = o.c1 + below; o.c0 = o.c0 + above; }
         }
-        st_sp_cs(out, base + site, o);
+        st_sp_cs(po, 0, o);
         below = (cb == 0) ? cur.c0 : cur.c1;
+        cur = next;
+        next = over;
+        pxf += V; pxb += V; pyf += V; pyb += V; pn += V; po += V;
     }
 }
 
-template <class LT, class R, bool DAG, int PF>
-__global__ void __launch_bounds__(256)
+constexpr int BLOCK_MAX = 128;             // threads per block of k_dwf2d and k_dwf2d_multi (block_threads)
+template <class LT, class R, bool DAG>
+__global__ void __launch_bounds__(BLOCK_MAX, sizeof(R) == 8 ? 4 : 8)
 k_dwf2d(const typename LT::store* __restrict__ U, const Sp2<R>* __restrict__ psi, Sp2<R>* __restrict__ out,
         Fine2dParams p) {
     const long long site = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (site >= p.V) return;
     const int s0 = p.s_base + blockIdx.y * p.s_chunk;
     if (s0 >= p.s_end) return;
-    dwf2d_site<LT, R, DAG, PF>(U, psi, out, p, site, s0, min(s0 + p.s_chunk, p.s_end));
+    dwf2d_site<LT, R, DAG, 2>(U, psi, out, p, site, s0, min(s0 + p.s_chunk, p.s_end));
 }
 
 // nrhs right-hand sides on the same lattice and links, stored back to back
 // (stride V * Ls spinors): grid.z walks the right-hand sides; skip[r] != 0
 // (device flags, may be null) leaves right-hand side r untouched.
 template <class LT, class R, bool DAG>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(BLOCK_MAX, sizeof(R) == 8 ? 4 : 8)
 k_dwf2d_multi(const typename LT::store* __restrict__ U, const Sp2<R>* __restrict__ psi, Sp2<R>* __restrict__ out,
               Fine2dParams p, const int* __restrict__ skip) {
     const int r = blockIdx.z;
@@ -236,14 +224,14 @@ k_dwf2d_multi(const typename LT::store* __restrict__ U, const Sp2<R>* __restrict
     const int s0 = blockIdx.y * p.s_chunk;
     if (s0 >= p.Ls) return;
     const long long off = (long long)r * p.V * p.Ls;
-    dwf2d_site<LT, R, DAG, 1>(U, psi + off, out + off, p, site, s0, min(s0 + p.s_chunk, p.Ls));
+    dwf2d_site<LT, R, DAG, 2>(U, psi + off, out + off, p, site, s0, min(s0 + p.s_chunk, p.Ls));
 }
 
 // Threads per block.  Fewer threads than 256 for each of the 152 SMs are spread over more SMs in blocks
 // of 64: in FP64 one block of 256 keeps its SM's FP64 unit busy for 3 us per slice while others
 // idle (32^2 x 8 in FP64: 7.9 -> 5.4 us a call).  Otherwise blocks of 128, which end more evenly
 // than ones of 256 (512 x 256 x 16: 17.0 against 18.6 us).
-static int block_threads(long long threads) { return threads < 152LL * 256 ? 64 : 128; }
+static int block_threads(long long threads) { return threads < 152LL * 256 ? 64 : BLOCK_MAX; }
 
 template <class LT, class R>
 static void launch2d_multi(const void* U, const void* psi, void* out, const Fine2dParams& p, int nrhs,
@@ -262,7 +250,7 @@ static void launch2d_multi(const void* U, const void* psi, void* out, const Fine
 // block vb of the concatenated block ranges maps to (right-hand side r, block
 // within r) through the descriptors' block offsets (binary search).
 template <class LT, class R, bool DAG>
-__global__ void __launch_bounds__(256, 4)
+__global__ void __launch_bounds__(256, sizeof(R) == 8 ? 2 : 4)
 k_dwf2d_batched(const __grid_constant__ BatchArgs2d a) {
     for (long long vb = blockIdx.x; vb < a.total_blocks; vb += gridDim.x) {
         int lo = 0, hi = a.nrhs - 1;                              // last r with block0 <= vb
@@ -315,11 +303,8 @@ static void launch2d(const void* U, const void* psi, void* out, const Fine2dPara
     auto Ut = reinterpret_cast<const typename LT::store*>(U);
     auto pi = reinterpret_cast<const Sp2<R>*>(psi);
     auto po = reinterpret_cast<Sp2<R>*>(out);
-    // one plane of look-ahead: measured best on GB300 (deeper windows lower the
-    // achieved bandwidth); full-Ls chunks unless the lattice is small
-    constexpr int PF = 1;
-    if (dagger) k_dwf2d<LT, R, true, PF><<<grid, threads, 0, st>>>(Ut, pi, po, p);
-    else        k_dwf2d<LT, R, false, PF><<<grid, threads, 0, st>>>(Ut, pi, po, p);
+    if (dagger) k_dwf2d<LT, R, true><<<grid, threads, 0, st>>>(Ut, pi, po, p);
+    else        k_dwf2d<LT, R, false><<<grid, threads, 0, st>>>(Ut, pi, po, p);
 }
 
 // Slices per thread.  A longer walk re-reads fewer boundary planes and loads the links less often, a
@@ -360,6 +345,8 @@ dwf_status fine_apply_2d_range(const Geom& g, const void* U, const void* psi, vo
     p.anti1 = g.anti[1];
     p.diag = (double)g.nd - M5 + 1.0;
     p.mf = mf;
+    p.diag_f = (float)p.diag;
+    p.mf_f = (float)p.mf;
     p.s_chunk = s_chunk > 0 ? s_chunk : choose_s_chunk(g.V, s_hi - s_lo, prec == DWF_F64);
     switch (prec) {
         case DWF_F64:      launch2d<LinkF64, double>(U, psi, out, p, dagger, st); break;
@@ -385,6 +372,8 @@ dwf_status fine_apply_2d_multi(const Geom& g, const void* U, const void* psi, vo
     p.anti1 = g.anti[1];
     p.diag = (double)g.nd - M5 + 1.0;
     p.mf = mf;
+    p.diag_f = (float)p.diag;
+    p.mf_f = (float)p.mf;
     p.s_chunk = choose_s_chunk(g.V * nrhs, g.Ls, prec == DWF_F64);
     p.s_base = 0;
     p.s_end = g.Ls;

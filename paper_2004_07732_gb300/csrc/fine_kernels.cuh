@@ -11,6 +11,7 @@ struct Fine2dParams {
     int anti0, anti1;
     double diag;   // d - M5 + 1
     double mf;
+    float diag_f, mf_f;   // the same in FP32 for the FP32 kernels
     int s_chunk;
     int s_base, s_end;   // slices [s_base, s_end) written by k_dwf2d (0, Ls for the whole operator)
 };
