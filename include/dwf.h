@@ -342,12 +342,14 @@ typedef struct {
     int coarse_block_prec;/* storage of the Galerkin blocks read by the coarse stencil:
                              DWF_F32 or DWF_F32_L16 (FP16 blocks, FP32 arithmetic; default) */
     int cgs_passes;       /* classical Gram-Schmidt passes per GCR step: 1 (default), or 2
-                             (re-orthogonalised).  With 1, a coarse GCR step takes its
-                             projections, |w'|^2, alpha and the next |r|^2 from one reduction
-                             pass (the orthogonality of the basis and of r to it gives |w'|^2
-                             and the next |r|^2 by Pythagoras) followed by one element-wise
-                             pass; a step whose |w'|^2 falls below 1e-5 |w|^2 ends that
-                             right-hand side's coarse solve                                  */
+                             (re-orthogonalised).  With 1, the coarse GCR and the smoother take
+                             their steps in blocks of up to four: the images of one direction
+                             under increasing powers of the operator, one reduction pass for
+                             the projections, the block's Gram matrix, the alphas and the next
+                             |r|^2 (the orthogonality of the basis and of r to it gives them by
+                             elimination and Pythagoras) and one element-wise pass; a step whose
+                             |w'|^2 falls below 1e-5 |w|^2 ends its block, and as a block's first
+                             step that right-hand side's coarse solve                          */
     int coarse_tc;        /* form of the many-right-hand-side coarse contraction: 0 (default) =
                              autotuned -- the first use for a given nrhs times mma.sync with 1, 2
                              and 4 column tiles per warp and, with FP16 blocks, the tcgen05 forms
@@ -463,8 +465,8 @@ DWF_API dwf_status mg_coarse_apply(const dwf_mg* h, const void* in, void* out, d
 /* The same coarse operator on nrhs right-hand sides at once, on the tensor
  * cores: in / out hold nrhs coarse vectors back to back ([rhs][s][site][dof],
  * complex64).  Per coarse site the stencil is a dense contraction over the
- * nrhs * Ls_c columns, evaluated on the tensor cores with TF32 products of
- * FP32 data split into high and low parts (FP32-level accuracy) and FP32
+ * nrhs * Ls_c columns, evaluated on the tensor cores with TF32 (or scaled
+ * FP16) products of FP32 data split into high and low parts (FP32-level accuracy) and FP32
  * accumulation: tcgen05 (accumulator in tensor memory; the data operand in
  * tensor memory or in shared memory) or mma.sync.  The blocks are the handle's
  * coarse block storage (coarse_block_prec), as for mg_coarse_apply; the

@@ -86,7 +86,7 @@ struct dwf_mg {
     double2* Y64;         // Galerkin blocks [xc][dir][row][col]
     float2* Y32;          // FP32 copy, column-major per block: [xc][dir][col][row]
     float2* Yd32;         // FP32 adjoint blocks Y[x+dir][-dir]^dag, column-major (generic stencil)
-    void* Ytile;          // blocks read by the 2-d tile stencil: Y32, or an FP16 column-major copy
+    void* Ytile;          // blocks read by the 2-d one-vector stencils: Y32, or an FP16 column-major copy
     int ytile_half;       // 1 when Ytile holds FP16 (half2) blocks
     void* Ymma;           // FP16 blocks in tensor-core fragment order (48 dof, FP16 blocks), else nullptr
     int* status;          // device status word of the setup kernels

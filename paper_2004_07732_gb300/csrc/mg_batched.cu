@@ -1084,7 +1084,7 @@ static dwf_status bcoarse_cycle(BSolver& s) {
         for (int i = 0; i < m; ++i) {
             float2* out = i + 1 < m ? v.Zc[k + i + 1] : v.Wc[k + m - 1];
             if (s.nrhs == 1) {
-                // one column: the shared-memory tile stencil has the shorter latency
+                // one column: the one-vector stencil has the shorter latency
                 DWF_TRY(coarse_dwf_apply(h, v.Zc[k + i], v.ct, h->mf, false, v.cdone, s.st));
                 DWF_TRY(coarse_dwf_apply(h, v.ct, out, 1.0, true, v.cdone, s.st));
             } else {
@@ -1399,7 +1399,7 @@ dwf_status mg_solve_batched_impl(dwf_mg* h, int nrhs, const double2* B, double2*
     }
     (void)hit;
     {
-        int st1 = 0;    // bounded bulk-copy waits of the tile stencil (one-column coarse solves)
+        int st1 = 0;    // bounded bulk-copy waits of the one-vector stencils (one-column coarse solves)
         DWF_CHECK_CUDA(cudaMemcpyAsync(&st1, h->status + 1, sizeof(int), cudaMemcpyDeviceToHost, s.st));
         DWF_CHECK_CUDA(cudaStreamSynchronize(s.st));
         if (st1 != 0) {

@@ -163,7 +163,8 @@ __device__ __forceinline__ double warp_site16(const float2* __restrict__ B, cons
 }
 
 // ---------------------------------------------------------------------------
-// 2-d tile kernel (16 coarse dof, Ls_c <= 4).  A block of 8 warps applies the
+// 2-d tiles of the persistent coarse solvers (16 coarse dof, Ls_c <= 4; a single apply is the faster
+// from global memory, k_coarse_w16).  A block of 8 warps applies the
 // operator on a 4 x 2 tile of coarse sites, one warp per site:
 //   * the five 16 x 16 blocks of every site of the tile (10 KB contiguous per
 //     site) are copied into shared memory by one cp.async.bulk per site,
@@ -1333,7 +1334,7 @@ __device__ double pcg_total(const double* partials, int k) {
 }
 
 // out = Dhat_DW(m) in (or adjoint) over all tiles (grid-stride), shared-memory
-// tiles as in k_coarse_tile.  `phase` is this block's mbarrier parity, flipped
+// tiles as described above.  `phase` is this block's mbarrier parity, flipped
 // per tile.  Returns this thread's share of |out|^2; false in *ok on a timeout.
 __device__ double pcg_apply(const PcgArgs& a, TileSmemT<float2>& sm, unsigned& phase, const float2* __restrict__ in,
                             float2* __restrict__ out, double mf, bool dag, bool* ok) {

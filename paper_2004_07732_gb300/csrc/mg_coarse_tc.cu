@@ -18,7 +18,8 @@
 // With FP16 blocks the contraction also has tcgen05 forms (accumulators in
 // tensor memory): k_coarse_umma and k_coarse_umma_p keep both operands in
 // shared memory (from 128 columns), k_coarse_umma_t keeps the data operand in
-// tensor memory (from 64 columns).  The autotuner (coarse_tc = 0) times the
+// tensor memory (from 64 columns); and k_coarse_f16 takes the data as scaled
+// FP16 high and low parts on mma.sync.m16n8k16.  The autotuner (coarse_tc = 0) times the
 // eligible forms on first use and keeps the fastest; coarse_tc 1-6 fix one.
 #include <cuda.h>
 #include <cudaTypedefs.h>
