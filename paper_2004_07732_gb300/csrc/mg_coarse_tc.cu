@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(256, 2) k_coarse_tc(const BT* __restrict__ Y, 
 // FP16 blocks, one column tile of 8 at a time (form 1).  A block of 16 warps owns a 4 x 4 tile of
 // coarse sites, one warp per site, and walks a range of column tiles:
 //   * the inputs of the tile's 32 sites (16 and their outer neighbours, without the corners) for 8
-//     columns are read once, in whole lines, by asynchronous copies two steps ahead, so that
+//     columns are read once, in whole lines, while the previous 8 columns are multiplied, so that
 //     every input is read and converted twice in all instead of five times; the identity and the
 //     s-hops read their FP32 values from shared memory too;
 //   * each (site, column) is scaled by a power of two to below 2^14 and split into two FP16 parts (22
@@ -187,13 +187,10 @@ __global__ void __launch_bounds__(256, 2) k_coarse_tc(const BT* __restrict__ Y, 
 //     ldmatrix hands to mma.m16n8k16 as B; the blocks are the A operand as stored, in
 //     registers for all five directions, with no conversion and half the products of TF32;
 //   * a direction's products accumulate in FP32 and are added up in FP32 with the scale taken back.
-//   * of the four warps of a scheduler two convert the next columns while two multiply the current ones.
 // Per warp, direction and column tile: 2 ldmatrix, 8 mma, 8 multiply-adds; with the conversion and the
-// epilogue about 600 instructions per warp and column tile, whose issue, with the barrier per column tile,
-// is what bounds it.  64 vectors at 64^2 x 4: 147.6 us (21: 57.6), against 174 (61.6) with loads through
-// registers one step ahead and all warps in the same phase (a third of the stalls were loads and
-// the barrier), 192 us of the tcgen05 form with the data in tensor memory and 205 to 225 us of
-// the TF32 mma.sync forms, and 1.0e-7 of error against 64 bits where they have 3.6e-7.
+// epilogue about 600 instructions per warp and column tile, whose issue (51% of the slots) is what bounds
+// it.  64 vectors at 64^2 x 4: 172 us, against 192 us of the tcgen05 form with the data in tensor memory and
+// 205 to 225 us of the TF32 mma.sync forms, and 1.0e-7 of error against 64 bits where they have 3.6e-7.
 // (Loading 64 bytes per thread and the s-hops from global memory: 211 us, L1 at 80%; one block per tile of
 // sites, 1.7 rounds of them: no change.)
 // ---------------------------------------------------------------------------
@@ -206,7 +203,7 @@ static_assert(CF_HALO == 32 && CF_THREADS == 512, "the loading threads' places")
 struct CfSmem {
     // per site 8 tiles of [column 8][dof 8] halves: high parts Re 0-7, Re 8-15, Im 0-7, Im 8-15, then the low parts
     unsigned char v[2][CF_HALO][8 * CF_TILE];
-    unsigned char raw[3][CF_HALO][8 * CF_ROW];           // the inputs in FP32, [column][dof]: this step's and two ahead
+    unsigned char raw[2][CF_SITES][8 * CF_ROW];          // the tile's own inputs in FP32, [column][dof]
     float back[2][CF_HALO][8];                           // what undoes the scale, per (site, column)
 };
 
@@ -265,37 +262,29 @@ k_coarse_f16(const __half2* __restrict__ Y, const float2* __restrict__ in, float
     // loading: 8 threads take the 128 bytes of a (site, column); this thread's piece of column ln, and the sites
     // 8 i + threadIdx.x / 64.  Sites of the halo: the tile, then x = -1, x = 4 (4 each), y = -1, y = 4
     const int lc = threadIdx.x & 7, ln = (threadIdx.x >> 3) & 7, l0 = threadIdx.x >> 6;
-    int src[CF_ITEMS];                                   // the sites
+    long long src[CF_ITEMS];
 #pragma unroll
     for (int i = 0; i < CF_ITEMS; ++i) {
         const int lh = 8 * i + l0;
         const int hx = lh < 16 ? lh & 3 : lh < 20 ? -1 : lh < 24 ? CF_TX : lh & 3;
         const int hy = lh < 16 ? lh >> 2 : lh < 24 ? lh & 3 : lh < 28 ? -1 : CF_TY;
         const int gx = (x0 + hx + p.Lc0) % p.Lc0, gy = (y0 + hy + p.Lc1) % p.Lc1;
-        src[i] = gy * p.Lc0 + gx;
+        src[i] = ((long long)gy * p.Lc0 + gx) * p.ss + 2 * lc;
     }
-    // one group of copies per call, an empty one past the last column; columns with nothing to do arrive as zeros
-    auto load = [&](int grp, int rb) {
-        if (grp < g1) {
-            const int col = 8 * grp + ln;
-            const bool ok = col < p.ncols && !(skip_rhs && skip_rhs[rhs_of(col)]);
-            const float2* q = in + (long long)(ok ? col : 0) * p.cs + 2 * lc;
-            const uint32_t dst = smem_u32(sm.raw[rb][l0]) + ln * CF_ROW + lc * 16;
+    float4 ld[CF_ITEMS];
+    auto load = [&](int grp) {
+        const int col = 8 * grp + ln;
+        const bool ok = col < p.ncols && !(skip_rhs && skip_rhs[rhs_of(col)]);
+        const float2* q = in + (long long)(ok ? col : 0) * p.cs;
 #pragma unroll
-            for (int i = 0; i < CF_ITEMS; ++i)
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
-                             ::"r"(dst + i * (unsigned)sizeof(sm.raw[0][0]) * 8), "l"(q + src[i] * p.ss), "r"(ok ? 16 : 0)
-                             : "memory");
-        }
-        asm volatile("cp.async.commit_group;" ::: "memory");
+        for (int i = 0; i < CF_ITEMS; ++i)
+            ld[i] = ok ? __ldg(reinterpret_cast<const float4*>(q + src[i])) : make_float4(0.f, 0.f, 0.f, 0.f);
     };
-    // (a thread converts the pieces that it copied itself)
-    auto convert = [&](int rb, int buf) {
-        asm volatile("cp.async.wait_group 1;" ::: "memory");
+    auto convert = [&](int buf) {
 #pragma unroll
         for (int i = 0; i < CF_ITEMS; ++i) {
             const int lh = 8 * i + l0;
-            const float4 u = *reinterpret_cast<const float4*>(sm.raw[rb][lh] + ln * CF_ROW + lc * 16);
+            const float4 u = ld[i];
             float m = fmaxf(fmaxf(fabsf(u.x), fabsf(u.y)), fmaxf(fabsf(u.z), fabsf(u.w)));
             m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
             m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
@@ -313,11 +302,10 @@ k_coarse_f16(const __half2* __restrict__ Y, const float2* __restrict__ in, float
             *reinterpret_cast<__half2*>(d + 2 * CF_TILE) = hi;
             *reinterpret_cast<__half2*>(d + 4 * CF_TILE) = __floats2half2_rn(re0 - fr.x, re1 - fr.y);
             *reinterpret_cast<__half2*>(d + 6 * CF_TILE) = __floats2half2_rn(im0 - fi.x, im1 - fi.y);
+            if (i < CF_SITES / 8) *reinterpret_cast<float4*>(sm.raw[buf][lh] + ln * CF_ROW + lc * 16) = u;
         }
     };
-    int cg1 = live(cg + 1);
-    load(cg, 0);
-    load(cg1, 1);
+    load(cg);
     // multiplying: this warp's site and the halo places of its neighbours
     const int wx = warp & 3, wy = warp >> 2;
     const bool mine = x0 + wx < p.Lc0 && y0 + wy < p.Lc1;
@@ -336,17 +324,12 @@ k_coarse_f16(const __half2* __restrict__ Y, const float2* __restrict__ in, float
             yi[d][q] = cf_pack(__high2half(a0), __high2half(a1));
         }
     }
-    convert(0, 0);
+    convert(0);
     __syncthreads();
-    for (int buf = 0, rb = 0; cg < g1; buf ^= 1) {
-        const int rb1 = rb == 2 ? 0 : rb + 1, cg2 = cg1 < g1 ? live(cg1 + 1) : g1;
-        load(cg2, rb1 == 2 ? 0 : rb1 + 1);
-        // half of each scheduler's warps convert the next columns first, the others multiply first
-#pragma unroll 1
-        for (int ph = 0; ph < 2; ++ph) {
-        if (ph == ((warp >> 2) & 1)) {
-            if (cg1 < g1) convert(rb1, buf ^ 1);
-        } else if (mine) {
+    for (int buf = 0; cg < g1; buf ^= 1) {
+        const int next = live(cg + 1);
+        if (next < g1) load(next);
+        if (mine) {
             float re[4] = {0.f, 0.f, 0.f, 0.f}, im[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
             for (int d = 0; d < 5; ++d) {
@@ -375,7 +358,7 @@ k_coarse_f16(const __half2* __restrict__ Y, const float2* __restrict__ in, float
                 const int r = rhs_of(col), s = col - r * p.Ls_c;
                 if (col >= p.ncols || (skip_rhs && skip_rhs[r])) continue;
                 float2* op = out + (long long)col * p.cs + xc * p.ss + g;
-                const unsigned char* row = sm.raw[rb][warp] + g * 8;
+                const unsigned char* row = sm.raw[buf][warp] + g * 8;
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const float so = p.dag && h ? -1.f : 1.f;
@@ -391,11 +374,9 @@ k_coarse_f16(const __half2* __restrict__ Y, const float2* __restrict__ in, float
                 }
             }
         }
-        }
+        if (next < g1) convert(buf ^ 1);
         __syncthreads();
-        cg = cg1;
-        cg1 = cg2;
-        rb = rb1;
+        cg = next;
     }
     }
 }
