@@ -199,6 +199,8 @@ def _stream(stream):
 
 
 def _ptr(t):
+    """The address alone: it keeps nothing alive, so a copy made for the call needs a name that
+    lasts until the call returns (a freed block is the next one the caching allocator gives out)."""
     return None if t is None else t.data_ptr()
 
 
@@ -385,7 +387,8 @@ def dwf_dot(x, y, stream=None) -> complex:
         raise ValueError("x and y must match in dtype and size")
     prec = PREC["f64"] if x.dtype == torch.complex128 else PREC["f32"]
     res = (ctypes.c_double * 2)()
-    check(lib().dwf_dot(_ptr(x.contiguous()), _ptr(y.contiguous()), x.numel(), prec, res, _stream(stream)))
+    x, y = x.contiguous(), y.contiguous()
+    check(lib().dwf_dot(_ptr(x), _ptr(y), x.numel(), prec, res, _stream(stream)))
     return complex(res[0], res[1])
 
 
@@ -473,8 +476,9 @@ def links_from_angles(geom, theta, stream=None):
     """complex128 links exp(i theta) computed on the GPU (U(1))."""
     if theta.dtype != torch.float64 or not theta.is_cuda or theta.numel() != link_size(geom):
         raise ValueError("theta must be a CUDA float64 tensor of the link size")
+    theta = theta.contiguous()
     U = torch.empty(theta.numel(), dtype=torch.complex128, device=theta.device)
-    check(lib().dwf_links_from_angles(ctypes.byref(geom), _ptr(theta.contiguous()), _ptr(U), _stream(stream)))
+    check(lib().dwf_links_from_angles(ctypes.byref(geom), _ptr(theta), _ptr(U), _stream(stream)))
     return U
 
 
@@ -574,8 +578,9 @@ def mg_setup(geom, U64, M5, mf, params=None, null_starts=None, stream=None) -> M
     if null_starts is None:
         raise ValueError("null_starts (the Gaussian starts of the near-null relaxation) are required")
     h = ctypes.c_void_p()
-    check(lib().mg_setup(ctypes.byref(geom), _ptr(U64.contiguous()), float(M5), float(mf), ctypes.byref(prm),
-                         _ptr(null_starts.contiguous()), ctypes.byref(h), _stream(stream)))
+    U64, null_starts = U64.contiguous(), null_starts.contiguous()
+    check(lib().mg_setup(ctypes.byref(geom), _ptr(U64), float(M5), float(mf), ctypes.byref(prm), _ptr(null_starts),
+                         ctypes.byref(h), _stream(stream)))
     return Multigrid(h, geom, prm)
 
 
@@ -630,7 +635,8 @@ def mg_check_operator(mg: Multigrid, U64, M5, mf, stream=None):
     """Raise DwfError unless mg was set up for exactly the links U64 (complex128), M5 and mf."""
     if U64.dtype != torch.complex128 or U64.numel() != link_size(mg.geom) or not U64.is_cuda:
         raise ValueError("U64 must be a CUDA complex128 tensor of the link size")
-    check(lib().mg_check_operator(mg.ptr, _ptr(U64.contiguous()), float(M5), float(mf), _stream(stream)))
+    U64 = U64.contiguous()
+    check(lib().mg_check_operator(mg.ptr, _ptr(U64), float(M5), float(mf), _stream(stream)))
 
 
 def mg_destroy(mg: Multigrid):
@@ -738,9 +744,9 @@ def mg_add_level(mg: Multigrid, params=None, null_starts=None, lanczos_start=Non
             setattr(p, k, v)
     if null_starts is None:
         raise ValueError("null_starts are required")
-    check(lib().mg_add_level(mg.ptr, ctypes.byref(p), _ptr(null_starts.contiguous()),
-                             _ptr(lanczos_start.contiguous()) if lanczos_start is not None else None,
-                             _stream(stream)))
+    null_starts = null_starts.contiguous()
+    lanczos_start = None if lanczos_start is None else lanczos_start.contiguous()
+    check(lib().mg_add_level(mg.ptr, ctypes.byref(p), _ptr(null_starts), _ptr(lanczos_start), _stream(stream)))
     cg = Geom()
     ncd = ctypes.c_int()
     check(lib().mg_level_geom(mg.ptr, ctypes.byref(cg), ctypes.byref(ncd)))
