@@ -10,6 +10,7 @@
 
 #include "mg.cuh"
 #include "async_copy.cuh"
+#include "mma_f16.cuh"
 
 namespace dwf {
 
@@ -572,12 +573,14 @@ __global__ void __launch_bounds__(512) k_coarse_site(const BT* __restrict__ B, c
 // Re(Y v) = C[i][Re] - C[48 + i][Im] and Im(Y v) = C[48 + i][Re] + C[i][Im]
 // are sums of its own accumulators.
 //
-// Inputs: a slice's 48 values are scaled by a power of two to below 2^14 and
-// split into two FP16 parts of 11 bits each (22 bits, what a TF32 high / low
-// pair keeps too), so that mma.m16n8k16 takes the blocks as they are stored:
-// half the products of the TF32 form and no conversion of a block.  The
-// products of one direction accumulate in FP32; directions are added up in
-// FP32 with the scale taken back.
+// Inputs: the 24 values of a slice and chirality are scaled by a power of two
+// and split into two FP16 parts (mma_f16.cuh: 22 bits, as a TF32 pair keeps), so
+// that mma.m16n8k16 takes the blocks as they are stored: half the products of
+// the TF32 form and no conversion of a block.  The chiralities are scaled apart
+// because on the slices near a wall they differ by orders of magnitude; the column
+// tiles of 16 that hold both are multiplied as two of 8.  The products of a
+// direction with the parts of a chirality accumulate in FP32, four sums that are
+// added up with their scales taken back, as the directions are.
 //
 // Only the self block and the four forward blocks of a site are stored: the
 // kernel is gamma_5-hermitian, so the backward block of x is
@@ -591,8 +594,9 @@ __global__ void __launch_bounds__(512) k_coarse_site(const BT* __restrict__ B, c
 // Each warp brings the block of direction d + 1 into the other half of its
 // shared-memory ring by one bulk copy while it multiplies that of direction
 // d: 9.2 KB per warp, 12 warps per SM.  Bound by the block bytes (L2 to SM:
-// 83 KB per site; HBM: 46 KB): 33 us at 6^3 x 12 sites x 4 slices and 81 us at 8^3 x 16
-// (8.4 TB/s of block bytes), where nine stored blocks and TF32 products took 44 and 114 us.
+// 83 KB per site; HBM: 46 KB): 35 us at 6^3 x 12 sites x 4 slices and 83 us at 8^3 x 16
+// (8.2 TB/s of block bytes), where nine stored blocks and TF32 products took 44 and 114 us.
+// (One scale per slice, with both parts and chiralities in one sum: 33 and 81 us.)
 // ---------------------------------------------------------------------------
 constexpr int CM_WARPS = 4;
 constexpr int CM_BLOCKS = 5;                             // stored blocks per site: self, +mu
@@ -602,23 +606,6 @@ struct CmSmem {
     unsigned long long bar[2];
     unsigned long long pad[14];                          // the next warp's ring on a 128-byte line
 };
-
-// four 8 x 8 tiles of halves: lane l gives the address of row l % 8 of tile l / 8
-template <bool TRANS>
-__device__ __forceinline__ void ldmatrix4(uint32_t (&a)[4], uint32_t addr) {
-    if (TRANS)
-        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
-                     : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]) : "r"(addr) : "memory");
-    else
-        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-                     : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]) : "r"(addr) : "memory");
-}
-__device__ __forceinline__ void mma_f16(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-                 "{%0,%1,%2,%3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
 
 // This lane's inputs of one direction: column g = 2 s + part, dof 8 j + 2 t and 8 j + 2 t + 1 (j < 6)
 template <bool V4>
@@ -630,30 +617,46 @@ __device__ __forceinline__ void cm_load(float (&v)[6][2], const float2* vin, boo
         v[j][1] = part ? u.w : u.z;
     }
 }
-// B fragments: hi[kt][h] and lo[kt][h] hold dof 16 kt + 8 h + 2 t, + 1; chirality - dof change sign with
-// `neg`.  Returns what undoes the scale of this lane's slice.
-__device__ __forceinline__ float cm_split(uint32_t (&hi)[3][2], uint32_t (&lo)[3][2], const float (&v)[6][2], bool neg) {
-    float m = 0.f;
+// B fragments: hi[j] and lo[j] hold dof 8 j + 2 t, + 1; chirality - dof (j >= 3) change sign with
+// `neg`.  back[c] undoes the scale of chirality c of this lane's slice.
+__device__ __forceinline__ void cm_split(uint32_t (&hi)[6], uint32_t (&lo)[6], const float (&v)[6][2], bool neg,
+                                         float (&back)[2]) {
 #pragma unroll
-    for (int j = 0; j < 6; ++j) m = fmaxf(m, fmaxf(fabsf(v[j][0]), fabsf(v[j][1])));
-    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));    // the slice's values: lanes t, and part
-    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
-    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 4));
-    // 2^(13 - exponent of m): |v| scaled < 2^14; tiny slices are left where 2^113 brings them
-    const int e = max((int)(__float_as_uint(m) >> 23), 27);
-    const float scale = __uint_as_float((unsigned)(127 + 13 + 127 - e) << 23);
-    const float back = __uint_as_float((unsigned)(e - 13) << 23);
+    for (int c = 0; c < 2; ++c) {
+        float m = 0.f;
 #pragma unroll
-    for (int j = 0; j < 6; ++j) {
-        const float sc = neg && j >= 3 ? -scale : scale;
-        const float a = v[j][0] * sc, b = v[j][1] * sc;
-        const __half2 h = __floats2half2_rn(a, b);
-        const float2 f = __half22float2(h);
-        const __half2 l = __floats2half2_rn(a - f.x, b - f.y);
-        hi[j >> 1][j & 1] = *reinterpret_cast<const uint32_t*>(&h);
-        lo[j >> 1][j & 1] = *reinterpret_cast<const uint32_t*>(&l);
+        for (int j = 3 * c; j < 3 * c + 3; ++j) m = fmaxf(m, fmaxf(fabsf(v[j][0]), fabsf(v[j][1])));
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));    // the chirality's values: lanes t, and part
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 4));
+        float scale;
+        f16_scale(m, scale, back[c]);
+        if (neg && c == 1) scale = -scale;
+#pragma unroll
+        for (int j = 3 * c; j < 3 * c + 3; ++j) {
+            __half2 h, l;
+            f16_split(v[j][0] * scale, v[j][1] * scale, h, l);
+            hi[j] = *reinterpret_cast<const uint32_t*>(&h);
+            lo[j] = *reinterpret_cast<const uint32_t*>(&l);
+        }
     }
-    return back;
+}
+// One row tile: C[0], C[1] the products with the high parts of chirality +, -, C[2], C[3] with the low
+// ones; a[kt] holds the columns 16 kt .., of which those from 24 on have chirality -
+__device__ __forceinline__ void cm_products(float (&C)[4][4], const uint32_t (&a)[3][4], const uint32_t (&hi)[6],
+                                            const uint32_t (&lo)[6]) {
+    mma_f16_zero(C[0], a[0][0], a[0][1], a[0][2], a[0][3], hi[0], hi[1]);
+    mma_f16_zero(C[1], a[2][0], a[2][1], a[2][2], a[2][3], hi[4], hi[5]);
+    mma_f16_zero(C[2], a[0][0], a[0][1], a[0][2], a[0][3], lo[0], lo[1]);
+    mma_f16_zero(C[3], a[2][0], a[2][1], a[2][2], a[2][3], lo[4], lo[5]);
+    mma_f16_k8(C[0], a[1][0], a[1][1], hi[2]);
+    mma_f16_k8(C[1], a[1][2], a[1][3], hi[3]);
+    mma_f16_k8(C[2], a[1][0], a[1][1], lo[2]);
+    mma_f16_k8(C[3], a[1][2], a[1][3], lo[3]);
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) C[c][q] = fmaf(F16_LOW, C[2 + c][q], C[c][q]);
 }
 
 template <bool V4>
@@ -699,10 +702,13 @@ __global__ void __launch_bounds__(CM_WARPS * 32, 3) k_coarse_mma(const unsigned 
 #pragma unroll 1
     for (int d = 0; d < STEPS; ++d) {
         const bool fwd = d < CM_BLOCKS;
-        uint32_t hi[3][2], lo[3][2];
+        uint32_t hi[6], lo[6];
+        float back[2];
         // sigma_3 on the inputs: of the adjoint operator, and of a backward block
-        float back = cm_split(hi, lo, v, dag != !fwd);
-        back = __shfl_sync(0xffffffffu, back, 8 * t);    // the scale of slice t, this lane's columns of C
+        cm_split(hi, lo, v, dag != !fwd, back);
+#pragma unroll
+        for (int c = 0; c < 2; ++c)                      // the scale of slice t, this lane's columns of C
+            back[c] = __shfl_sync(0xffffffffu, back[c], 8 * t);
         if (d + 1 < STEPS) cm_load<V4>(v, vb + (long long)neighbour(d + 1) * 48, colv, part);
         if (!__all_sync(0xffffffffu, mbar_wait_bounded(&sm.bar[d & 1], (d >> 1) & 1, TILE_WAIT_NS))) {
             if (lane == 0) atomicExch(status, 2);
@@ -712,53 +718,50 @@ __global__ void __launch_bounds__(CM_WARPS * 32, 3) k_coarse_mma(const unsigned 
             return;
         }
         const uint32_t ring = smem_u32(sm.ring[d & 1]);
-        float C[6][4];
-#pragma unroll
-        for (int m = 0; m < 6; ++m)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) C[m][q] = 0.f;
         if (fwd) {
             // tiles (row 2 m, 2 m + 1) x (column 2 kt, 2 kt + 1)
             const uint32_t base = ring + (i8 * 6 + i16) * 128 + r8 * 16;
 #pragma unroll
-            for (int kt = 0; kt < 3; ++kt) {
-                uint32_t a[6][4];
+            for (int m = 0; m < 3; ++m) {
+                uint32_t a[2][3][4];                     // Re Y, Im Y
+                float C[2][4][4];
 #pragma unroll
-                for (int m = 0; m < 6; ++m) ldmatrix4<false>(a[m], base + (12 * m + 2 * kt) * 128);
+                for (int ri = 0; ri < 2; ++ri)
 #pragma unroll
-                for (int m = 0; m < 6; ++m) mma_f16(C[m], a[m], hi[kt]);
+                    for (int kt = 0; kt < 3; ++kt) ldmatrix4<false>(a[ri][kt], base + (12 * (m + 3 * ri) + 2 * kt) * 128);
+                cm_products(C[0], a[0], hi, lo);
+                cm_products(C[1], a[1], hi, lo);
 #pragma unroll
-                for (int m = 0; m < 6; ++m) mma_f16(C[m], a[m], lo[kt]);
+                for (int c = 0; c < 2; ++c)
+#pragma unroll
+                    for (int q = 0; q < 4; q += 2) {
+                        acc[m][q] = fmaf(back[c], C[0][c][q] - C[1][c][q + 1], acc[m][q]);
+                        acc[m][q + 1] = fmaf(back[c], C[0][c][q + 1] + C[1][c][q], acc[m][q + 1]);
+                    }
             }
-#pragma unroll
-            for (int m = 0; m < 3; ++m)
-#pragma unroll
-                for (int q = 0; q < 4; q += 2) {
-                    acc[m][q] = fmaf(back, C[m][q] - C[m + 3][q + 1], acc[m][q]);
-                    acc[m][q + 1] = fmaf(back, C[m][q + 1] + C[m + 3][q], acc[m][q + 1]);
-                }
         } else {
             // outputs 16 m .. are columns (tiles 2 m, 2 m + 1), inputs 16 kt .. rows (tiles 2 kt, 2 kt + 1) of Re Y and Im Y
             const uint32_t base = ring + (i16 * 6 + i8) * 128 + r8 * 16;
 #pragma unroll
-            for (int kt = 0; kt < 3; ++kt) {
-                uint32_t a[6][4];
+            for (int m = 0; m < 3; ++m) {
+                uint32_t a[2][3][4];
+                float C[2][4][4];
 #pragma unroll
-                for (int m = 0; m < 6; ++m) ldmatrix4<true>(a[m], base + (12 * (kt + (m < 3 ? 0 : 3)) + 2 * (m % 3)) * 128);
+                for (int ri = 0; ri < 2; ++ri)
 #pragma unroll
-                for (int m = 0; m < 6; ++m) mma_f16(C[m], a[m], hi[kt]);
+                    for (int kt = 0; kt < 3; ++kt) ldmatrix4<true>(a[ri][kt], base + (12 * (kt + 3 * ri) + 2 * m) * 128);
+                cm_products(C[0], a[0], hi, lo);
+                cm_products(C[1], a[1], hi, lo);
 #pragma unroll
-                for (int m = 0; m < 6; ++m) mma_f16(C[m], a[m], lo[kt]);
+                for (int c = 0; c < 2; ++c)
+#pragma unroll
+                    for (int q = 0; q < 4; q += 2) {
+                        // conj(Y): Re + Im parts; sigma_3 on outputs 8 (2 m + q / 2) and up
+                        const float sb = 2 * m + q / 2 >= 3 ? -back[c] : back[c];
+                        acc[m][q] = fmaf(sb, C[0][c][q] + C[1][c][q + 1], acc[m][q]);
+                        acc[m][q + 1] = fmaf(sb, C[0][c][q + 1] - C[1][c][q], acc[m][q + 1]);
+                    }
             }
-#pragma unroll
-            for (int m = 0; m < 3; ++m)
-#pragma unroll
-                for (int q = 0; q < 4; q += 2) {
-                    // conj(Y): Re + Im parts; sigma_3 on outputs 8 (2 m + q / 2) and up
-                    const float sb = 2 * m + q / 2 >= 3 ? -back : back;
-                    acc[m][q] = fmaf(sb, C[m][q] + C[m + 3][q + 1], acc[m][q]);
-                    acc[m][q + 1] = fmaf(sb, C[m][q + 1] - C[m + 3][q], acc[m][q + 1]);
-                }
         }
         __syncwarp();                                    // every lane has read this half of the ring
         if (d + 2 < STEPS) issue(d + 2, neighbour(d + 2));
