@@ -28,6 +28,7 @@
 
 #include "mg.cuh"
 #include "async_copy.cuh"
+#include "mma_f16.cuh"
 #include "mma_tf32.cuh"
 
 namespace dwf {
@@ -182,15 +183,19 @@ __global__ void __launch_bounds__(256, 2) k_coarse_tc(const BT* __restrict__ Y, 
 //     columns are read once, in whole lines, while the previous 8 columns are multiplied, so that
 //     every input is read and converted twice in all instead of five times; the identity and the
 //     s-hops read their FP32 values from shared memory too;
-//   * each (site, column) is scaled by a power of two to below 2^14 and split into two FP16 parts (22
-//     bits, what a TF32 high / low pair keeps), in shared memory as the 8 x 8 tiles that
-//     ldmatrix hands to mma.m16n8k16 as B; the blocks are the A operand as stored, in
-//     registers for all five directions, with no conversion and half the products of TF32;
-//   * a direction's products accumulate in FP32 and are added up in FP32 with the scale taken back.
-// Per warp, direction and column tile: 2 ldmatrix, 8 mma, 8 multiply-adds; with the conversion and the
-// epilogue about 600 instructions per warp and column tile, whose issue (51% of the slots) is what bounds
-// it.  64 vectors at 64^2 x 4: 172 us, against 192 us of the tcgen05 form with the data in tensor memory and
-// 205 to 225 us of the TF32 mma.sync forms, and 1.0e-7 of error against 64 bits where they have 3.6e-7.
+//   * the eight values of a (site, column, chirality) are scaled by a power of two and split into two
+//     FP16 parts (mma_f16.cuh: 22 bits, as a TF32 pair keeps), in shared memory as the 8 x 8
+//     tiles that ldmatrix hands to mma.m16n8k16 as B; the blocks are the A operand as stored, in
+//     registers for all five directions, with no conversion and half the products of TF32.  The
+//     real and imaginary parts of one chirality fill the 16 columns of a product, so that each
+//     chirality has its own sum and scale (near a wall they differ by orders of magnitude);
+//   * a direction's products with the parts of a chirality accumulate in FP32 and are added up, with their
+//     scales taken back, by packed multiply-adds.
+// Per warp, direction and column tile: 2 ldmatrix, 8 mma, 16 packed multiply-adds; with the conversion and
+// the epilogue, their issue is what bounds it.  64 vectors at 64^2 x 4: 152 us, against 192 us of the
+// tcgen05 form with the data in tensor memory and 205 to 225 us of the TF32 mma.sync forms, and 6.8e-8 of error
+// against 64 bits where they have 3.6e-7.  (One scale per (site, column) and one sum of all products: 176 us
+// and 1.0e-7.)
 // (Loading 64 bytes per thread and the s-hops from global memory: 211 us, L1 at 80%; one block per tile of
 // sites, 1.7 rounds of them: no change.)
 // ---------------------------------------------------------------------------
@@ -204,26 +209,9 @@ struct CfSmem {
     // per site 8 tiles of [column 8][dof 8] halves: high parts Re 0-7, Re 8-15, Im 0-7, Im 8-15, then the low parts
     unsigned char v[2][CF_HALO][8 * CF_TILE];
     unsigned char raw[2][CF_SITES][8 * CF_ROW];          // the tile's own inputs in FP32, [column][dof]
-    float back[2][CF_HALO][8];                           // what undoes the scale, per (site, column)
+    float back[2][CF_HALO][2][8];                        // what undoes the scale, per (site, chirality, column)
 };
 
-__device__ __forceinline__ void cf_ldmatrix(uint32_t (&a)[4], uint32_t addr) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]) : "r"(addr) : "memory");
-}
-__device__ __forceinline__ void cf_mma(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-                 "{%0,%1,%2,%3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-// c = A b
-__device__ __forceinline__ void cf_mma0(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-                 "{%10,%10,%10,%10};"
-                 : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
-}
 __device__ __forceinline__ uint32_t cf_pack(__half a, __half b) {
     const __half2 h = __halves2half2(a, b);
     return *reinterpret_cast<const uint32_t*>(&h);
@@ -262,23 +250,23 @@ k_coarse_f16(const __half2* __restrict__ Y, const float2* __restrict__ in, float
     // loading: 8 threads take the 128 bytes of a (site, column); this thread's piece of column ln, and the sites
     // 8 i + threadIdx.x / 64.  Sites of the halo: the tile, then x = -1, x = 4 (4 each), y = -1, y = 4
     const int lc = threadIdx.x & 7, ln = (threadIdx.x >> 3) & 7, l0 = threadIdx.x >> 6;
-    long long src[CF_ITEMS];
+    int src[CF_ITEMS];
 #pragma unroll
     for (int i = 0; i < CF_ITEMS; ++i) {
         const int lh = 8 * i + l0;
         const int hx = lh < 16 ? lh & 3 : lh < 20 ? -1 : lh < 24 ? CF_TX : lh & 3;
         const int hy = lh < 16 ? lh >> 2 : lh < 24 ? lh & 3 : lh < 28 ? -1 : CF_TY;
         const int gx = (x0 + hx + p.Lc0) % p.Lc0, gy = (y0 + hy + p.Lc1) % p.Lc1;
-        src[i] = ((long long)gy * p.Lc0 + gx) * p.ss + 2 * lc;
+        src[i] = gy * p.Lc0 + gx;
     }
     float4 ld[CF_ITEMS];
     auto load = [&](int grp) {
         const int col = 8 * grp + ln;
         const bool ok = col < p.ncols && !(skip_rhs && skip_rhs[rhs_of(col)]);
-        const float2* q = in + (long long)(ok ? col : 0) * p.cs;
+        const float2* q = in + (long long)(ok ? col : 0) * p.cs + 2 * lc;
 #pragma unroll
         for (int i = 0; i < CF_ITEMS; ++i)
-            ld[i] = ok ? __ldg(reinterpret_cast<const float4*>(q + src[i])) : make_float4(0.f, 0.f, 0.f, 0.f);
+            ld[i] = ok ? __ldg(reinterpret_cast<const float4*>(q + src[i] * p.ss)) : make_float4(0.f, 0.f, 0.f, 0.f);
     };
     auto convert = [&](int buf) {
 #pragma unroll
@@ -287,21 +275,19 @@ k_coarse_f16(const __half2* __restrict__ Y, const float2* __restrict__ in, float
             const float4 u = ld[i];
             float m = fmaxf(fmaxf(fabsf(u.x), fabsf(u.y)), fmaxf(fabsf(u.z), fabsf(u.w)));
             m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
-            m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
-            m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 4));
-            // 2^(13 - exponent of m); tiny columns are left where 2^113 brings them
-            const int e = max((int)(__float_as_uint(m) >> 23), 27);
-            float scale = __uint_as_float((unsigned)(127 + 13 + 127 - e) << 23);
-            if (lc == 0) sm.back[buf][lh][ln] = __uint_as_float((unsigned)(e - 13) << 23);
+            m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));     // lc 0 .. 3: chirality +, 4 .. 7: -
+            float scale, back;
+            f16_scale(m, scale, back);
+            if ((lc & 3) == 0) sm.back[buf][lh][lc >> 2][ln] = back;
             if (p.dag && lc >= 4) scale = -scale;        // sigma_3 on the chirality - inputs
-            const float re0 = u.x * scale, im0 = u.y * scale, re1 = u.z * scale, im1 = u.w * scale;
-            const __half2 hr = __floats2half2_rn(re0, re1), hi = __floats2half2_rn(im0, im1);
-            const float2 fr = __half22float2(hr), fi = __half22float2(hi);
+            __half2 hr, hi, lr, li;
+            f16_split(u.x * scale, u.z * scale, hr, lr);
+            f16_split(u.y * scale, u.w * scale, hi, li);
             unsigned char* d = sm.v[buf][lh] + (lc >> 2) * CF_TILE + ln * 16 + (lc & 3) * 4;
             *reinterpret_cast<__half2*>(d) = hr;
             *reinterpret_cast<__half2*>(d + 2 * CF_TILE) = hi;
-            *reinterpret_cast<__half2*>(d + 4 * CF_TILE) = __floats2half2_rn(re0 - fr.x, re1 - fr.y);
-            *reinterpret_cast<__half2*>(d + 6 * CF_TILE) = __floats2half2_rn(im0 - fi.x, im1 - fi.y);
+            *reinterpret_cast<__half2*>(d + 4 * CF_TILE) = lr;
+            *reinterpret_cast<__half2*>(d + 6 * CF_TILE) = li;
             if (i < CF_SITES / 8) *reinterpret_cast<float4*>(sm.raw[buf][lh] + ln * CF_ROW + lc * 16) = u;
         }
     };
@@ -330,25 +316,34 @@ k_coarse_f16(const __half2* __restrict__ Y, const float2* __restrict__ in, float
         const int next = live(cg + 1);
         if (next < g1) load(next);
         if (mine) {
-            float re[4] = {0.f, 0.f, 0.f, 0.f}, im[4] = {0.f, 0.f, 0.f, 0.f};
+            // columns 2 t, 2 t + 1 of row g and of row g + 8
+            float2 re[2], im[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) re[h] = im[h] = make_float2(0.f, 0.f);
+            const float2 low = make_float2(F16_LOW, F16_LOW);
 #pragma unroll
             for (int d = 0; d < 5; ++d) {
                 const uint32_t addr = smem_u32(sm.v[buf][place[d]]) + (lane >> 3) * CF_TILE + (lane & 7) * 16;
                 uint32_t bh[4], bl[4];                   // Re 0-7, Re 8-15, Im 0-7, Im 8-15
-                cf_ldmatrix(bh, addr);
-                cf_ldmatrix(bl, addr + 4 * CF_TILE);
-                const float2 sc = *reinterpret_cast<const float2*>(&sm.back[buf][place[d]][2 * t]);
-                const uint32_t ny[4] = {yi[d][0] ^ 0x80008000u, yi[d][1] ^ 0x80008000u, yi[d][2] ^ 0x80008000u,
-                                        yi[d][3] ^ 0x80008000u};
-                float c0[4], c1[4];
-                cf_mma0(c0, yr[d], bh[0], bh[1]); cf_mma0(c1, yi[d], bh[0], bh[1]);
-                cf_mma(c0, ny, bh[2], bh[3]);    cf_mma(c1, yr[d], bh[2], bh[3]);
-                cf_mma(c0, yr[d], bl[0], bl[1]); cf_mma(c1, yi[d], bl[0], bl[1]);
-                cf_mma(c0, ny, bl[2], bl[3]);    cf_mma(c1, yr[d], bl[2], bl[3]);
+                ldmatrix4<false>(bh, addr);
+                ldmatrix4<false>(bl, addr + 4 * CF_TILE);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    re[q] = fmaf(q & 1 ? sc.y : sc.x, c0[q], re[q]);
-                    im[q] = fmaf(q & 1 ? sc.y : sc.x, c1[q], im[q]);
+                for (int c = 0; c < 2; ++c) {
+                    const float2 sc = *reinterpret_cast<const float2*>(&sm.back[buf][place[d]][c][2 * t]);
+                    const uint32_t r0 = yr[d][2 * c], r1 = yr[d][2 * c + 1], i0 = yi[d][2 * c], i1 = yi[d][2 * c + 1];
+                    float h4[4], l4[4];                  // products with the high and the low parts
+                    auto add = [&](float2 (&sum)[2]) {
+#pragma unroll
+                        for (int h = 0; h < 2; ++h)
+                            sum[h] = __ffma2_rn(sc, __ffma2_rn(low, make_float2(l4[2 * h], l4[2 * h + 1]),
+                                                               make_float2(h4[2 * h], h4[2 * h + 1])), sum[h]);
+                    };
+                    mma_f16_zero(h4, i0, i1, r0, r1, bh[c], bh[2 + c]);
+                    mma_f16_zero(l4, i0, i1, r0, r1, bl[c], bl[2 + c]);
+                    add(im);
+                    mma_f16_zero(h4, r0, r1, i0 ^ 0x80008000u, i1 ^ 0x80008000u, bh[c], bh[2 + c]);
+                    mma_f16_zero(l4, r0, r1, i0 ^ 0x80008000u, i1 ^ 0x80008000u, bl[c], bl[2 + c]);
+                    add(re);
                 }
             }
             // lane: rows g and g + 8 of columns 2 t, 2 t + 1; the identity and the chiral hops along s in FP32
@@ -369,8 +364,8 @@ k_coarse_f16(const __half2* __restrict__ Y, const float2* __restrict__ in, float
                     const int hc = r * p.Ls_c + sh - 8 * cg;     // the hop's column in this tile, if it is there
                     const float2 hv = hc >= 0 && hc < 8 ? *reinterpret_cast<const float2*>(row + hc * CF_ROW + 64 * h)
                                                         : __ldg(in + (long long)(col - s + sh) * p.cs + xc * p.ss + g + 8 * h);
-                    op[8 * h] = make_float2(so * re[2 * h + w] + self.x + f * hv.x,
-                                            so * im[2 * h + w] + self.y + f * hv.y);
+                    op[8 * h] = make_float2(so * (w ? re[h].y : re[h].x) + self.x + f * hv.x,
+                                            so * (w ? im[h].y : im[h].x) + self.y + f * hv.y);
                 }
             }
         }

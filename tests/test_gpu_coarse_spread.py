@@ -101,3 +101,35 @@ def test_48dof_spread(dw, kind, small):
         assert np.linalg.norm(want) > 0
         assert np.linalg.norm(got - want) <= TOL * np.linalg.norm(want), (kind, dag)
     h.close()
+
+
+@pytest.mark.parametrize("kind,small", [("within", 2.0 ** -27), ("chirality", 2.0 ** -45)])
+def test_multi_vector_spread(dw, kind, small):
+    """coarse_tc = 2: the many-vector operator on FP16 blocks, one column tile at a time"""
+    cdims, Ls_c, nvec, nrhs, mf = (5, 3), 3, 8, 5, 0.07
+    dims = tuple(4 * c for c in cdims)
+    rng = synth.rng_for(131)
+    U = synth.u1_links(synth.u1_angles(rng, dims, 0.5))
+    V, Vc = int(np.prod(dims)), int(np.prod(cdims))
+    # vector k: both components of the site (x0, x1) = (k % 4, k // 4) of every aggregate
+    x = _coords(dims) % 4
+    place = x[0] + 4 * x[1]
+    starts = np.zeros((nvec, V, 2), complex)
+    for k in range(nvec):
+        starts[k, place == k] = 1.0
+    h = dw.mg_setup(dw.make_geom(dims, 8), _dev(U), 1.0, 0.05, {"setup_maxiter": 0, "Ls_c": Ls_c, "coarse_tc": 2},
+                    _dev(starts))
+    Y = _round16(dw.mg_get_coarse_links(h).cpu().numpy().reshape(Vc, 5, 16, 16))
+    rows = np.r_[0:2, 8:10]                              # sites (0, 0) and (1, 0)
+    large = np.array([6])                                # site (2, 1)
+    assert not Y[:, :, rows][..., large].any() and Y[:, :, rows].any()
+    v = _spread(synth.gaussian_complex(rng, (nrhs, Ls_c, Vc, 16)), kind, large, small)
+    for dag in (False, True):
+        want = _apply(Y, v, _neighbours(cdims), mf, dag)[..., rows]
+        vin = _dev(v, torch.complex64)
+        got = dw.mg_coarse_apply_multi(h, vin, torch.empty_like(vin), nrhs, mf, dag).cpu().numpy()
+        got = got.reshape(v.shape)[..., rows]
+        for r in range(nrhs):
+            assert np.linalg.norm(want[r]) > 0
+            assert np.linalg.norm(got[r] - want[r]) <= TOL * np.linalg.norm(want[r]), (kind, dag, r)
+    h.close()
