@@ -62,7 +62,7 @@ __device__ __forceinline__ float2 block_val(const float2* p) { return __ldg(p); 
 __device__ __forceinline__ float2 block_val(const __half2* p) { return __half22float2(__ldg(p)); }
 
 // BT = float2: FP32 blocks, split into TF32 high and low parts (three products
-// per term).  BT = __half2 (from two column tiles per warp on): FP16 blocks, exact in TF32 (same 11-bit
+// per term).  BT = __half2: FP16 blocks, exact in TF32 (same 11-bit
 // significand), so only the vectors are split (two products per term).
 template <int NT, class BT>
 __global__ void __launch_bounds__(256, 2) k_coarse_tc(const BT* __restrict__ Y, const float2* __restrict__ in,
@@ -1268,8 +1268,12 @@ __global__ void __maxnreg__(128) k_coarse_umma_t(const __half2* __restrict__ Y,
 
 }  // namespace
 
-// forms of the contraction: 1, 2, 4 = mma.sync with that many column tiles per warp; TC_UMMA = tcgen05,
-// one item per CTA; TC_UMMA_P = tcgen05, persistent and warp-specialised
+// forms of the contraction: 1, 2, 4 = mma.sync with that many column tiles per warp (1 with FP16 blocks:
+// k_coarse_f16); TC_ONE_TF32 = one column tile of k_coarse_tc with FP16 blocks, the faster one where few
+// columns leave k_coarse_f16 less than a step per SM (512^2, Ls_c 4: 2 vectors 35 against 43 us;
+// 128^2: 5 vectors 10.9 against 12.4); TC_UMMA = tcgen05, one item per CTA; TC_UMMA_P = tcgen05,
+// persistent and warp-specialised
+constexpr int TC_ONE_TF32 = 3;
 constexpr int TC_UMMA = 0x100;
 constexpr int TC_UMMA_P = 0x101;
 constexpr int TC_UMMA_T = 0x102;
@@ -1394,7 +1398,7 @@ static dwf_status launch_form(const dwf_mg* h, int form, const TcParams& p, cons
         DWF_CHECK_LAUNCH();
         return DWF_OK;
     }
-    const int NT = form;
+    const int NT = form == TC_ONE_TF32 ? 1 : form;
     const long long warps = p.Vc * ((p.ncols + 8 * NT - 1) / (8 * NT));
     const long long blocks = (warps * 32 + 255) / 256;
     if (blocks > 0x7fffffffLL) { set_error("coarse batch too large for one launch"); return DWF_ERR_ARG; }
@@ -1403,7 +1407,7 @@ static dwf_status launch_form(const dwf_mg* h, int form, const TcParams& p, cons
         k_coarse_tc<N, __half2><<<(unsigned)blocks, 256, 0, st>>>((const __half2*)h->Ytile, in, out, p, skip_rhs);   \
     else                                                                                                               \
         k_coarse_tc<N, float2><<<(unsigned)blocks, 256, 0, st>>>(h->Y32, in, out, p, skip_rhs);
-    if (NT == 1) k_coarse_tc<1, float2><<<(unsigned)blocks, 256, 0, st>>>(h->Y32, in, out, p, skip_rhs);
+    if (NT == 1) { DWF_TC_LAUNCH(1) }
     else if (NT == 2) { DWF_TC_LAUNCH(2) }
     else { DWF_TC_LAUNCH(4) }
 #undef DWF_TC_LAUNCH
@@ -1433,8 +1437,9 @@ dwf_status coarse_tc_tune(const dwf_mg* h, int nrhs, const float2* in, float2* o
     if (h->mg.nd != 2 || h->mg.ncd != 16 || nrhs < 1) return DWF_OK;
     if (h->tc_choice.count(tc_key(nrhs, layout))) return DWF_OK;
     const TcParams p = tc_params(h, nrhs, h->mf, false, layout);
-    int forms[6] = {1, 2, 4, 0, 0, 0};
+    int forms[7] = {1, 2, 4};
     int nforms = 3;
+    if (h->ytile_half) forms[nforms++] = TC_ONE_TF32;
     if (umma_eligible(h, p.ncols)) forms[nforms++] = TC_UMMA;
     if (umma_p_eligible(h, p.ncols)) forms[nforms++] = TC_UMMA_P;
     if (umma_t_eligible(h, p.ncols)) forms[nforms++] = TC_UMMA_T;
@@ -1511,7 +1516,8 @@ extern "C" dwf_status mg_coarse_apply_multi(const dwf_mg* h, int nrhs, const voi
 extern "C" int mg_coarse_tc_form_layout(const dwf_mg* h, int nrhs, int layout) {
     if (!h) return 0;
     auto it = h->tc_choice.find(tc_key(nrhs, layout));
-    return it == h->tc_choice.end() ? 0 : it->second;
+    if (it == h->tc_choice.end()) return 0;
+    return it->second == TC_ONE_TF32 ? 1 : it->second;   // one column tile in either arithmetic
 }
 
 extern "C" int mg_coarse_tc_form(const dwf_mg* h, int nrhs) {
