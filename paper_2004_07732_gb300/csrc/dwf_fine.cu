@@ -8,6 +8,8 @@
 // the site are loaded once per s-chunk and reused on every slice (they do not
 // depend on s).  The s-hops P_+ psi_{s-1} and P_- psi_{s+1} are a component
 // select in the chiral basis (gamma_5 diagonal), fused into the same pass.
+#include <algorithm>
+
 #include "common.cuh"
 #include "fine_kernels.cuh"
 
@@ -308,17 +310,27 @@ static void launch2d(const void* U, const void* psi, void* out, const Fine2dPara
 }
 
 // Slices per thread.  A longer walk re-reads fewer boundary planes and loads the links less often, a
-// shorter one gives the SMs more threads: the walk is halved until there are 512 threads per SM
-// in FP32 (256^2 x 16, FP16 links: 10.3 us with 8 slices, 12.4 with 2; 512 x 256 x 16: 17.0 with 16,
-// 20.6 with 4) and 2048 in FP64, which is bound by issue and wants its SMs evenly loaded (D_PV^dag
-// D_DW at 250 x 333 x 13: 181 us with 4 slices, 193 with 2, 210 with 1).
+// shorter one gives the SMs more threads: the walk is split until there are 512 threads per SM
+// in FP32 (256^2 x 16, FP16 links: 8.6 us with 8 slices, 11.4 with 2; 400^2 x 16: 18.5 with 16, 19.1
+// with 4) and 2048 in FP64, which is bound by issue and wants its SMs evenly loaded (D_PV^dag
+// D_DW at 250 x 333 x 13: 181 us with 4 slices, 193 with 2, 210 with 1).  A walk of more than 16
+// slices is as long as the whole call where its blocks come in one round or in a few and a bit more
+// (400^2 x 32: 1250 blocks of which 1216 are resident): it is kept where 768 threads per SM come in one
+// round (256^2 x 64: 26.7 us with 32 slices, 27.6 with 16) or from four rounds on (1024^2 x 32: 181
+// with 32, 189 with 16), else 16 slices are the most (400^2 x 32: 37.1 against 43.0, 280^2 x 128: 60.7
+// against 70.0, 700^2 x 32: 96.6 against 98.5).
+constexpr int WALK_MAX = 16;
 static int choose_s_chunk(long long V, int Ls, bool f64) {
-    const long long target = 152LL * (f64 ? 2048 : 512);
-    long long nchunks = (target + V - 1) / V;
-    if (nchunks < 1) nchunks = 1;
-    if (nchunks > Ls) nchunks = Ls;
-    const int chunk = (int)((Ls + nchunks - 1) / nchunks);
-    return chunk < 1 ? 1 : chunk;
+    auto slices = [&](long long threads) {
+        const long long n = std::min({std::max((threads + V - 1) / V, 1LL), (long long)Ls, 65535LL});   // grid.y
+        return (int)((Ls + n - 1) / n);
+    };
+    const int chunk = slices(152LL * (f64 ? 2048 : 512));
+    if (f64 || chunk <= WALK_MAX) return chunk;
+    const int walk = slices(152LL * 768);
+    const long long blocks = (V + BLOCK_MAX - 1) / BLOCK_MAX * ((Ls + walk - 1) / walk), resident = 152LL * 8;
+    if (blocks <= resident || blocks >= 4 * resident) return walk;
+    return std::max(WALK_MAX, (Ls + 65534) / 65535);
 }
 
 dwf_status fine_apply_2d(const Geom& g, const void* U, const void* psi, void* out, double M5, double mf,
