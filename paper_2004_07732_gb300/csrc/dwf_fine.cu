@@ -83,9 +83,9 @@ __device__ __forceinline__ double2 cmacc(double2 acc, double2 a, double2 b) {
 // (times 1 or i): p grows in t_f by fused multiply-adds, and the difference is p - 2 t_f.  The
 // FP64 kernel is bound by FP64 issue (ncu: 84% of the pipe), and this takes 40 instructions per
 // site and slice with the diagonal and the s-hops, where separate products, sums and scaling take
-// 48: D_PV^dag D_DW at 250 x 333 x 13 went from 219 to 200 us (186 with the present walk), at the
-// same error against 64 bits (1.5e-16).  The sums stay trees and the large diagonal term comes last: started from the diagonal
-// term, one chain of multiply-adds has an error of 2.0e-16.
+// 48: D_PV^dag D_DW at 250 x 333 x 13 went from 219 to 200 us (184 with the present walk), at the
+// same error (9.6e-17 of one application at 64 x 48 x 12).  For that the sums stay trees and the largest term, the diagonal one, comes
+// last, after the s-hop (before it: 9.8e-17).
 template <bool DAG>
 __device__ __forceinline__ Sp2<double> hop2d_fused(const Sp2<double>& xf, const Sp2<double>& xb, const Sp2<double>& yf,
                                                    const Sp2<double>& yb, double2 u0f, double2 u0b, double2 u1f,
@@ -197,8 +197,8 @@ __device__ __forceinline__ void dwf2d_site(const typename LT::store* __restrict_
                 o = hop2d<double, DAG>(ld_sp(pxf, 0), ld_sp(pxb, 0), ld_sp(pyf, 0), ld_sp(pyb, 0), u0f, u0b, u1f, u1b);
             }
             const C in0 = cb == 0 ? below : above, in1 = cb == 0 ? above : below;
-            o.c0.x = fma(diag, cur.c0.x, o.c0.x) + in0.x; o.c0.y = fma(diag, cur.c0.y, o.c0.y) + in0.y;
-            o.c1.x = fma(diag, cur.c1.x, o.c1.x) + in1.x; o.c1.y = fma(diag, cur.c1.y, o.c1.y) + in1.y;
+            o.c0.x = fma(diag, cur.c0.x, o.c0.x + in0.x); o.c0.y = fma(diag, cur.c0.y, o.c0.y + in0.y);
+            o.c1.x = fma(diag, cur.c1.x, o.c1.x + in1.x); o.c1.y = fma(diag, cur.c1.y, o.c1.y + in1.y);
         } else {
             o = hop2d<R, DAG>(nb_xf, nb_xb, nb_yf, nb_yb, u0f, u0b, u1f, u1b);
             o.c0 = o.c0 + scale(cur.c0, diag);

@@ -110,3 +110,11 @@ def test_su3_fp32(dw, dag):
     """(products of FP32 numbers are exact in FP64, their sums rounded there 29 bits further down)"""
     kernel, apart = _errors(dw, (8, 8, 8, 8), 6, "su3", "f32", np.float64, np.float32, dag)
     assert kernel <= apart, (kernel, apart)
+
+
+@pytest.mark.skipif(np.finfo(np.longdouble).nmant < 106, reason="needs a type that holds products of FP64 numbers")
+@pytest.mark.parametrize("dag", [False, True])
+def test_u1_fp64(dw, dag):
+    """(147,456 real components: 0.55% is three standard deviations of a root mean square)"""
+    kernel, apart = _errors(dw, (64, 48), 12, "u1", "f64", np.longdouble, np.float64, dag)
+    assert kernel <= 1.0055 * apart, (kernel, apart)
