@@ -87,7 +87,7 @@ __device__ __forceinline__ void sum_slice_groups(double (&v)[N], double* sh) {
 //   gradient: Re(lam^dag dD x) = Re(conj(G) dU) for any change dU (the backward hop reads
 //     conj(U)): G = -1/2 ph (R + i I);
 //   FORCE: the derivative along theta (dU = i U dtheta): -1/2 ph (U.x I - U.y R).
-// 16 FP64 instructions per (link, slice) and 4 adds of half spinors per side.
+// 10 FP64 instructions per (link, slice) and quantity of R, I, and 4 adds of half spinors per side.
 template <bool FORCE>
 __global__ void __launch_bounds__(LINK_THREADS)
 k_linkgrad_u1_2d(const double2* __restrict__ U, const double2* __restrict__ lam, const double2* __restrict__ x,
@@ -111,9 +111,12 @@ k_linkgrad_u1_2d(const double2* __restrict__ U, const double2* __restrict__ lam,
                 // h = c0 -+ (c1 or -i c1): gamma_1 pairs c0 with c1, gamma_2 with -i c1
                 const double2 p = mu == 0 ? l0 - l1 : l0 + times_i(l1), q = mu == 0 ? y0 - y1 : y0 + times_i(y1);
                 const double2 r = mu == 0 ? m0 + m1 : m0 - times_i(m1), t = mu == 0 ? x0v + x1v : x0v - times_i(x1v);
-                v[2 * mu] += p.x * q.x; v[2 * mu] += p.y * q.y; v[2 * mu] += r.x * t.x; v[2 * mu] += r.y * t.y;
-                v[2 * mu + 1] += p.y * q.x; v[2 * mu + 1] -= p.x * q.y;
-                v[2 * mu + 1] += r.x * t.y; v[2 * mu + 1] -= r.y * t.x;
+                // (a slice's four products first: see link_sum_su3)
+                double re = p.x * q.x, im = p.y * q.x;
+                re = fma(p.y, q.y, re); re = fma(r.x, t.x, re); re = fma(r.y, t.y, re);
+                im = fma(-p.x, q.y, im); im = fma(r.x, t.y, im); im = fma(-r.y, t.x, im);
+                v[2 * mu] += re;
+                v[2 * mu + 1] += im;
             }
         }
     sum_slice_groups<4>(v, link_sh);
@@ -166,18 +169,34 @@ __device__ __forceinline__ void outer_half(const double2 (&a)[6], const double2 
             }
 }
 
+// The thread's slices: 8 products per slice and real number of G.  Runs of LINK_RUN slices are
+// summed by themselves before they are added to the total: one chain of multiply-adds over all slices, whose
+// every product is rounded at the size of the whole sum, has an error of 3.4e-16 at Ls = 12, runs of
+// four slices 2.2e-16 and of two 1.8e-16 (sums of four products and no half spinors: 2.6e-16).  A run costs 18 more
+// FP64 instructions (SU(3) force at 12^3 x 24 x 12: 757 us, 778 and 798 us); the totals live in shared memory,
+// since the registers hold one set of 18.
+constexpr int LINK_RUN = 4;
 template <int MU>
 __device__ __forceinline__ void link_sum_su3(const double2* __restrict__ lam, const double2* __restrict__ x,
-                                             long long V, int Ls, long long site, long long nb, double (&G)[18]) {
-    for (int s = threadIdx.y; s < Ls; s += blockDim.y) {
-        const long long b = (long long)s * V;
-        double2 h[6], k[6];
-        half_spinor<MU, -1>(lam + 12 * (b + site), h);
-        half_spinor<MU, -1>(x + 12 * (b + nb), k);
-        outer_half(h, k, G);
-        half_spinor<MU, 1>(x + 12 * (b + site), h);
-        half_spinor<MU, 1>(lam + 12 * (b + nb), k);
-        outer_half(h, k, G);
+                                             long long V, int Ls, long long site, long long nb, double* total) {
+    const int step = blockDim.y, run = LINK_RUN * step;
+    for (int s0 = threadIdx.y; s0 < Ls; s0 += run) {
+        double G[18];
+#pragma unroll
+        for (int e = 0; e < 18; ++e) G[e] = 0.0;
+#pragma unroll 1
+        for (int s = s0; s < min(Ls, s0 + run); s += step) {
+            const long long b = (long long)s * V;
+            double2 h[6], k[6];
+            half_spinor<MU, -1>(lam + 12 * (b + site), h);
+            half_spinor<MU, -1>(x + 12 * (b + nb), k);
+            outer_half(h, k, G);
+            half_spinor<MU, 1>(x + 12 * (b + site), h);
+            half_spinor<MU, 1>(lam + 12 * (b + nb), k);
+            outer_half(h, k, G);
+        }
+#pragma unroll
+        for (int e = 0; e < 18; ++e) total[e * LINK_THREADS] = s0 == (int)threadIdx.y ? G[e] : total[e * LINK_THREADS] + G[e];
     }
 }
 
@@ -188,7 +207,7 @@ __device__ __forceinline__ void link_sum_su3(const double2* __restrict__ lam, co
 // Re(lam^dag dD x) = tr(H F) under U -> exp(i eps H) U.
 // grid.y = mu, a compile-time constant of each branch, so that gamma_mu is a choice of
 // components and signs: 192 FP64 instructions per (link, slice), 0.66 ms of the FP64 rate at
-// 12^3 x 24 x 12 (the memory floor is 35 us); measured 0.76 ms.  With gamma_mu looked up at run
+// 12^3 x 24 x 12 (the memory floor is 35 us); measured 0.78 ms.  With gamma_mu looked up at run
 // time and all four spins multiplied out the kernel ran 3.20 ms.
 template <bool FORCE>
 __global__ void __launch_bounds__(LINK_THREADS, 4)
@@ -206,21 +225,25 @@ k_linkgrad_su3(const double2* __restrict__ U, const double2* __restrict__ lam, c
     const long long nb = cross ? site - (long long)(Lm - 1) * stride : site + stride;
     const int am = mu == 0 ? anti.x : mu == 1 ? anti.y : mu == 2 ? anti.z : anti.w;
     const double ph = (cross && am) ? 0.5 : -0.5;
-    double G[18];
-#pragma unroll
-    for (int e = 0; e < 18; ++e) G[e] = 0.0;
     if (in) {
+        double* total = link_sh + threadIdx.y * blockDim.x + threadIdx.x;
         switch (mu) {
-            case 0: link_sum_su3<0>(lam, x, V, Ls, site, nb, G); break;
-            case 1: link_sum_su3<1>(lam, x, V, Ls, site, nb, G); break;
-            case 2: link_sum_su3<2>(lam, x, V, Ls, site, nb, G); break;
-            default: link_sum_su3<3>(lam, x, V, Ls, site, nb, G); break;
+            case 0: link_sum_su3<0>(lam, x, V, Ls, site, nb, total); break;
+            case 1: link_sum_su3<1>(lam, x, V, Ls, site, nb, total); break;
+            case 2: link_sum_su3<2>(lam, x, V, Ls, site, nb, total); break;
+            default: link_sum_su3<3>(lam, x, V, Ls, site, nb, total); break;
         }
     }
-    sum_slice_groups<18>(G, link_sh);
+    __syncthreads();
     if (!in || threadIdx.y != 0) return;
+    // the groups' sums in order (every group has a slice: link_slice_groups)
+    double G[18];
 #pragma unroll
-    for (int e = 0; e < 18; ++e) G[e] *= ph;
+    for (int e = 0; e < 18; ++e) {
+        double t = link_sh[e * LINK_THREADS + threadIdx.x];
+        for (int g = 1; g < (int)blockDim.y; ++g) t += link_sh[e * LINK_THREADS + g * blockDim.x + threadIdx.x];
+        G[e] = ph * t;
+    }
     const long long t = mu * V + site;
     double2* o = out + 9 * t;
     if (!FORCE) {
@@ -264,7 +287,8 @@ static dwf_status launch_link(const Geom& G, const void* U, const void* lam, con
     const int sp = link_slice_groups(su3 ? 4 * G.V : G.V, G.Ls);
     const dim3 block(LINK_THREADS / sp, sp);
     const dim3 grid((unsigned)((G.V + block.x - 1) / block.x), su3 ? 4u : 1u);
-    const size_t sh = (size_t)(sp - 1) * (su3 ? 18 : 4) * block.x * sizeof(double);
+    // SU(3): the 18 totals of every thread; U(1): the sums of groups 1 .. sp - 1
+    const size_t sh = (su3 ? 18 * LINK_THREADS : (size_t)(sp - 1) * 4 * block.x) * sizeof(double);
     if (su3)
         k_linkgrad_su3<FORCE><<<grid, block, sh, st>>>((const double2*)U, (const double2*)lam, (const double2*)x,
                                                        (double2*)out, make_int4(G.L[0], G.L[1], G.L[2], G.L[3]), G.V,
