@@ -462,6 +462,15 @@ DWF_API dwf_status mg_coarse_solve(dwf_mg* h, const void* rc, void* ec, double t
 DWF_API dwf_status mg_coarse_apply(const dwf_mg* h, const void* in, void* out, double mf, int dagger,
                                    void* stream);
 
+/* The wide-block stencils (4-d, third level) wait for copies of their blocks,
+ * each wait at most 2 s.  mg_coarse_apply is asynchronous, so a wait that gave
+ * up shows in its result as NaN at the site concerned, and the next call on the handle that
+ * synchronises (mg_solve, mg_solve_batched, mg_solve_groups, mg_coarse_solve,
+ * mg_transfer_oblique) returns DWF_ERR_TIMEOUT, once.  mg_check_wait_timeout is the diagnostic
+ * for that path (compare dwf_check_wait_timeout): it runs a kernel whose wait for a copy that
+ * nothing starts gives up after `seconds` (at most 10) and is recorded on the handle in the same way. */
+DWF_API dwf_status mg_check_wait_timeout(dwf_mg* h, double seconds, void* stream);
+
 /* The same coarse operator on nrhs right-hand sides at once, on the tensor
  * cores: in / out hold nrhs coarse vectors back to back ([rhs][s][site][dof],
  * complex64).  Per coarse site the stencil is a dense contraction over the

@@ -13,7 +13,7 @@ from ._lib import (  # noqa: F401
 from ._lib import (  # noqa: F401
     MgParams, Multigrid, mg_default_params, mg_setup, mg_solve, mg_destroy, mg_get_prolongator,
     mg_get_null_vectors, mg_get_coarse_links, mg_restrict, mg_prolong, mg_coarse_apply, mg_coarse_apply_multi,
-    mg_solve_batched, mg_solve_groups, mg_coarse_tc_form, mg_check_operator,
+    mg_solve_batched, mg_solve_groups, mg_coarse_tc_form, mg_check_operator, mg_check_wait_timeout,
     LevelParams, mg_default_level_params, mg_add_level, mg_level_get, mg_level_apply, mg_level_restrict,
     mg_level_prolong, mg_level_coarsest_solve, mg_level_ritz_values, mg_level_last_iterations, mg_level_deflation_info,
     mg_transfer_colinearity, mg_transfer_oblique, mg_coarse_solve,

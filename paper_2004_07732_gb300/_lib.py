@@ -132,6 +132,7 @@ def _setup_signatures(L):
         "mg_restrict": [_VP, _VP, _VP, _VP],
         "mg_prolong": [_VP, _VP, _VP, _VP],
         "mg_coarse_apply": [_VP, _VP, _VP, _D, _I, _VP],
+        "mg_check_wait_timeout": [_VP, _D, _VP],
         "mg_transfer_colinearity": [_VP, _VP, _VP, _VP],
         "mg_transfer_oblique": [_VP, _VP, _VP, _D, ctypes.POINTER(ctypes.c_int), _VP],
         "mg_coarse_solve": [_VP, _VP, _VP, _D, _I, ctypes.POINTER(ctypes.c_int), _VP],
@@ -694,6 +695,12 @@ def mg_coarse_apply(mg: Multigrid, vin, vout, mf, dagger=False, stream=None):
             raise ValueError("coarse vectors must be complex64 CUDA tensors of the coarse size")
     check(lib().mg_coarse_apply(mg.ptr, _ptr(vin), _ptr(vout), float(mf), int(bool(dagger)), _stream(stream)))
     return vout
+
+
+def mg_check_wait_timeout(mg: Multigrid, seconds=0.05, stream=None):
+    """Let a coarse stencil's bounded wait on this handle expire: the next call on it that
+    synchronises raises DwfError with status ERR_TIMEOUT."""
+    check(lib().mg_check_wait_timeout(mg.ptr, float(seconds), _stream(stream)))
 
 
 COARSE_LAYOUTS = {"slice_major": 0, "site_major": 1}

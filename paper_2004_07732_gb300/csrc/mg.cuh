@@ -118,6 +118,7 @@ dwf_status mg_alloc(dwf_mg* h, void** p, size_t bytes);
 // `skip` (device, may be null): the launch does nothing when *skip != 0.
 dwf_status coarse_dwf_apply(const dwf_mg* h, const float2* in, float2* out, double mf, bool dagger,
                             const int* skip, cudaStream_t st);
+dwf_status coarse_wait_status(const dwf_mg* h, cudaStream_t st);
 dwf_status build_adjoint_blocks(dwf_mg* h, cudaStream_t st);
 // tensor-core coarse stencil on nrhs right-hand sides, vectors in `layout`
 // (DWF_COARSE_SLICE_MAJOR: [rhs][s][site][dof]; DWF_COARSE_SITE_MAJOR:

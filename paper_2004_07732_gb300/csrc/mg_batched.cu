@@ -1398,15 +1398,7 @@ dwf_status mg_solve_batched_impl(dwf_mg* h, int nrhs, const double2* B, double2*
         DWF_CHECK_LAUNCH();
     }
     (void)hit;
-    {
-        int st1 = 0;    // bounded bulk-copy waits of the one-vector stencils (one-column coarse solves)
-        DWF_CHECK_CUDA(cudaMemcpyAsync(&st1, h->status + 1, sizeof(int), cudaMemcpyDeviceToHost, s.st));
-        DWF_CHECK_CUDA(cudaStreamSynchronize(s.st));
-        if (st1 != 0) {
-            set_error("coarse stencil: a bulk copy wait timed out");
-            return DWF_ERR_TIMEOUT;
-        }
-    }
+    DWF_TRY(coarse_wait_status(h, s.st));
     int nconv = 0;
     for (int r = 0; r < nrhs; ++r) nconv += conv[r];
     const double secs = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();

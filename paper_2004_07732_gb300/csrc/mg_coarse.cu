@@ -314,6 +314,35 @@ __device__ __forceinline__ double tile_site(const TileSmemT<BT>& sm, float2* __r
 
 constexpr unsigned long long TILE_WAIT_NS = 2000000000ULL;   // 2 s
 
+__device__ __forceinline__ float2 not_a_number2() {
+    const float q = __int_as_float(0x7fffffff);
+    return make_float2(q, q);
+}
+
+// A bulk-copy wait that nothing will end, which records its expiry as the stencils do
+__global__ void k_coarse_wait_expires(unsigned long long budget_ns, int* status) {
+    __shared__ unsigned long long bar;
+    if (threadIdx.x == 0) {
+        mbar_init(&bar, 1);
+        mbar_expect_tx(&bar, 16);
+    }
+    __syncthreads();
+    if (!mbar_wait_bounded(&bar, 0, budget_ns) && threadIdx.x == 0) atomicExch(status, 2);
+}
+
+// DWF_ERR_TIMEOUT if a coarse stencil on this handle gave up waiting for a copy since the last call of this
+// function, which forgets it: the end of every call that synchronises anyway.
+dwf_status coarse_wait_status(const dwf_mg* h, cudaStream_t st) {
+    int hs = 0;
+    DWF_CHECK_CUDA(cudaMemcpyAsync(&hs, h->status + 1, sizeof(int), cudaMemcpyDeviceToHost, st));
+    DWF_CHECK_CUDA(cudaStreamSynchronize(st));
+    if (hs == 0) return DWF_OK;
+    DWF_CHECK_CUDA(cudaMemsetAsync(h->status + 1, 0, sizeof(int), st));
+    DWF_CHECK_CUDA(cudaStreamSynchronize(st));
+    set_error("coarse stencil: a bulk copy wait timed out");
+    return DWF_ERR_TIMEOUT;
+}
+
 static bool tile_ok(const CoarseParams& p) { return p.nd == 2 && p.ncd == 16 && p.Ls_c <= 4; }
 
 static dwf_status site_init_attributes();
@@ -516,8 +545,10 @@ __global__ void __launch_bounds__(512) k_coarse_site(const BT* __restrict__ B, c
     }
     __syncthreads();
     if (!mbar_wait_bounded(mbar, 0, TILE_WAIT_NS)) {
-        if (threadIdx.x == 0) atomicExch(status, 2);
+        atomicExch(status, 2);
         mbar_wait_bounded(mbar, 0, TILE_WAIT_NS);          // let the copy land before the block exits
+        const int e = threadIdx.x;
+        if (e < ncd * Ls_c) out[e / ncd * slice + xc * ncd + e % ncd] = not_a_number2();
         return;
     }
     const int i = threadIdx.x % ncd, s = threadIdx.x / ncd;
@@ -715,6 +746,7 @@ __global__ void __launch_bounds__(CM_WARPS * 32, 3) k_coarse_mma(const unsigned 
             // let the copies land before the warp exits
             mbar_wait_bounded(&sm.bar[d & 1], (d >> 1) & 1, TILE_WAIT_NS);
             if (d + 1 < STEPS) mbar_wait_bounded(&sm.bar[(d + 1) & 1], ((d + 1) >> 1) & 1, TILE_WAIT_NS);
+            for (int e = lane; e < 48 * Ls_c; e += 32) out[e / 48 * slice + (long long)xc * 48 + e % 48] = not_a_number2();
             return;
         }
         const uint32_t ring = smem_u32(sm.ring[d & 1]);
@@ -1211,6 +1243,15 @@ dwf_status mg_coarse_apply(const dwf_mg* h, const void* in, void* out, double mf
     if (!h || !in || !out) { set_error("NULL argument"); return DWF_ERR_ARG; }
     if (in == out) { set_error("in and out must be distinct buffers"); return DWF_ERR_ARG; }
     return coarse_dwf_apply(h, (const float2*)in, (float2*)out, mf, dagger != 0, nullptr, as_stream(stream));
+}
+
+dwf_status mg_check_wait_timeout(dwf_mg* h, double seconds, void* stream) {
+    clear_error();
+    if (!h) { set_error("NULL argument"); return DWF_ERR_ARG; }
+    if (!(seconds > 0.0) || seconds > 10.0) { set_error("seconds must be in (0, 10]"); return DWF_ERR_ARG; }
+    k_coarse_wait_expires<<<1, 32, 0, as_stream(stream)>>>((unsigned long long)(seconds * 1e9), h->status + 1);
+    DWF_CHECK_LAUNCH();
+    return DWF_OK;
 }
 
 }  // extern "C"

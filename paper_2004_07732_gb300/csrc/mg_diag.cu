@@ -150,7 +150,7 @@ dwf_status coarse_gcr_solve(dwf_mg* h, const float2* rc, float2* ec, double tol,
         }
     }
     if (iters) *iters = it;
-    return DWF_OK;
+    return coarse_wait_status(h, st);
 }
 
 }  // namespace

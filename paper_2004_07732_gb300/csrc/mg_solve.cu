@@ -768,15 +768,8 @@ extern "C" dwf_status mg_solve(dwf_mg* h, const void* b, void* x, double tol, in
             status = DWF_ERR_TIMEOUT;
         }
     }
-    {
-        int st1 = 0;
-        DWF_CHECK_CUDA(cudaMemcpyAsync(&st1, h->status + 1, sizeof(int), cudaMemcpyDeviceToHost, s.st));
-        DWF_CHECK_CUDA(cudaStreamSynchronize(s.st));
-        if (st1 != 0) {
-            set_error("coarse stencil: a bulk copy wait timed out");
-            status = DWF_ERR_TIMEOUT;
-        }
-    }
+    const dwf_status waits = coarse_wait_status(h, s.st);
+    if (waits != DWF_OK) status = waits;
     if (status != DWF_OK && dwf_last_error()[0] == 0)
         set_error("mg_solve stopped after %d outer iterations with true residual %.3e > tol %.3e", outer, res, tol);
     if (stats) {
