@@ -625,9 +625,10 @@ __global__ void __launch_bounds__(512) k_coarse_site(const BT* __restrict__ B, c
 // Each warp brings the block of direction d + 1 into the other half of its
 // shared-memory ring by one bulk copy while it multiplies that of direction
 // d: 9.2 KB per warp, 12 warps per SM.  Bound by the block bytes (L2 to SM:
-// 83 KB per site; HBM: 46 KB): 35 us at 6^3 x 12 sites x 4 slices and 83 us at 8^3 x 16
-// (8.2 TB/s of block bytes), where nine stored blocks and TF32 products took 44 and 114 us.
-// (One scale per slice, with both parts and chiralities in one sum: 33 and 81 us.)
+// 83 KB per site; HBM: 46 KB): 34 us at 6^3 x 12 sites x 4 slices and 82 us at 8^3 x 16
+// (8.3 TB/s of block bytes), where nine stored blocks and TF32 products took 44 and 114 us.
+// (One scale per slice, with both parts and chiralities in one sum: 33 and 81 us.  The
+// inputs of direction d + 1 are split behind the products of d: before them, 37 and 89 us.)
 // ---------------------------------------------------------------------------
 constexpr int CM_WARPS = 4;
 constexpr int CM_BLOCKS = 5;                             // stored blocks per site: self, +mu
@@ -730,17 +731,15 @@ __global__ void __launch_bounds__(CM_WARPS * 32, 3) k_coarse_mma(const unsigned 
     const int r8 = lane & 7, i8 = (lane >> 3) & 1, i16 = lane >> 4;
     float v[6][2];
     cm_load<V4>(v, vb + (long long)xc * 48, colv, part);
+    uint32_t hi[6], lo[6];
+    float back[2];
+    cm_split(hi, lo, v, dag, back);                      // sigma_3 on the inputs: of the adjoint operator
+#pragma unroll
+    for (int c = 0; c < 2; ++c) back[c] = __shfl_sync(0xffffffffu, back[c], 8 * t);
+    cm_load<V4>(v, vb + (long long)neighbour(1) * 48, colv, part);
 #pragma unroll 1
     for (int d = 0; d < STEPS; ++d) {
         const bool fwd = d < CM_BLOCKS;
-        uint32_t hi[6], lo[6];
-        float back[2];
-        // sigma_3 on the inputs: of the adjoint operator, and of a backward block
-        cm_split(hi, lo, v, dag != !fwd, back);
-#pragma unroll
-        for (int c = 0; c < 2; ++c)                      // the scale of slice t, this lane's columns of C
-            back[c] = __shfl_sync(0xffffffffu, back[c], 8 * t);
-        if (d + 1 < STEPS) cm_load<V4>(v, vb + (long long)neighbour(d + 1) * 48, colv, part);
         if (!__all_sync(0xffffffffu, mbar_wait_bounded(&sm.bar[d & 1], (d >> 1) & 1, TILE_WAIT_NS))) {
             if (lane == 0) atomicExch(status, 2);
             // let the copies land before the warp exits
@@ -794,6 +793,13 @@ __global__ void __launch_bounds__(CM_WARPS * 32, 3) k_coarse_mma(const unsigned 
                         acc[m][q + 1] = fmaf(sb, C[0][c][q + 1] - C[1][c][q], acc[m][q + 1]);
                     }
             }
+        }
+        if (d + 1 < STEPS) {
+            // the next direction's inputs; sigma_3 of the adjoint operator and of a backward block
+            cm_split(hi, lo, v, dag != (d + 1 >= CM_BLOCKS), back);
+#pragma unroll
+            for (int c = 0; c < 2; ++c) back[c] = __shfl_sync(0xffffffffu, back[c], 8 * t);
+            if (d + 2 < STEPS) cm_load<V4>(v, vb + (long long)neighbour(d + 2) * 48, colv, part);
         }
         __syncwarp();                                    // every lane has read this half of the ring
         if (d + 2 < STEPS) issue(d + 2, neighbour(d + 2));
