@@ -883,8 +883,8 @@ dwf_status coarse_dwf_apply(const dwf_mg* h, const float2* in, float2* out, doub
         else
             k_coarse_site<float2><<<(unsigned)p.Vc, threads, site_smem_bytes<float2>(p.ndir, p.ncd, p.Ls_c), st>>>(
                 (const float2*)h->Ytile, in, out, p, dagger, skip, h->status + 1);
-    } else if (p.ncd == 16) k_coarse_dwf<16><<<grid, thr, 0, st>>>(B, in, out, p, dagger, skip);
-    else             k_coarse_dwf<0><<<grid, thr, 0, st>>>(B, in, out, p, dagger, skip);
+    } else if (p.ncd == 16 && aligned16(in)) k_coarse_dwf<16><<<grid, thr, 0, st>>>(B, in, out, p, dagger, skip);
+    else k_coarse_dwf<0><<<grid, thr, 0, st>>>(B, in, out, p, dagger, skip);   // also for vectors on an 8-byte boundary
     DWF_CHECK_LAUNCH();
     return DWF_OK;
 }
