@@ -360,7 +360,8 @@ __global__ void __launch_bounds__(256) k_coarse_dwf(const float2* __restrict__ B
     if (skip && *skip) return;
     const long long xc = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (xc >= p.Vc) return;
-    if (NCD == 16 && p.Ls_c <= 4) warp_site16<false>(B, in, out, p, xc, p.mf, dag, threadIdx.x & 31);
+    // (a caller's vector may start on an 8-byte boundary; warp_site16 reads its input 16 bytes at a time)
+    if (NCD == 16 && p.Ls_c <= 4 && (reinterpret_cast<uintptr_t>(in) & 15) == 0) warp_site16<false>(B, in, out, p, xc, p.mf, dag, threadIdx.x & 31);
     else warp_site_apply<NCD, false>(B, in, out, p, xc, p.mf, dag, threadIdx.x & 31);
 }
 
@@ -883,8 +884,8 @@ dwf_status coarse_dwf_apply(const dwf_mg* h, const float2* in, float2* out, doub
         else
             k_coarse_site<float2><<<(unsigned)p.Vc, threads, site_smem_bytes<float2>(p.ndir, p.ncd, p.Ls_c), st>>>(
                 (const float2*)h->Ytile, in, out, p, dagger, skip, h->status + 1);
-    } else if (p.ncd == 16 && aligned16(in)) k_coarse_dwf<16><<<grid, thr, 0, st>>>(B, in, out, p, dagger, skip);
-    else k_coarse_dwf<0><<<grid, thr, 0, st>>>(B, in, out, p, dagger, skip);   // also for vectors on an 8-byte boundary
+    } else if (p.ncd == 16) k_coarse_dwf<16><<<grid, thr, 0, st>>>(B, in, out, p, dagger, skip);
+    else             k_coarse_dwf<0><<<grid, thr, 0, st>>>(B, in, out, p, dagger, skip);
     DWF_CHECK_LAUNCH();
     return DWF_OK;
 }
