@@ -6,6 +6,7 @@
 //     exact adjoint of the stored operator;
 //   * truncated wall restriction / prolongation (Eq. TruncProjectInterpolate).
 // Coarse vectors are [s][coarse site][chirality][vec], complex64.
+#include <algorithm>
 #include <mutex>
 
 #include "mg.cuh"
@@ -1090,7 +1091,7 @@ __device__ __forceinline__ float2 prolong_row(const float2* __restrict__ Pr, con
 // dof): P_- P e_1 onto fine slice 1 and P_+ P e_{Lhat_s} onto slice Ls, with the zeros of the
 // other chirality there; the remaining blocks only store the zeros of the slices in between
 // (all of the output but two slices), as one contiguous range of zero_n complex values from
-// zero_0.  Bulk: no range of zeros, every slice is computed.  V4: the layout allows 16-byte
+// zero_0.  Bulk: no range of zeros, every slice is computed (grid.z: its slices).  V4: the layout allows 16-byte
 // accesses (see prolong_wall).  Bound by the stores: 16.8 MB at 256^2 x 16, 64 MB at
 // 12^3 x 24 x 16; one thread per value with its index divisions took 34 us and 160 us.
 constexpr int PROLONG_ZERO = 16;   // complex values stored per thread of a zero block
@@ -1138,7 +1139,7 @@ k_prolong(const float2* __restrict__ P, const float2* __restrict__ e, float2* __
     const float2* ev = e + agg_of(p, x) * p.ncd + c * p.nvec;
     const float2 zero = make_float2(0.f, 0.f);
     if (p.bulk) {
-        for (int s = 0; s < p.Ls; ++s)
+        for (int s = blockIdx.z; s < p.Ls; s += gridDim.z)
             out[fine_idx(p, s, x, d)] = prolong_row<V4>(Pr, ev + (long long)s * p.Vc * p.ncd, p.nvec);
         return;
     }
@@ -1216,7 +1217,11 @@ dwf_status prolong_wall(const dwf_mg* h, const float2* e_coarse, float2* e_fine,
     const long long zero_0 = ends * plane;
     const long long zero_n = p.bulk || p.Ls <= 2 * ends ? 0 : (p.Ls - 2 * ends) * plane;
     const unsigned zero_blocks = (unsigned)((zero_n + 256 * PROLONG_ZERO - 1) / (256 * PROLONG_ZERO));
-    const dim3 grid(wall_blocks + zero_blocks, (unsigned)nrhs);
+    // bulk: a thread takes all slices, with one set of indexes and prolongator values, where that leaves two blocks per SM (4-d
+    // 8^3 x 16 x 8, 384 blocks: 31.7 us, 36.9 in four parts; 4^4 x 8, 12 blocks: 16.4 us, 6.2 in eight)
+    const long long per_slice = (long long)wall_blocks * nrhs;
+    const long long splits = p.bulk ? std::min<long long>({(152 * 2 + per_slice - 1) / per_slice, p.Ls, 65535}) : 1;
+    const dim3 grid(wall_blocks + zero_blocks, (unsigned)nrhs, (unsigned)splits);
     // 16-byte accesses: prolongator rows, coarse vectors and the zero range start on 16-byte boundaries (dof is
     // even, so plane is) when nvec is even and the caller's vectors are aligned
     if (p.nvec % 2 == 0 && aligned16(e_coarse) && aligned16(e_fine))
