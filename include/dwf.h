@@ -455,8 +455,10 @@ DWF_API dwf_status mg_coarse_solve(dwf_mg* h, const void* rc, void* ec, double t
                                    void* stream);
 
 /* Coarse Dhat_DW(mf) (or its adjoint) of Eq. coarsenDW on complex64 coarse
- * vectors; mf = 1 gives Dhat_PV.  FP32 arithmetic on the handle's coarse block
- * storage (coarse_block_prec: FP16 blocks by default, or the FP32 copy); the
+ * vectors; mf = 1 gives Dhat_PV.  FP32-level arithmetic on the handle's coarse block
+ * storage (coarse_block_prec: FP16 blocks by default, or the FP32 copy): FP32 multiply-adds,
+ * or with 48 dof and FP16 blocks tensor-core products of the inputs split into two FP16 parts
+ * (22 bits) and FP32 sums; the
  * adjoint reads the same blocks through Dhat_W^dag = sigma_3 Dhat_W sigma_3
  * (the generic narrow-block stencil reads pre-transposed FP32 adjoint blocks). */
 DWF_API dwf_status mg_coarse_apply(const dwf_mg* h, const void* in, void* out, double mf, int dagger,

@@ -72,13 +72,6 @@ __device__ __forceinline__ Sp2<R> hop2d(const Sp2<R>& xf, const Sp2<R>& xb, cons
     return o;
 }
 
-// acc + conj(a) * b, every product fused into the running sum
-__device__ __forceinline__ double2 cmacc(double2 acc, double2 a, double2 b) {
-    acc.x = fma(a.x, b.x, acc.x); acc.x = fma(a.y, b.y, acc.x);
-    acc.y = fma(a.x, b.y, acc.y); acc.y = fma(-a.y, b.x, acc.y);
-    return acc;
-}
-
 // The same in FP64.  With t_f, t_b the transported half spinors of a direction, the two components take p = t_f + t_b and t_b - t_f
 // (times 1 or i): p grows in t_f by fused multiply-adds, and the difference is p - 2 t_f.  The
 // FP64 kernel is bound by FP64 issue (ncu: 84% of the pipe), and this takes 40 instructions per
@@ -123,17 +116,13 @@ __device__ __forceinline__ void st_sp_cs(Sp2<double>* p, long long i, const Sp2<
     __stcs(q + 1, s.c1);
 }
 
-template <class R> __device__ __forceinline__ R param_cast(double d, float f);
-template <> __device__ __forceinline__ double param_cast<double>(double d, float) { return d; }
-template <> __device__ __forceinline__ float param_cast<float>(double, float f) { return f; }
-
 // One site, slices [s0, s1): the body shared by the single-lattice kernel and
 // the batched (many right-hand sides, mixed lattices) kernel.  While slice s is computed, the load
 // of psi_{s+2} at this site is in flight and psi_{s+4} on its way to L2.  Every stream has a
 // pointer of its own that moves by a plane: with the addresses formed from slice and site, 152
 // instructions per slice kept the FP32 kernel at 72% issue.  1024^2 x 16, FP16 links: 96.8 us
 // against 98.3 (5.6 TB/s; without the L2 prefetch 112, one plane nearer or two farther 102 and
-// 101); 256^2 x 16 9.4 against 10.3; FP64 D_PV^dag D_DW at 250 x 333 x 13 180 against 186.  UNROLL 2
+// 101); 256^2 x 16 9.4 against 10.3; FP64 D_PV^dag D_DW at 250 x 333 x 13 180 against 186 (184 with the check for infinities).  UNROLL 2
 // saves the window's moves; the batched kernel is the faster without (151 against 158 us).
 template <class LT, class R, bool DAG, int UNROLL>
 __device__ __forceinline__ void dwf2d_site(const typename LT::store* __restrict__ U, const Sp2<R>* __restrict__ psi,

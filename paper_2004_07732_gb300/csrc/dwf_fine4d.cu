@@ -92,18 +92,6 @@ __device__ __forceinline__ void st_spin4(C* p, const C (&v)[4][3]) {
     for (int e = 0; e < 12; e += P32) st_piece(p + e, &v[0][0] + e, W32);
 }
 
-// acc + a b, acc + conj(a) b
-template <class C> __device__ __forceinline__ C cmac(C acc, C a, C b) {
-    acc.x = fma(a.x, b.x, acc.x); acc.x = fma(-a.y, b.y, acc.x);
-    acc.y = fma(a.x, b.y, acc.y); acc.y = fma(a.y, b.x, acc.y);
-    return acc;
-}
-template <class C> __device__ __forceinline__ C cmacc(C acc, C a, C b) {
-    acc.x = fma(a.x, b.x, acc.x); acc.x = fma(a.y, b.y, acc.x);
-    acc.y = fma(a.x, b.y, acc.y); acc.y = fma(-a.y, b.x, acc.y);
-    return acc;
-}
-
 // A psi_low for direction mu (A = -i sigma_1, -i sigma_2, -i sigma_3, 1)
 template <class C>
 __device__ __forceinline__ void apply_A(int mu, const C (&l)[2][3], C (&o)[2][3]) {
@@ -133,10 +121,6 @@ template <class C, class R>
 __device__ __forceinline__ C small_first(C hops, C h, R f, C v, R diag) {
     return mk<C>(fma(diag, v.x, fma(f, h.x, R(-0.5) * hops.x)), fma(diag, v.y, fma(f, h.y, R(-0.5) * hops.y)));
 }
-
-template <class R> __device__ __forceinline__ R param_cast(double d, float f);
-template <> __device__ __forceinline__ double param_cast<double>(double d, float) { return d; }
-template <> __device__ __forceinline__ float param_cast<float>(double, float f) { return f; }
 
 // Block: 32 consecutive sites x 8 slices.  Blocks are numbered slice group
 // fastest, so the slice groups of one set of sites run together and share its

@@ -27,6 +27,23 @@ struct Fine4dParams {
     int s_chunk;
 };
 
+// The parameter in the kernel's precision
+template <class R> __device__ __forceinline__ R param_cast(double d, float f);
+template <> __device__ __forceinline__ double param_cast<double>(double d, float) { return d; }
+template <> __device__ __forceinline__ float param_cast<float>(double, float f) { return f; }
+
+// acc + a b, acc + conj(a) b, every product fused into the running sum
+template <class C> __device__ __forceinline__ C cmac(C acc, C a, C b) {
+    acc.x = fma(a.x, b.x, acc.x); acc.x = fma(-a.y, b.y, acc.x);
+    acc.y = fma(a.x, b.y, acc.y); acc.y = fma(a.y, b.x, acc.y);
+    return acc;
+}
+template <class C> __device__ __forceinline__ C cmacc(C acc, C a, C b) {
+    acc.x = fma(a.x, b.x, acc.x); acc.x = fma(a.y, b.y, acc.x);
+    acc.y = fma(a.x, b.y, acc.y); acc.y = fma(-a.y, b.x, acc.y);
+    return acc;
+}
+
 // One right-hand side of a batched 2-d apply: its lattice, links and vectors,
 // and the first virtual block of its range (blocks of 256 sites).
 constexpr int BATCH_MAX = 256;

@@ -88,8 +88,8 @@ struct dwf_mg {
     float2* Yd32;         // FP32 adjoint blocks Y[x+dir][-dir]^dag, column-major (generic stencil)
     void* Ytile;          // blocks read by the 2-d one-vector stencils: Y32, or an FP16 column-major copy
     int ytile_half;       // 1 when Ytile holds FP16 (half2) blocks
-    void* Ymma;           // FP16 blocks in tensor-core fragment order (48 dof, FP16 blocks), else nullptr
-    int* status;          // device status word of the setup kernels
+    void* Ymma;           // FP16 self and forward blocks as 8 x 8 tiles (k_coarse_mma; 48 dof, FP16 blocks), else nullptr
+    int* status;          // device status words: [0] the setup kernels, [1] expired waits of the coarse stencils
     std::vector<void*> allocs;
     // solver workspace (allocated on first solve)
     bool ws_ready;

@@ -881,7 +881,8 @@ static void carve(const dwf_mg* h, int nrhs, char* base, BView& v, size_t* total
     v.nc = coarse_len(h);
     const size_t F = (size_t)nrhs * v.nf, C = (size_t)nrhs * v.nc;
     v.rA = c.take<float2>(F); v.r = c.take<float2>(F);
-    v.tmp = c.take<float2>(F); v.rs_ = c.take<float2>(F); v.ps = c.take<float2>(F);
+    v.tmp = c.take<float2>(F); v.ps = c.take<float2>(F);
+    v.rs_ = h->prm.cgs_passes == 2 ? c.take<float2>(F) : nullptr;
     for (int k = 0; k < BK_MAX; ++k) {
         v.Z[k] = k < K ? c.take<float2>(F) : nullptr;
         v.W[k] = k < K ? c.take<float2>(F) : nullptr;

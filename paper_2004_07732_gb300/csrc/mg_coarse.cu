@@ -192,7 +192,7 @@ template <class BT> __host__ __device__ constexpr unsigned site_block_bytes() { 
 __device__ __forceinline__ float2 to_f2(float2 a) { return a; }
 __device__ __forceinline__ float2 to_f2(__half2 a) { return __half22float2(a); }
 
-template <bool CG, class BT>
+template <class BT>
 __device__ __forceinline__ void tile_stage(TileSmemT<BT>& sm, const float2* __restrict__ in, const CoarseParams& p,
                                            int x0, int y0) {
     const int L0 = p.Lc[0], L1 = p.Lc[1];
@@ -207,7 +207,7 @@ __device__ __forceinline__ void tile_stage(TileSmemT<BT>& sm, const float2* __re
         gx = (gx % L0 + L0) % L0;
         gy = (gy % L1 + L1) % L1;
         const long long site = (long long)gy * L0 + gx;
-        sm.v[s][hy][hx][j] = CG ? __ldcg(in + s * slice + site * 16 + j) : __ldg(in + s * slice + site * 16 + j);
+        sm.v[s][hy][hx][j] = __ldcg(in + s * slice + site * 16 + j);   // written by other blocks of this launch
     }
 }
 
@@ -1403,7 +1403,7 @@ __device__ double pcg_apply(const PcgArgs& a, TileSmemT<float2>& sm, unsigned& p
         const int x0 = (tile % ntx) * TILE_X, y0 = (tile / ntx) * TILE_Y;
         __syncthreads();                        // previous tile's shared data fully consumed
         tile_issue_blocks(sm, B, p, x0, y0);
-        tile_stage<true, float2>(sm, in, p, x0, y0);
+        tile_stage<float2>(sm, in, p, x0, y0);
         __syncthreads();
         const bool okw = mbar_wait_bounded(&sm.mbar, phase, TILE_WAIT_NS);
         if (__syncthreads_or(!okw)) {                      // the whole block leaves together
