@@ -72,13 +72,13 @@ __device__ __forceinline__ Sp2<R> hop2d(const Sp2<R>& xf, const Sp2<R>& xb, cons
     return o;
 }
 
-// The same in FP64.  With t_f, t_b the transported half spinors of a direction, the two components take p = t_f + t_b and t_b - t_f
-// (times 1 or i): p grows in t_f by fused multiply-adds, and the difference is p - 2 t_f.  The
-// FP64 kernel is bound by FP64 issue (ncu: 84% of the pipe), and this takes 40 instructions per
-// site and slice with the diagonal and the s-hops, where separate products, sums and scaling take
-// 48: D_PV^dag D_DW at 250 x 333 x 13 went from 219 to 200 us (184 with the present walk), at the
-// same error (9.6e-17 of one application at 64 x 48 x 12).  For that the sums stay trees and the largest term, the diagonal one, comes
-// last, after the s-hop (before it: 9.8e-17).
+// The same in FP64.  With t_f, t_b the transported half spinors of a direction, the two components
+// take p = t_f + t_b and t_b - t_f (times 1 or i): p grows in t_f by fused multiply-adds, and the
+// difference is p - 2 t_f.  The FP64 kernel is bound by FP64 issue (ncu: 86% of the pipe), and this
+// takes 40 instructions per site and slice with the diagonal and the s-hops, where separate
+// products, sums and scaling take 48: D_PV^dag D_DW at 250 x 333 x 13 184 us against 219 (with longer
+// walks too), at the same error (9.6e-17 of one application at 64 x 48 x 12).  For that the sums stay
+// trees and the largest term, the diagonal one, comes last, after the s-hop (before it: 9.8e-17).
 template <bool DAG>
 __device__ __forceinline__ Sp2<double> hop2d_fused(const Sp2<double>& xf, const Sp2<double>& xb, const Sp2<double>& yf,
                                                    const Sp2<double>& yb, double2 u0f, double2 u0b, double2 u1f,
@@ -119,10 +119,9 @@ __device__ __forceinline__ void st_sp_cs(Sp2<double>* p, long long i, const Sp2<
 // One site, slices [s0, s1): the body shared by the single-lattice kernel and
 // the batched (many right-hand sides, mixed lattices) kernel.  While slice s is computed, the load
 // of psi_{s+2} at this site is in flight and psi_{s+4} on its way to L2.  Every stream has a
-// pointer of its own that moves by a plane: with the addresses formed from slice and site, 152
-// instructions per slice kept the FP32 kernel at 72% issue.  1024^2 x 16, FP16 links: 96.8 us
-// against 98.3 (5.6 TB/s; without the L2 prefetch 112, one plane nearer or two farther 102 and
-// 101); 256^2 x 16 9.4 against 10.3; FP64 D_PV^dag D_DW at 250 x 333 x 13 180 against 186 (184 with the check for infinities).  UNROLL 2
+// pointer of its own that moves by a plane: addresses formed from slice and site kept the FP32
+// kernel at 72% issue.  Bound by HBM: 1024^2 x 16, FP16 links, 96.6 us (5.6 TB/s) against 98.3 with
+// such addresses; without the L2 prefetch 112, one plane nearer or two farther 102 and 101.  UNROLL 2
 // saves the window's moves; the batched kernel is the faster without (151 against 158 us).
 template <class LT, class R, bool DAG, int UNROLL>
 __device__ __forceinline__ void dwf2d_site(const typename LT::store* __restrict__ U, const Sp2<R>* __restrict__ psi,

@@ -999,10 +999,9 @@ __device__ __forceinline__ int chir_dof(const TransferParams& p, int c, int cd) 
 // cd sums meet in shared memory.  The two chiralities of an aggregate are neighbouring groups,
 // so every site's prolongator is read in one piece.  grid.y = right-hand side (vectors back to
 // back); skip[r]: per right-hand side.  Bound by the read of P (and by launch latency below a
-// few MB): with one thread per output, walking the sites one after the other through the index
-// divisions, 256^2 took 30 us and 12^3 x 24 (nvec 24) 132 us; the two transfers and two coarse
-// applies of a 256^2 hierarchy together went from 96.6 to 51.3 us (and from 42.9 to 35.7 later, with
-// eight sites' loads before the first product and 32-bit offsets).
+// few MB): 256^2 8 us, where one thread per output, walking the sites one after the other
+// through the index divisions, took 30; eight sites' loads before the first product and 32-bit
+// offsets took the two transfers and two coarse applies of that hierarchy from 42.9 to 36 us.
 constexpr int RESTRICT_THREADS = 288;   // both chiralities of one aggregate at 4-d, nvec 24
 constexpr int RESTRICT_TABLE = 2048;    // aggregates up to this many sites keep their offsets in shared memory
 
