@@ -79,6 +79,7 @@ __device__ __forceinline__ Sp2<R> hop2d(const Sp2<R>& xf, const Sp2<R>& xb, cons
 // products, sums and scaling take 48: D_PV^dag D_DW at 250 x 333 x 13 184 us against 219 (with longer
 // walks too), at the same error (9.6e-17 of one application at 64 x 48 x 12).  For that the sums stay
 // trees and the largest term, the diagonal one, comes last, after the s-hop (before it: 9.8e-17).
+// The adjoint's c1 comes with the opposite sign, which rides on the sum with the s-hop.
 template <bool DAG>
 __device__ __forceinline__ Sp2<double> hop2d_fused(const Sp2<double>& xf, const Sp2<double>& xb, const Sp2<double>& yf,
                                                    const Sp2<double>& yb, double2 u0f, double2 u0b, double2 u1f,
@@ -94,7 +95,6 @@ __device__ __forceinline__ Sp2<double> hop2d_fused(const Sp2<double>& xf, const 
     Sp2<double> o;
     o.c0 = p0 + p1;
     o.c1 = m0 + times_i(m1);
-    if (DAG) o.c1 = mk<C>(-o.c1.x, -o.c1.y);
     return o;
 }
 
@@ -183,10 +183,12 @@ __device__ __forceinline__ void dwf2d_site(const typename LT::store* __restrict_
             if (__builtin_expect(not_finite(o), 0)) {
                 asm volatile("" ::: "memory");
                 o = hop2d<double, DAG>(ld_sp(pxf, 0), ld_sp(pxb, 0), ld_sp(pyf, 0), ld_sp(pyb, 0), u0f, u0b, u1f, u1b);
+                if (DAG) o.c1 = scale(o.c1, -1.0);
             }
             const C in0 = cb == 0 ? below : above, in1 = cb == 0 ? above : below;
             o.c0.x = fma(diag, cur.c0.x, o.c0.x + in0.x); o.c0.y = fma(diag, cur.c0.y, o.c0.y + in0.y);
-            o.c1.x = fma(diag, cur.c1.x, o.c1.x + in1.x); o.c1.y = fma(diag, cur.c1.y, o.c1.y + in1.y);
+            o.c1.x = fma(diag, cur.c1.x, DAG ? in1.x - o.c1.x : o.c1.x + in1.x);
+            o.c1.y = fma(diag, cur.c1.y, DAG ? in1.y - o.c1.y : o.c1.y + in1.y);
         } else {
             o = hop2d<R, DAG>(nb_xf, nb_xb, nb_yf, nb_yb, u0f, u0b, u1f, u1b);
             o.c0 = o.c0 + scale(cur.c0, diag);
