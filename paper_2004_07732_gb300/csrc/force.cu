@@ -87,7 +87,9 @@ __device__ __forceinline__ void sum_slice_groups(double (&v)[N], double* sh) {
 //   gradient: Re(lam^dag dD x) = Re(conj(G) dU) for any change dU (the backward hop reads
 //     conj(U)): G = -1/2 ph (R + i I);
 //   FORCE: the derivative along theta (dU = i U dtheta): -1/2 ph (U.x I - U.y R).
-// 10 FP64 instructions per (link, slice) and quantity of R, I, and 4 adds of half spinors per side.
+// 16 FP64 instructions per (link, slice): each of the four products of R and of I has a sum of its
+// own, since one chain of all of them rounds every product at the size of the whole sum (error 1.9e-16 at
+// 300 x 400 x 12).  512^2 x 16: 261 us; 254 with the one chain, 295 with each slice's products summed first.
 template <bool FORCE>
 __global__ void __launch_bounds__(LINK_THREADS)
 k_linkgrad_u1_2d(const double2* __restrict__ U, const double2* __restrict__ lam, const double2* __restrict__ x,
@@ -98,7 +100,7 @@ k_linkgrad_u1_2d(const double2* __restrict__ U, const double2* __restrict__ lam,
     const int x0 = (int)(site % L0);
     const bool cross[2] = {x0 == L0 - 1, site + L0 >= V};
     const long long nb[2] = {cross[0] ? site - (L0 - 1) : site + 1, cross[1] ? site + L0 - V : site + L0};
-    double v[4] = {0.0, 0.0, 0.0, 0.0};           // R, I for mu = 0, 1
+    double part[4][4] = {};                       // the four products of R, I for mu = 0, 1
     if (in)
         for (int s = threadIdx.y; s < Ls; s += blockDim.y) {
             const long long b = (long long)s * V;
@@ -111,14 +113,16 @@ k_linkgrad_u1_2d(const double2* __restrict__ U, const double2* __restrict__ lam,
                 // h = c0 -+ (c1 or -i c1): gamma_1 pairs c0 with c1, gamma_2 with -i c1
                 const double2 p = mu == 0 ? l0 - l1 : l0 + times_i(l1), q = mu == 0 ? y0 - y1 : y0 + times_i(y1);
                 const double2 r = mu == 0 ? m0 + m1 : m0 - times_i(m1), t = mu == 0 ? x0v + x1v : x0v - times_i(x1v);
-                // (a slice's four products first: see link_sum_su3)
-                double re = p.x * q.x, im = p.y * q.x;
-                re = fma(p.y, q.y, re); re = fma(r.x, t.x, re); re = fma(r.y, t.y, re);
-                im = fma(-p.x, q.y, im); im = fma(r.x, t.y, im); im = fma(-r.y, t.x, im);
-                v[2 * mu] += re;
-                v[2 * mu + 1] += im;
+                double(&re)[4] = part[2 * mu], (&im)[4] = part[2 * mu + 1];
+                re[0] = fma(p.x, q.x, re[0]); re[1] = fma(p.y, q.y, re[1]);
+                re[2] = fma(r.x, t.x, re[2]); re[3] = fma(r.y, t.y, re[3]);
+                im[0] = fma(p.y, q.x, im[0]); im[1] = fma(-p.x, q.y, im[1]);
+                im[2] = fma(r.x, t.y, im[2]); im[3] = fma(-r.y, t.x, im[3]);
             }
         }
+    double v[4];                                  // R, I for mu = 0, 1
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = (part[k][0] + part[k][1]) + (part[k][2] + part[k][3]);
     sum_slice_groups<4>(v, link_sh);
     if (!in || threadIdx.y != 0) return;
 #pragma unroll
@@ -173,7 +177,7 @@ __device__ __forceinline__ void outer_half(const double2 (&a)[6], const double2 
 // summed by themselves before they are added to the total: one chain of multiply-adds over all slices, whose
 // every product is rounded at the size of the whole sum, has an error of 3.4e-16 at Ls = 12, runs of
 // four slices 2.2e-16 and of two 1.8e-16 (sums of four products and no half spinors: 2.6e-16).  A run costs 18 more
-// FP64 instructions (SU(3) force at 12^3 x 24 x 12: 757 us, 778 and 798 us); the totals live in shared memory,
+// FP64 instructions, but the first (SU(3) force at 12^3 x 24 x 12: one run 757 us, four slices 771, two about 795); the totals live in shared memory,
 // since the registers hold one set of 18.
 constexpr int LINK_RUN = 4;
 template <int MU>
@@ -195,8 +199,12 @@ __device__ __forceinline__ void link_sum_su3(const double2* __restrict__ lam, co
             half_spinor<MU, 1>(lam + 12 * (b + nb), k);
             outer_half(h, k, G);
         }
+        if (s0 != (int)threadIdx.y) {                    // not the first run
 #pragma unroll
-        for (int e = 0; e < 18; ++e) total[e * LINK_THREADS] = s0 == (int)threadIdx.y ? G[e] : total[e * LINK_THREADS] + G[e];
+            for (int e = 0; e < 18; ++e) G[e] += total[e * LINK_THREADS];
+        }
+#pragma unroll
+        for (int e = 0; e < 18; ++e) total[e * LINK_THREADS] = G[e];
     }
 }
 
@@ -207,7 +215,7 @@ __device__ __forceinline__ void link_sum_su3(const double2* __restrict__ lam, co
 // Re(lam^dag dD x) = tr(H F) under U -> exp(i eps H) U.
 // grid.y = mu, a compile-time constant of each branch, so that gamma_mu is a choice of
 // components and signs: 192 FP64 instructions per (link, slice), 0.66 ms of the FP64 rate at
-// 12^3 x 24 x 12 (the memory floor is 35 us); measured 0.78 ms.  With gamma_mu looked up at run
+// 12^3 x 24 x 12 (the memory floor is 35 us); measured 0.77 ms.  With gamma_mu looked up at run
 // time and all four spins multiplied out the kernel ran 3.20 ms.
 template <bool FORCE>
 __global__ void __launch_bounds__(LINK_THREADS, 4)
