@@ -115,13 +115,6 @@ __device__ __forceinline__ void apply_Adag(int mu, const C (&h)[2][3], C (&o)[2]
     }
 }
 
-// -1/2 hops + f h + diag v.  The largest term comes last: the error against 64 bits is 5.0e-8 in FP32 and
-// 9.2e-17 in FP64, where diag v before f h gives 5.4e-8 and 1.0e-16.
-template <class C, class R>
-__device__ __forceinline__ C small_first(C hops, C h, R f, C v, R diag) {
-    return mk<C>(fma(diag, v.x, fma(f, h.x, R(-0.5) * hops.x)), fma(diag, v.y, fma(f, h.y, R(-0.5) * hops.y)));
-}
-
 // Block: 32 consecutive sites x 8 slices.  Blocks are numbered slice group
 // fastest, so the slice groups of one set of sites run together and share its
 // links and boundary slices in L2.  Bound by L1 (a spinor piece touches 24 lines per warp) and FP32
@@ -155,11 +148,35 @@ __global__ void __launch_bounds__(256, sizeof(R) == 8 ? 2 : 3) k_dwf4d(const typ
             st *= p.L[mu];
         }
     }
-    C up[2][3], lo[2][3];     // accumulated -1/2 sum of hops, upper / lower spin pairs
+    // s-hops.  D: up += psi_{s-1}.up (or -m psi_{Ls-1}.up), lo += psi_{s+1}.lo (or -m psi_0.lo)
+    //          D^dag: up from s+1 / wall psi_0, lo from s-1 / wall psi_{Ls-1}
+    const R mf = param_cast<R>(p.mf, p.mf_f);
+    const int s_up = DAG ? (s + 1 < p.Ls ? s + 1 : 0) : (s > 0 ? s - 1 : p.Ls - 1);
+    const int s_lo = DAG ? (s > 0 ? s - 1 : p.Ls - 1) : (s + 1 < p.Ls ? s + 1 : 0);
+    const R f_up = DAG ? (s + 1 < p.Ls ? R(1) : -mf) : (s > 0 ? R(1) : -mf);
+    const R f_lo = DAG ? (s > 0 ? R(1) : -mf) : (s + 1 < p.Ls ? R(1) : -mf);
+    C up[2][3], lo[2][3];     // upper / lower spin pairs
+    // In FP64 the sums start with the s-hops (at the end, all their inputs beside the sums made 100 registers
+    // spill: 12^3 x 24 x 12 837 us against 798); in FP32 they end with them
+    constexpr bool FIRST = sizeof(R) == 8;
+    auto s_hops = [&] {
+        C hu[2][3], hl[2][3];
+        ld_half<W32, 0>(psi + ((long long)s_up * V + site) * 12, hu);
+        ld_half<W32, 1>(psi + ((long long)s_lo * V + site) * 12, hl);
 #pragma unroll
-    for (int a = 0; a < 2; ++a)
+        for (int a = 0; a < 2; ++a)
 #pragma unroll
-        for (int c = 0; c < 3; ++c) { up[a][c] = mk<C>(R(0), R(0)); lo[a][c] = mk<C>(R(0), R(0)); }
+            for (int c = 0; c < 3; ++c) {
+                up[a][c] = FIRST ? scale(hu[a][c], f_up) : up[a][c] + scale(hu[a][c], f_up);
+                lo[a][c] = FIRST ? scale(hl[a][c], f_lo) : lo[a][c] + scale(hl[a][c], f_lo);
+            }
+    };
+    if (FIRST) s_hops();
+    else
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) { up[a][c] = mk<C>(R(0), R(0)); lo[a][c] = mk<C>(R(0), R(0)); }
     const C* plane = psi + (long long)s * V * 12;
 
 #pragma unroll
@@ -172,7 +189,7 @@ __global__ void __launch_bounds__(256, sizeof(R) == 8 ? 2 : 3) k_dwf4d(const typ
             const bool cross = fwd ? (coord[mu] == L - 1) : (coord[mu] == 0);
             const int nb = fwd ? (cross ? site - (L - 1) * stride[mu] : site + stride[mu])
                                : (cross ? site + (L - 1) * stride[mu] : site - stride[mu]);
-            const R ph = (cross && p.anti[mu]) ? R(-1) : R(1);
+            const R ph = (cross && p.anti[mu]) ? R(0.5) : R(-0.5);
             // projector sign: D uses (1 - gamma) forward, (1 + gamma) backward; D^dag the opposite
             const bool minus = (fwd != DAG);
             C v[4][3];
@@ -207,32 +224,23 @@ __global__ void __launch_bounds__(256, sizeof(R) == 8 ? 2 : 3) k_dwf4d(const typ
             for (int a = 0; a < 2; ++a)
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
-                    // the boundary phase rides on the accumulating multiply-adds
+                    // the -1/2 and the boundary phase ride on the accumulating multiply-adds
                     up[a][c] = up[a][c] + scale(uh[a][c], ph);
                     lo[a][c] = lo[a][c] + scale(Ad[a][c], minus ? -ph : ph);
                 }
         }
     }
+    if (!FIRST) s_hops();
+    // The diagonal term is the largest and comes last: error against 64 bits 5.0e-8 in FP32, 5.4e-8 with the s-hop after it
     const R diag = param_cast<R>(p.diag, p.diag_f);
-    const R mf = param_cast<R>(p.mf, p.mf_f);
-    C self[4][3];
+    C self[4][3], o[4][3];
     ld_spin4<W32>(plane + (long long)site * 12, self);
-    // s-hops: D: up += psi_{s-1}.up (or -m psi_{Ls-1}.up), lo += psi_{s+1}.lo (or -m psi_0.lo)
-    //         D^dag: up from s+1 / wall psi_0, lo from s-1 / wall psi_{Ls-1}
-    const int s_up = DAG ? (s + 1 < p.Ls ? s + 1 : 0) : (s > 0 ? s - 1 : p.Ls - 1);
-    const int s_lo = DAG ? (s > 0 ? s - 1 : p.Ls - 1) : (s + 1 < p.Ls ? s + 1 : 0);
-    const R f_up = DAG ? (s + 1 < p.Ls ? R(1) : -mf) : (s > 0 ? R(1) : -mf);
-    const R f_lo = DAG ? (s > 0 ? R(1) : -mf) : (s + 1 < p.Ls ? R(1) : -mf);
-    C hu[2][3], hl[2][3];
-    ld_half<W32, 0>(psi + ((long long)s_up * V + site) * 12, hu);
-    ld_half<W32, 1>(psi + ((long long)s_lo * V + site) * 12, hl);
-    C o[4][3];
 #pragma unroll
     for (int a = 0; a < 2; ++a)
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            o[a][c] = small_first(up[a][c], hu[a][c], f_up, self[a][c], diag);
-            o[a + 2][c] = small_first(lo[a][c], hl[a][c], f_lo, self[a + 2][c], diag);
+            o[a][c] = up[a][c] + scale(self[a][c], diag);
+            o[a + 2][c] = lo[a][c] + scale(self[a + 2][c], diag);
         }
     st_spin4<W32>(out + ((long long)s * V + site) * 12, o);
 }
