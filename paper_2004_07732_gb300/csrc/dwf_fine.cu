@@ -76,7 +76,7 @@ __device__ __forceinline__ Sp2<R> hop2d(const Sp2<R>& xf, const Sp2<R>& xb, cons
 // take p = t_f + t_b and t_b - t_f (times 1 or i): p grows in t_f by fused multiply-adds, and the
 // difference is p - 2 t_f.  The FP64 kernel is bound by FP64 issue (ncu: 86% of the pipe), and this
 // takes 40 instructions per site and slice with the diagonal and the s-hops, where separate
-// products, sums and scaling take 48: D_PV^dag D_DW at 250 x 333 x 13 184 us against 219 (with longer
+// products, sums and scaling take 48: D_PV^dag D_DW at 250 x 333 x 13 180 us against 219 (with longer
 // walks too), at the same error (9.6e-17 of one application at 64 x 48 x 12).  For that the sums stay
 // trees and the largest term, the diagonal one, comes last, after the s-hop (before it: 9.8e-17).
 // The adjoint's c1 comes with the opposite sign, which rides on the sum with the s-hop.
@@ -178,8 +178,8 @@ __device__ __forceinline__ void dwf2d_site(const typename LT::store* __restrict_
         if constexpr (sizeof(R) == 8) {
             o = hop2d_fused<DAG>(nb_xf, nb_xb, nb_yf, nb_yb, u0f, u0b, u1f, u1b);
             // p - 2 t_f turns an infinite t_f into NaN: take the differences themselves (the empty
-            // statement keeps this a branch: D_PV^dag D_DW at 250 x 333 x 13 184 us, without the check 180,
-            // with both forms computed and one selected 266)
+            // statement keeps this a branch: D_PV^dag D_DW at 250 x 333 x 13 180 us, as without the check; with
+            // both forms computed and one selected 266)
             if (__builtin_expect(not_finite(o), 0)) {
                 asm volatile("" ::: "memory");
                 o = hop2d<double, DAG>(ld_sp(pxf, 0), ld_sp(pxb, 0), ld_sp(pyf, 0), ld_sp(pyb, 0), u0f, u0b, u1f, u1b);
