@@ -115,12 +115,12 @@ __device__ __forceinline__ void apply_Adag(int mu, const C (&h)[2][3], C (&o)[2]
     }
 }
 
-// Block: 32 consecutive sites x 8 slices.  Blocks are numbered slice group
+// Block: 32 consecutive sites x 8 slices (fewer where there are fewer).  Blocks are numbered slice group
 // fastest, so the slice groups of one set of sites run together and share its
 // links and boundary slices in L2.  Bound by L1 (a spinor piece touches 24 lines per warp) and FP32
-// issue; FP64 by the FP64 pipe.  16^3 x 32 x 16, FP16 links: 162 us against 222 us with 16-byte
+// issue; FP64 by the FP64 pipe.  16^3 x 32 x 16, FP16 links: 160 us against 222 us with 16-byte
 // pieces and products and sums apart; 12^3 x 24 x 12 in FP64, at the 128 registers its values need,
-// 834 against 1159 us.  (One table of neighbours per block in shared memory: 173 us, its barrier
+// 799 against 1159 us.  (One table of neighbours per block in shared memory: 173 us, its barrier
 // costs more than the divisions; the block's links in shared memory too: 191 us, and 226 us for
 // the adjoint, whose registers then spill.)
 template <class LT, class R, bool DAG, bool W32>
