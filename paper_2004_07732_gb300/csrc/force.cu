@@ -61,9 +61,12 @@ constexpr int LINK_THREADS = 128;
 // 152 SMs hold 16 warps each at the 128 registers of the SU(3) kernel: the slices are split until
 // two such waves are there.  SU(3) force at 12^3 x 24 x 12 (2.1 waves unsplit) with 1, 2, 4, 8
 // groups: 756, 767, 760, 884 us.
-static int link_slice_groups(long long threads, int Ls) {
+// U(1), with 36 warps per SM and as many adds per group as two slices take: two thirds of a wave (128^2 x 8 with 4
+// and 8 groups: 12.8 and 16.0 us; 256^2 x 4 with 1 and 2: 20.5 and 22.7).
+static int link_slice_groups(bool su3, long long threads, int Ls) {
+    const long long target = 152LL * (su3 ? 1024 : 768);
     int sp = 1;
-    while (sp < 8 && 2 * sp <= Ls && threads * sp < 2LL * 152 * 512) sp *= 2;
+    while (sp < 8 && 2 * sp <= Ls && threads * sp < target) sp *= 2;
     return sp;
 }
 
@@ -89,7 +92,31 @@ __device__ __forceinline__ void sum_slice_groups(double (&v)[N], double* sh) {
 //   FORCE: the derivative along theta (dU = i U dtheta): -1/2 ph (U.x I - U.y R).
 // 16 FP64 instructions per (link, slice): each of the four products of R and of I has a sum of its
 // own, since one chain of all of them rounds every product at the size of the whole sum (error 1.9e-16 at
-// 300 x 400 x 12).  512^2 x 16: 261 us; 254 with the one chain, 295 with each slice's products summed first.
+// 300 x 400 x 12).  512^2 x 16: 252 us; 254 with the one chain, 295 with each slice's products summed first.
+// grid.y = mu, as for SU(3): a thread with the sums of both needs 78 registers instead of 56, and the 1024 blocks of
+// a 128^2 lattice then come in a round and a bit (128^2 x 8: 17 us against 12.8).
+template <int MU>
+__device__ __forceinline__ void link_sum_u1(const double2* __restrict__ lam, const double2* __restrict__ x, long long V,
+                                            int Ls, long long site, long long nb, double (&v)[2]) {
+    double re[4] = {0.0, 0.0, 0.0, 0.0}, im[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int s = threadIdx.y; s < Ls; s += blockDim.y) {
+        const long long b = (long long)s * V;
+        const double2 l0 = __ldg(lam + 2 * (b + site)), l1 = __ldg(lam + 2 * (b + site) + 1);
+        const double2 x0 = __ldg(x + 2 * (b + site)), x1 = __ldg(x + 2 * (b + site) + 1);
+        const double2 m0 = __ldg(lam + 2 * (b + nb)), m1 = __ldg(lam + 2 * (b + nb) + 1);
+        const double2 y0 = __ldg(x + 2 * (b + nb)), y1 = __ldg(x + 2 * (b + nb) + 1);
+        // h = c0 -+ (c1 or -i c1): gamma_1 pairs c0 with c1, gamma_2 with -i c1
+        const double2 p = MU == 0 ? l0 - l1 : l0 + times_i(l1), q = MU == 0 ? y0 - y1 : y0 + times_i(y1);
+        const double2 r = MU == 0 ? m0 + m1 : m0 - times_i(m1), t = MU == 0 ? x0 + x1 : x0 - times_i(x1);
+        re[0] = fma(p.x, q.x, re[0]); re[1] = fma(p.y, q.y, re[1]);
+        re[2] = fma(r.x, t.x, re[2]); re[3] = fma(r.y, t.y, re[3]);
+        im[0] = fma(p.y, q.x, im[0]); im[1] = fma(-p.x, q.y, im[1]);
+        im[2] = fma(r.x, t.y, im[2]); im[3] = fma(-r.y, t.x, im[3]);
+    }
+    v[0] = (re[0] + re[1]) + (re[2] + re[3]);
+    v[1] = (im[0] + im[1]) + (im[2] + im[3]);
+}
+
 template <bool FORCE>
 __global__ void __launch_bounds__(LINK_THREADS)
 k_linkgrad_u1_2d(const double2* __restrict__ U, const double2* __restrict__ lam, const double2* __restrict__ x,
@@ -97,44 +124,23 @@ k_linkgrad_u1_2d(const double2* __restrict__ U, const double2* __restrict__ lam,
     extern __shared__ double link_sh[];
     const long long site = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const bool in = site < V;
-    const int x0 = (int)(site % L0);
-    const bool cross[2] = {x0 == L0 - 1, site + L0 >= V};
-    const long long nb[2] = {cross[0] ? site - (L0 - 1) : site + 1, cross[1] ? site + L0 - V : site + L0};
-    double part[4][4] = {};                       // the four products of R, I for mu = 0, 1
-    if (in)
-        for (int s = threadIdx.y; s < Ls; s += blockDim.y) {
-            const long long b = (long long)s * V;
-            const double2 l0 = __ldg(lam + 2 * (b + site)), l1 = __ldg(lam + 2 * (b + site) + 1);
-            const double2 x0v = __ldg(x + 2 * (b + site)), x1v = __ldg(x + 2 * (b + site) + 1);
-#pragma unroll
-            for (int mu = 0; mu < 2; ++mu) {
-                const double2 m0 = __ldg(lam + 2 * (b + nb[mu])), m1 = __ldg(lam + 2 * (b + nb[mu]) + 1);
-                const double2 y0 = __ldg(x + 2 * (b + nb[mu])), y1 = __ldg(x + 2 * (b + nb[mu]) + 1);
-                // h = c0 -+ (c1 or -i c1): gamma_1 pairs c0 with c1, gamma_2 with -i c1
-                const double2 p = mu == 0 ? l0 - l1 : l0 + times_i(l1), q = mu == 0 ? y0 - y1 : y0 + times_i(y1);
-                const double2 r = mu == 0 ? m0 + m1 : m0 - times_i(m1), t = mu == 0 ? x0v + x1v : x0v - times_i(x1v);
-                double(&re)[4] = part[2 * mu], (&im)[4] = part[2 * mu + 1];
-                re[0] = fma(p.x, q.x, re[0]); re[1] = fma(p.y, q.y, re[1]);
-                re[2] = fma(r.x, t.x, re[2]); re[3] = fma(r.y, t.y, re[3]);
-                im[0] = fma(p.y, q.x, im[0]); im[1] = fma(-p.x, q.y, im[1]);
-                im[2] = fma(r.x, t.y, im[2]); im[3] = fma(-r.y, t.x, im[3]);
-            }
-        }
-    double v[4];                                  // R, I for mu = 0, 1
-#pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] = (part[k][0] + part[k][1]) + (part[k][2] + part[k][3]);
-    sum_slice_groups<4>(v, link_sh);
+    const int mu = blockIdx.y;
+    const bool cross = mu == 0 ? (int)(site % L0) == L0 - 1 : site + L0 >= V;
+    const long long nb = mu == 0 ? (cross ? site - (L0 - 1) : site + 1) : (cross ? site + L0 - V : site + L0);
+    double v[2] = {0.0, 0.0};                     // R, I
+    if (in) {
+        if (mu == 0) link_sum_u1<0>(lam, x, V, Ls, site, nb, v);
+        else         link_sum_u1<1>(lam, x, V, Ls, site, nb, v);
+    }
+    sum_slice_groups<2>(v, link_sh);
     if (!in || threadIdx.y != 0) return;
-#pragma unroll
-    for (int mu = 0; mu < 2; ++mu) {
-        const double ph = (cross[mu] && (mu == 0 ? anti0 : anti1)) ? 0.5 : -0.5;
-        const long long t = mu * V + site;
-        if (FORCE) {
-            const double2 u = __ldg(U + t);
-            out[t] = ph * (u.x * v[2 * mu + 1] - u.y * v[2 * mu]);
-        } else {
-            reinterpret_cast<double2*>(out)[t] = make_double2(ph * v[2 * mu], ph * v[2 * mu + 1]);
-        }
+    const double ph = (cross && (mu == 0 ? anti0 : anti1)) ? 0.5 : -0.5;
+    const long long t = mu * V + site;
+    if (FORCE) {
+        const double2 u = __ldg(U + t);
+        out[t] = ph * (u.x * v[1] - u.y * v[0]);
+    } else {
+        reinterpret_cast<double2*>(out)[t] = make_double2(ph * v[0], ph * v[1]);
     }
 }
 
@@ -292,11 +298,11 @@ template <bool FORCE>
 static dwf_status launch_link(const Geom& G, const void* U, const void* lam, const void* x, void* out,
                               cudaStream_t st) {
     const bool su3 = G.nd == 4;
-    const int sp = link_slice_groups(su3 ? 4 * G.V : G.V, G.Ls);
+    const int sp = link_slice_groups(su3, (su3 ? 4 : 2) * G.V, G.Ls);
     const dim3 block(LINK_THREADS / sp, sp);
-    const dim3 grid((unsigned)((G.V + block.x - 1) / block.x), su3 ? 4u : 1u);
+    const dim3 grid((unsigned)((G.V + block.x - 1) / block.x), su3 ? 4u : 2u);
     // SU(3): the 18 totals of every thread; U(1): the sums of groups 1 .. sp - 1
-    const size_t sh = (su3 ? 18 * LINK_THREADS : (size_t)(sp - 1) * 4 * block.x) * sizeof(double);
+    const size_t sh = (su3 ? 18 * LINK_THREADS : (size_t)(sp - 1) * 2 * block.x) * sizeof(double);
     if (su3)
         k_linkgrad_su3<FORCE><<<grid, block, sh, st>>>((const double2*)U, (const double2*)lam, (const double2*)x,
                                                        (double2*)out, make_int4(G.L[0], G.L[1], G.L[2], G.L[3]), G.V,
